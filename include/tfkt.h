@@ -119,8 +119,10 @@ typedef struct tfkt_ctx tfkt_ctx;
 enum {
   TFKT_K_MOMENTS = 0,  /* pull-read of all populations -> moment planes */
   TFKT_K_STEP,         /* two-pass path: pull, collide and write of all populations */
-  TFKT_K_FUSED,        /* fused path: pull, collide, write and next-step moments */
-  TFKT_K_FIXUP,        /* fused path: completion of the tiles' border moments */
+  TFKT_K_FUSED,        /* fused path: pull, collide, write and next-step moments (the moments
+                          excepted in FP64 and on grids of up to 100 tiles) */
+  TFKT_K_FIXUP,        /* fused path: completion of the next step's moments (of the tiles'
+                          border nodes; in FP64 and on grids of up to 100 tiles of all nodes) */
   TFKT_NKERNELS
 };
 

@@ -134,6 +134,23 @@ double polymer_scale(const Lattice& L) {
   return std::ldexp(1.0, (int)std::lround(std::log2(target)));
 }
 
+// The Q-split kernels instead of the fused kernel: FP64 always (both are bound by
+// the FP64 pipe, of which the fused kernel needs about twice as much: 512 x 512 nodes, 32
+// Q-nodes, 4739 us per step against 3071), other precisions where the fused
+// kernel's tiles leave most SMs idle. That kernel takes the same time up to one
+// tile per SM, the Q-split kernels a time that grows with the nodes. FP32, us per
+// step, with 32 Q-nodes: 61.8 against 12.1 at 64 x 64 nodes (16 tiles), 64 against 35
+// at 128 x 128 (64), 71.5 against 60 at 160 x 160 (100), 77.5 against 90 at 192 x 192
+// (144); with 9 Q-nodes 25.4 against 13.8 at 128 x 128, 26.8 against 16.2 at 160 x 160,
+// 36 against 57 at 256 x 256. The line is drawn at 100 tiles. A slab steps as its
+// whole run does, so the whole run's size decides.
+constexpr size_t SPLIT_TILES = 100;
+bool split_path(const Lattice& L) {
+  if (L.precision == TFKT_FP64) return true;
+  const size_t ny = L.ny_global > 0 ? L.ny_global : L.ny;
+  return (size_t)(L.nx / TX) * (ny / TY) <= SPLIT_TILES;
+}
+
 size_t store_size(const Lattice& L) {
   return L.precision == TFKT_FP64 ? 8 : (L.precision == TFKT_FP16 ? 2 : 4);
 }
@@ -166,7 +183,8 @@ size_t layout(const Lattice& L, Workspace* w) {
   o = align_up(o + 2 * L.plane * sz, A);
   w->off_tab = o;
   const size_t tab = (5 * (size_t)L.nq + 25 * (size_t)L.nq + 2 * (size_t)L.ny) * sz +
-                     25 * (size_t)L.nq * sizeof(int) + 10 * A;
+                     25 * (size_t)L.nq * sizeof(int) +
+                     (size_t)L.nq * (sz == 8 ? sizeof(QRow<double>) : sizeof(QRow<float>)) + 11 * A;
   o = align_up(o + tab, A);
   w->off_part = o;
   o = align_up(o + (size_t)diag_blocks_for(L) * TFKT_NDIAG * sizeof(double), A);
@@ -271,6 +289,7 @@ KernelArgs<real> make_args(const Ctx* c, const HostTables* ht = nullptr) {
   a.nx = L.nx;
   a.ny = L.ny;
   a.nq = L.nq;
+  a.mom_warps = moment_warps(L);
   a.pitch = L.pitch;
   a.plane = L.plane;
   const double b = 1.0 / (2.0 * L.tau1 + 1.0);
@@ -310,6 +329,7 @@ KernelArgs<real> make_args(const Ctx* c, const HostTables* ht = nullptr) {
   a.tab.delta = (const real*)take(nq * 25 * sizeof(real));
   a.tab.arow = (const real*)take((size_t)L.ny * sizeof(real));
   a.tab.urow = (const real*)take((size_t)L.ny * sizeof(real));
+  a.tab.row = (const QRow<real>*)take(nq * sizeof(QRow<real>));
   (void)ht;
   return a;
 }
@@ -364,6 +384,9 @@ tfkt_status upload_tables(Ctx* c, const HostTables& t) {
   TFKT_CUDA(c, put(a.tab.delta, t.delta));
   TFKT_CUDA(c, put(a.tab.arow, t.arow));
   TFKT_CUDA(c, put(a.tab.urow, t.urow));
+  const std::vector<QRow<real>> rows = build_rows<real>(c->L, t);
+  TFKT_CUDA(c, cudaMemcpy((void*)a.tab.row, rows.data(), rows.size() * sizeof(QRow<real>),
+                          cudaMemcpyHostToDevice));
   if (c->fused) return upload_fused_tables<real>(c, t);
   return TFKT_OK;
 }
@@ -382,10 +405,23 @@ tfkt_status init_state(Ctx* c, const double* perturb) {
   a.perturb = dpert;
   a.dst = (char*)c->ws.base + c->ws.off_pop[0];
   TFKT_CUDA(c, launch_init<real, S>(a, c->stream));   // populations and their moments
+  // the Q-split kernels sum the moments in another order: take theirs from the start,
+  // so that a step gives the same bits whether or not its moments were formed again
+  if (!c->fused || c->split) TFKT_CUDA(c, launch_moments<real, S>(a, c->stream));
   c->cur = 0;
   c->m_valid = true;
   TFKT_CUDA(c, cudaStreamSynchronize(c->stream));
   return TFKT_OK;
+}
+
+// Whether the caller is capturing a stream (or that cannot be told).
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
 }
 
 template <typename real, typename S>
@@ -397,24 +433,43 @@ tfkt_status ensure_moments(Ctx* c) {
   return TFKT_OK;
 }
 
+// Whether a step of a fused-path context takes the Q-split kernels. A pending
+// learned-block increment rides on the pull of the fused kernel only.
+inline bool step_split(const Ctx* c) { return c->split && !c->lpm_pending; }
+
 // One step. Fused path: the step kernel also produces the next state's
-// moment planes (completed at tile borders by the fix-up kernel), so the
-// moments stay valid. Two-pass path: moments kernel, then the step kernel.
+// moment planes (completed at tile borders by the fix-up kernel), or, where the
+// Q-split kernels are faster (split_path), the collision and then the moments
+// of the populations it wrote; either way the moments stay valid. Two-pass
+// path: moments kernel, then the collision, with one set of moment planes.
 template <typename real, typename S>
 tfkt_status do_step(Ctx* c, int64_t n) {
+  // Under a stream capture no programmatic serialisation (the node before may be no
+  // kernel), and a two-pass context's first step takes its own moments, so that
+  // every replay does.
+  const bool q_split = n > 0 && (c->split || !c->fused);
+  const bool cap = q_split && capturing(c->stream), dep = q_split && !cap;
+  if (cap && !c->fused) c->m_valid = false;
   for (int64_t k = 0; k < n; ++k) {
-    tfkt_status s = ensure_moments<real, S>(c);
-    if (s != TFKT_OK) return s;
     KernelArgs<real> a = make_args<real>(c);
+    if (!c->m_valid) {
+      TFKT_CUDA(c, launch_moments<real, S>(a, c->stream, dep));
+      c->m_valid = true;
+    }
     if (c->fused) {
       FusedArgs<real> f = make_fused<real>(c);
-      if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
-      TFKT_CUDA(c, launch_step_fused<real, S>(a, f, c->stream));
-      TFKT_CUDA(c, launch_fixup<real>(a, f, c->stream));
+      if (step_split(c)) {
+        TFKT_CUDA(c, launch_step<real, S>(a, c->stream, dep));
+        TFKT_CUDA(c, launch_moments<real, S>(next_moments_args(a, f), c->stream, dep));
+      } else {
+        if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
+        TFKT_CUDA(c, launch_step_fused<real, S>(a, f, c->stream));
+        TFKT_CUDA(c, launch_fixup<real>(a, f, c->stream));
+      }
       c->lpm_pending = false;
       c->mcur ^= 1;
     } else {
-      TFKT_CUDA(c, launch_step<real, S>(a, c->stream));
+      TFKT_CUDA(c, launch_step<real, S>(a, c->stream, dep));
       c->m_valid = false;
     }
     c->cur ^= 1;
@@ -477,12 +532,17 @@ tfkt_status do_step_profiled(Ctx* c, int64_t n, double* ms, int64_t* launches) {
     KernelArgs<real> a = make_args<real>(c);
     if (c->fused) {
       FusedArgs<real> f = make_fused<real>(c);
+      const bool split = step_split(c);
       if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
-      tfkt_status s =
-          timed(TFKT_K_FUSED, [&] { return launch_step_fused<real, S>(a, f, c->stream); });
+      tfkt_status s = timed(TFKT_K_FUSED, [&] {
+        return split ? launch_step<real, S>(a, c->stream) : launch_step_fused<real, S>(a, f, c->stream);
+      });
       if (s != TFKT_OK) return s;
       c->lpm_pending = false;
-      s = timed(TFKT_K_FIXUP, [&] { return launch_fixup<real>(a, f, c->stream); });
+      s = timed(TFKT_K_FIXUP, [&] {
+        return split ? launch_moments<real, S>(next_moments_args(a, f), c->stream)
+                     : launch_fixup<real>(a, f, c->stream);
+      });
       if (s != TFKT_OK) return s;
       c->mcur ^= 1;
     } else {
@@ -666,6 +726,7 @@ tfkt_status ctx_create(const Lattice& L, const double* perturb, void* dev_worksp
   c->L = L;
   c->stream = (cudaStream_t)stream;
   c->fused = fused_path(L);
+  c->split = c->fused && split_path(L);
   const size_t need = layout(L, &c->ws);
   c->diag_blocks = diag_blocks_for(L);
   if (dev_workspace) {

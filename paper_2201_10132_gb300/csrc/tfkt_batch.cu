@@ -98,7 +98,15 @@ cudaError_t launch_per_run(tfkt_batch* b, int parity, cudaStream_t s) {
     e = cudaStreamWaitEvent(b->pool[k], b->fork, 0);
   for (size_t j = 0; j < b->order.size() && e == cudaSuccess; ++j) {
     const int i = b->order[j];
-    e = launch_single_fp32(b->host[i].a[parity], b->host[i].f[parity], b->pool[j % b->pool.size()]);
+    const KernelArgs<float>& a = b->host[i].a[parity];
+    const FusedArgs<float>& f = b->host[i].f[parity];
+    cudaStream_t p = b->pool[j % b->pool.size()];
+    if (ctx_of(b->runs[i])->split) {
+      e = launch_step<float, float>(a, p, false, b->runs.size() > 1);
+      if (e == cudaSuccess) e = launch_moments<float, float>(next_moments_args(a, f), p);
+    } else {
+      e = launch_single_fp32(a, f, p);
+    }
   }
   for (size_t k = 0; k < b->pool.size() && e == cudaSuccess; ++k) {
     e = cudaEventRecord(b->join[k], b->pool[k]);

@@ -94,6 +94,25 @@ struct Lattice {
 // Moment field planes (M): delta psi(q) for q < nq, then these.
 enum { M_DRHO = 0, M_JX, M_JY, M_THXX, M_THXY, M_THYY, M_NSCALAR };
 
+// Per-Q-node table of the Q-split kernels (tfkt_split.cu). The Q-displacement
+// groups that move in Q fill eight slots; values in stored units (times the
+// polymer storage scale) are marked [s].
+template <typename real>
+struct alignas(16) QRow {
+  int src[8];        // first population plane of the pull's source Q-node, or ~(first plane
+                     // of this Q-node) where the pull bounces
+  real bd[8];        // [s] shift difference of the group's pull, times (1 - 2 beta) where it
+                     // is folded into the collision (FP64, momentum quasi-equilibrium)
+  real psi0;
+  real dpsi;         // [s] sum of the shift differences of all 25 pulls
+  real dq[2];        // [s] their Q-momentum (their r-momentum is zero)
+  real q[2], hq[2];  // Q and Q / 2
+  real kf[2];        // kappa phi_q Q
+  real cf[2];        // tau_m (H ell^2 / 2) phi_q Q
+  real tq[3];        // phi_q Q Q (xx, xy, yy)
+  real pad;
+};
+
 // Device tables of a context (one copy per precision in use).
 template <typename real>
 struct Tables {
@@ -106,6 +125,7 @@ struct Tables {
   const real* delta;     // [nq*25]: w_i (psi0(q - Qdot_i) - psi0(q)), 0 for bounce-back
   const real* arow;      // [ny] forcing a(y)
   const real* urow;      // [ny] initial base flow U_x(y)
+  const QRow<real>* row; // [nq] per-Q-node table of the Q-split kernels
 };
 
 // Conversions between the storage type S of the populations and the compute
@@ -156,6 +176,7 @@ struct KernelArgs {
   real* U;                       // scratch: 2 planes (U_x, U_y)
   const double* perturb;         // [2][ny][nx] (init only)
   int nx, ny, nq;
+  int mom_warps;                 // warps that share a node's moment sums (moment_warps)
   size_t pitch, plane;
   real tau2, c2, inv_c2p1;       // tau2, 2 tau2, 1 / (2 tau2 + 1)
   real om2b, tb, omb;            // 1 - 2 beta, 2 beta, 1 - beta
@@ -195,6 +216,16 @@ struct BatchRun {
   int pad[2];
 };
 
+// The Q-split step's second half: the next state's moment planes from the
+// populations that the collision has just written.
+template <typename real>
+KernelArgs<real> next_moments_args(const KernelArgs<real>& a, const FusedArgs<real>& f) {
+  KernelArgs<real> m = a;
+  m.src = a.dst;
+  m.M = f.Mout;
+  return m;
+}
+
 struct Workspace {
   void* base = nullptr;
   size_t bytes = 0;
@@ -213,7 +244,8 @@ struct Ctx {
   bool poisoned = false;
   int64_t step = 0;
   int diag_blocks = 0;
-  bool fused = false;     // grid fits the fused single-pass kernel
+  bool fused = false;     // grid fits the fused single-pass kernel (double-buffered moments)
+  bool split = false;     // a fused-path context that steps with the Q-split kernels
   int mcur = 0;           // moment buffer (0: off_M, 1: off_M2) of the current state
   double dvx = 0, dvy = 0;  // r-momentum of all pull shift differences (fused path)
   void* lpm = nullptr;    // scratch of the learned block (allocated on first use)
@@ -242,13 +274,23 @@ struct HostTables {
 };
 HostTables build_tables(const Lattice& L);
 
+// Q-split kernels (tfkt_split.cu): the moment planes a.M of the populations a.src,
+// and one collision of a.src (with its moment planes a.M) into a.dst. dependent:
+// the launch may begin while the stream's previous kernel finishes (both kernels
+// wait for it before they touch the state); shared: it runs beside launches that fill
+// the GPU.
+template <typename real>
+std::vector<QRow<real>> build_rows(const Lattice& L, const HostTables& t);
+template <typename real, typename S>
+cudaError_t launch_moments(const KernelArgs<real>& a, cudaStream_t s, bool dependent = false);
+template <typename real, typename S>
+cudaError_t launch_step(const KernelArgs<real>& a, cudaStream_t s, bool dependent = false,
+                        bool shared = false);
+int moment_warps(const Lattice& L);   // KernelArgs::mom_warps of a run
+
 // Launchers (tfkt_kernels.cu). Each returns the launch status.
 template <typename real, typename S>
 cudaError_t launch_init(const KernelArgs<real>& a, cudaStream_t s);
-template <typename real, typename S>
-cudaError_t launch_moments(const KernelArgs<real>& a, cudaStream_t s);
-template <typename real, typename S>
-cudaError_t launch_step(const KernelArgs<real>& a, cudaStream_t s);
 template <typename real>
 cudaError_t launch_velocity(const KernelArgs<real>& a, cudaStream_t s);
 template <typename real>
@@ -277,6 +319,8 @@ cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cu
 // Whether a context of this lattice takes the fused path (tile multiples and the
 // kernel's shared memory; either quasi-equilibrium).
 bool fused_path(const Lattice& L);
+// Whether a fused-path context steps with the Q-split kernels instead (tfkt_api.cu).
+bool split_path(const Lattice& L);
 
 // Each run's single-run FP32 kernels (fused step + fix-up) without API calls
 // besides the launches, after prepare_single_fp32 for the largest nq.

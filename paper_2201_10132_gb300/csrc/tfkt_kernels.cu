@@ -17,11 +17,6 @@ namespace tfkt {
 
 namespace {
 
-__device__ __forceinline__ int wrapi(int v, int n) {
-  v %= n;
-  return v < 0 ? v + n : v;
-}
-
 // The nine pull offsets of node (x, y): source displaced by (sx, sy).
 struct Offsets {
   size_t o[9];
@@ -73,8 +68,8 @@ __device__ __forceinline__ void mixture_velocity(const KernelArgs<real>& a, int 
 // first pull reads for it, so the first step starts from exactly this state.
 // For the same reason the pulled populations of a node are its own stored
 // values: the kernel also writes the state's moment planes M, rebuilding each
-// value from its stored form and summing exactly as moments_kernel does, so
-// the moments need no second pass over the populations.
+// value from its stored form, so the moments need no second pass over the
+// populations.
 template <typename real, typename S>
 __global__ void __launch_bounds__(256) init_kernel(KernelArgs<real> a) {
   using SS = SolventT<S>;
@@ -152,394 +147,6 @@ __global__ void __launch_bounds__(256) init_kernel(KernelArgs<real> a) {
   a.M[(size_t)(nq + M_THXX) * P + n] = a.hl2h * txx;
   a.M[(size_t)(nq + M_THXY) * P + n] = a.hl2h * txy;
   a.M[(size_t)(nq + M_THYY) * P + n] = a.hl2h * tyy;
-}
-
-// --------------------------------------------------------------- moments
-// Pull-read every population of node (x, y) and write its moments to M
-// (Sec. VI-A / VI-B moment definitions; Theta of Sec. III, Eq. IDef, with the
-// spring force H phi_q Q).
-template <typename real, typename S>
-__global__ void __launch_bounds__(256) moments_kernel(KernelArgs<real> a) {
-  // The pull tables go to shared memory, and the populations of Q-node q + 1
-  // are loaded into each register as soon as Q-node q has used it, so the
-  // loads of one Q-node are in flight while the previous one is summed.
-  extern __shared__ __align__(16) unsigned char mom_smem[];
-  const int nq = a.nq;
-  real* s_delta = reinterpret_cast<real*>(mom_smem);
-  int* s_pull = reinterpret_cast<int*>(mom_smem + sizeof(real) * (size_t)nq * 25);
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  for (int k = tid; k < nq * 25; k += TX * TY) {
-    s_delta[k] = a.tab.delta[k];
-    s_pull[k] = a.tab.pull[k];
-  }
-  __syncthreads();
-  const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
-  if (x >= a.nx || y >= a.ny) return;
-  const Offsets off = node_offsets(x, y, a.nx, a.ny, a.pitch);
-  const size_t P = a.plane;
-  const size_t n = off.o[4];
-  const S* __restrict__ src = (const S*)a.src;
-  const SolventT<S>* __restrict__ ssrc = solvent_planes<S>(a.src, P, a.nq);
-  auto pull = [&](int q, int i) {
-    const V4 c = c25(i);
-    const int e = s_pull[q * 25 + i];
-    const size_t o = e >= 0 ? off.o[shift_index(-c.rx, -c.ry)] : off.o[4];
-    return src[(size_t)(e >= 0 ? e : ~e) * P + o];
-  };
-  S h[25];
-  if (nq > 0) {
-#pragma unroll
-    for (int i = 0; i < 25; ++i) h[i] = pull(0, i);
-  }
-  real drho = 0, jx = 0, jy = 0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const real v = from_store<real>(ssrc[(size_t)i * P + off.o[shift_index(-c9x(i), -c9y(i))]]);
-    drho += v;
-    jx += real(c9x(i)) * v;
-    jy += real(c9y(i)) * v;
-  }
-  real txx = 0, txy = 0, tyy = 0;
-  for (int q = 0; q < nq; ++q) {
-    const bool more = q + 1 < nq;
-    real dpsi = 0, rx = 0, ry = 0;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      const V4 c = c25(i);
-      const real v = from_store<real>(h[i]) * a.pinv + s_delta[q * 25 + i];
-      if (more) h[i] = pull(q + 1, i);
-      dpsi += v;
-      rx += real(c.rx) * v;
-      ry += real(c.ry) * v;
-    }
-    a.M[(size_t)q * P + n] = dpsi;
-    drho += dpsi;
-    jx += rx;
-    jy += ry;
-    const real Qx = a.tab.qx[q], Qy = a.tab.qy[q], Fx = a.tab.fx[q], Fy = a.tab.fy[q];
-    txx += dpsi * Fx * Qx;
-    txy += dpsi * Fx * Qy;
-    tyy += dpsi * Fy * Qy;
-  }
-  a.M[(size_t)(nq + M_DRHO) * P + n] = drho;
-  a.M[(size_t)(nq + M_JX) * P + n] = jx;
-  a.M[(size_t)(nq + M_JY) * P + n] = jy;
-  a.M[(size_t)(nq + M_THXX) * P + n] = a.hl2h * txx;
-  a.M[(size_t)(nq + M_THXY) * P + n] = a.hl2h * txy;
-  a.M[(size_t)(nq + M_THYY) * P + n] = a.hl2h * tyy;
-}
-
-// ------------------------------------------------------------------ step
-// One collision of the pulled state, written unstreamed to dst:
-//   U from M (tile + 1-node halo in shared memory), grad U by central
-//   differences; solvent J_S(f) = (2 tau2 J_S(g) + rho_S U + tau2 rho a) /
-//   (2 tau2 + 1), u_S = J_S(f) / rho_S; polymer J^r_eq = psi U + tau2 D,
-//   D = (H ell^2 / 2) phi_q Q (Q . grad_r psi), J^Q_eq = psi (Q . grad U - kappa phi_q Q)
-//   (phi_q Q = spring force / H: phi_q = 1 Hookean, 1 / (1 - Q^2/Q0^2) FENE),
-//   J(f) = (2 tau2 J(g) + J_eq) / (2 tau2 + 1);
-//   g' = (1 - 2 beta) g + 2 beta [(1 - tau1/tau2) f* + (tau1/tau2) f^eq]
-//        + (1 - beta) S_i,   beta = 1 / (2 tau1 + 1)
-// with the quadratic solvent equilibria (Eq. dis_eq), the linear polymer
-// equilibria (Eqs. feq_rq_space, fstar_rq_space) and the Guo source S_i of the
-// force density rho a (solvent only).
-template <typename real, typename S>
-__global__ void __launch_bounds__(256) step_kernel(KernelArgs<real> a) {
-  __shared__ real sUx[TY + 2][TX + 2];
-  __shared__ real sUy[TY + 2][TX + 2];
-  // pull tables in shared memory (dynamic: nq * 25 shift differences, then plane entries)
-  extern __shared__ __align__(16) unsigned char step_smem[];
-  real* s_delta = reinterpret_cast<real*>(step_smem);
-  int* s_pull = reinterpret_cast<int*>(step_smem + sizeof(real) * (size_t)a.nq * 25);
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  for (int k = tid; k < a.nq * 25; k += TX * TY) {
-    s_delta[k] = a.tab.delta[k];
-    s_pull[k] = a.tab.pull[k];
-  }
-  for (int k = tid; k < (TX + 2) * (TY + 2); k += TX * TY) {
-    const int hx = k % (TX + 2), hy = k / (TX + 2);
-    const int gx = wrapi(x0 - 1 + hx, a.nx), gy = wrapi(y0 - 1 + hy, a.ny);
-    real ux, uy, rho;
-    mixture_velocity(a, gx, gy, ux, uy, rho);
-    sUx[hy][hx] = ux;
-    sUy[hy][hx] = uy;
-  }
-  __syncthreads();
-  const int x = x0 + tx, y = y0 + ty;
-  if (x >= a.nx || y >= a.ny) return;
-  const real Ux = sUx[ty + 1][tx + 1], Uy = sUy[ty + 1][tx + 1];
-  const real G00 = real(0.5) * (sUx[ty + 1][tx + 2] - sUx[ty + 1][tx]);  // d_x U_x
-  const real G01 = real(0.5) * (sUy[ty + 1][tx + 2] - sUy[ty + 1][tx]);  // d_x U_y
-  const real G10 = real(0.5) * (sUx[ty + 2][tx + 1] - sUx[ty][tx + 1]);  // d_y U_x
-  const real G11 = real(0.5) * (sUy[ty + 2][tx + 1] - sUy[ty][tx + 1]);  // d_y U_y
-
-  const Offsets off = node_offsets(x, y, a.nx, a.ny, a.pitch);
-  const size_t P = a.plane;
-  const size_t n = off.o[4];
-  const int nq = a.nq;
-  const real rho = a.rho0 + a.M[(size_t)(nq + M_DRHO) * P + n];
-  const real force = rho * a.tab.arow[y];
-  using SS = SolventT<S>;
-  const S* __restrict__ src = (const S*)a.src;
-  S* __restrict__ dst = (S*)a.dst;
-  const SS* __restrict__ ssrc = solvent_planes<S>(a.src, P, a.nq);
-  SS* __restrict__ sdst = solvent_planes<S>(a.dst, P, a.nq);
-
-  // ---- solvent
-  {
-    real h[9];
-    real drs = 0, jsx = 0, jsy = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      h[i] = from_store<real>(ssrc[(size_t)i * P + off.o[shift_index(-c9x(i), -c9y(i))]]);
-      drs += h[i];
-      jsx += real(c9x(i)) * h[i];
-      jsy += real(c9y(i)) * h[i];
-    }
-    const real rs = real(1) + drs;
-    const real jfx = (a.c2 * jsx + rs * Ux + a.tau2 * force) * a.inv_c2p1;
-    const real jfy = (a.c2 * jsy + rs * Uy) * a.inv_c2p1;
-    const real usx = jfx / rs, usy = jfy / rs;
-    const real vx = a.omr * usx + a.r * Ux, vy = a.omr * usy + a.r * Uy;
-    const real sq = a.omr * (usx * usx + usy * usy) + a.r * (Ux * Ux + Uy * Uy);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const real cx = real(c9x(i)), cy = real(c9y(i));
-      const real cus = cx * usx + cy * usy, cu = cx * Ux + cy * Uy;
-      const real feq_dev =
-          real(w9(i)) * (drs + rs * (real(3) * (cx * vx + cy * vy) +
-                                     real(4.5) * (a.omr * cus * cus + a.r * cu * cu) -
-                                     real(1.5) * sq));
-      const real srcterm = real(w9(i)) * (real(3) * (cx - Ux) + real(9) * cu * cx) * force;
-      sdst[(size_t)i * P + n] = to_store<SS>(a.om2b * h[i] + a.tb * feq_dev + a.omb * srcterm);
-    }
-  }
-
-  // ---- polymer, one Q-node at a time; the populations (and psi neighbours) of
-  // Q-node q + 1 are loaded while Q-node q is collided
-  const size_t nxm = off.o[3], nxp = off.o[5], nym = off.o[1], nyp = off.o[7];
-  auto pull = [&](int q, int i) {
-    const V4 c = c25(i);
-    const int e = s_pull[q * 25 + i];
-    const size_t o = e >= 0 ? off.o[shift_index(-c.rx, -c.ry)] : off.o[4];
-    return from_store<real>(src[(size_t)(e >= 0 ? e : ~e) * P + o]);
-  };
-  real h[25], mn[4];
-  if (nq > 0) {
-#pragma unroll
-    for (int i = 0; i < 25; ++i) h[i] = pull(0, i);
-    mn[0] = a.M[nxp];
-    mn[1] = a.M[nxm];
-    mn[2] = a.M[nyp];
-    mn[3] = a.M[nym];
-  }
-  for (int q = 0; q < nq; ++q) {
-    const bool more = q + 1 < nq;
-    const real dpx = real(0.5) * (mn[0] - mn[1]);
-    const real dpy = real(0.5) * (mn[2] - mn[3]);
-    if (more) {
-      const real* Mq = a.M + (size_t)(q + 1) * P;
-      mn[0] = Mq[nxp];
-      mn[1] = Mq[nxm];
-      mn[2] = Mq[nyp];
-      mn[3] = Mq[nym];
-    }
-    real dpsi = 0, rx = 0, ry = 0, qx = 0, qy = 0;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      const V4 c = c25(i);
-      h[i] = h[i] * a.pinv + s_delta[q * 25 + i];
-      dpsi += h[i];
-      rx += real(c.rx) * h[i];
-      ry += real(c.ry) * h[i];
-      qx += real(c.qx) * h[i];
-      qy += real(c.qy) * h[i];
-    }
-    const real Qx = a.tab.qx[q], Qy = a.tab.qy[q], Fx = a.tab.fx[q], Fy = a.tab.fy[q];
-    const real psi = a.tab.psi0[q] + dpsi;
-    const real qg = Qx * dpx + Qy * dpy;
-    const real jrex = psi * Ux + a.tau2 * a.hl2h * Fx * qg;
-    const real jrey = psi * Uy + a.tau2 * a.hl2h * Fy * qg;
-    const real jqex = psi * (Qx * G00 + Qy * G10 - a.kappa * Fx);
-    const real jqey = psi * (Qx * G01 + Qy * G11 - a.kappa * Fy);
-    // mixture (1 - r) J(f) + r J_eq of the two equilibria's momenta
-    const real mrx = a.omr * (a.c2 * rx + jrex) * a.inv_c2p1 + a.r * jrex;
-    const real mry = a.omr * (a.c2 * ry + jrey) * a.inv_c2p1 + a.r * jrey;
-    const real mqx = a.omr * (a.c2 * qx + jqex) * a.inv_c2p1 + a.r * jqex;
-    const real mqy = a.omr * (a.c2 * qy + jqey) * a.inv_c2p1 + a.r * jqey;
-    S* dq = dst + (size_t)(9 + 25 * q) * P + n;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      const V4 c = c25(i);
-      const real fdev = real(w25(i)) * (dpsi + real(3) * (mrx * real(c.rx) + mry * real(c.ry) +
-                                                           mqx * real(c.qx) + mqy * real(c.qy)));
-      dq[(size_t)i * P] = to_store<S>((a.om2b * h[i] + a.tb * fdev) * a.pscale);
-      if (more) h[i] = pull(q + 1, i);
-    }
-  }
-}
-
-// The same step with the component stresses quasi-conserved (Sec. V, Eq.
-// quasieq2; f*_S and f**_P of Sec. VI): the targets carry the equilibrium
-// momenta (rho_S U; J^r_eq = psi U + tau1 D, J^Q_eq) and the current stresses
-// of f, P(f) = (2 tau2 P(g) + P_eq [+ tau2 (F U + U F) for the solvent]) /
-// (2 tau2 + 1), entered through the second-order Hermite terms normalised so
-// that <f**, vv> = P; momenta relax at tau1, stresses at tau2.
-template <typename real, typename S>
-__global__ void __launch_bounds__(256) step_stress_kernel(KernelArgs<real> a) {
-  __shared__ real sUx[TY + 2][TX + 2];
-  __shared__ real sUy[TY + 2][TX + 2];
-  // pull tables in shared memory (dynamic: nq * 25 shift differences, then plane entries)
-  extern __shared__ __align__(16) unsigned char stress_smem[];
-  real* s_delta = reinterpret_cast<real*>(stress_smem);
-  int* s_pull = reinterpret_cast<int*>(stress_smem + sizeof(real) * (size_t)a.nq * 25);
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  for (int k = tid; k < a.nq * 25; k += TX * TY) {
-    s_delta[k] = a.tab.delta[k];
-    s_pull[k] = a.tab.pull[k];
-  }
-  for (int k = tid; k < (TX + 2) * (TY + 2); k += TX * TY) {
-    const int hx = k % (TX + 2), hy = k / (TX + 2);
-    const int gx = wrapi(x0 - 1 + hx, a.nx), gy = wrapi(y0 - 1 + hy, a.ny);
-    real ux, uy, rho;
-    mixture_velocity(a, gx, gy, ux, uy, rho);
-    sUx[hy][hx] = ux;
-    sUy[hy][hx] = uy;
-  }
-  __syncthreads();
-  const int x = x0 + tx, y = y0 + ty;
-  if (x >= a.nx || y >= a.ny) return;
-  const real Ux = sUx[ty + 1][tx + 1], Uy = sUy[ty + 1][tx + 1];
-  const real G00 = real(0.5) * (sUx[ty + 1][tx + 2] - sUx[ty + 1][tx]);
-  const real G01 = real(0.5) * (sUy[ty + 1][tx + 2] - sUy[ty + 1][tx]);
-  const real G10 = real(0.5) * (sUx[ty + 2][tx + 1] - sUx[ty][tx + 1]);
-  const real G11 = real(0.5) * (sUy[ty + 2][tx + 1] - sUy[ty][tx + 1]);
-  const Offsets off = node_offsets(x, y, a.nx, a.ny, a.pitch);
-  const size_t P = a.plane;
-  const size_t n = off.o[4];
-  const int nq = a.nq;
-  const real rho = a.rho0 + a.M[(size_t)(nq + M_DRHO) * P + n];
-  const real force = rho * a.tab.arow[y];
-  using SS = SolventT<S>;
-  const S* __restrict__ src = (const S*)a.src;
-  S* __restrict__ dst = (S*)a.dst;
-  const SS* __restrict__ ssrc = solvent_planes<S>(a.src, P, a.nq);
-  SS* __restrict__ sdst = solvent_planes<S>(a.dst, P, a.nq);
-  const real cs2 = real(1) / real(3);
-  const real rmix = a.r, omr = a.omr;
-
-  // ---- solvent
-  {
-    real h[9];
-    real drs = 0, pxx = 0, pxy = 0, pyy = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      h[i] = from_store<real>(ssrc[(size_t)i * P + off.o[shift_index(-c9x(i), -c9y(i))]]);
-      drs += h[i];
-      pxx += real(c9x(i) * c9x(i)) * h[i];
-      pxy += real(c9x(i) * c9y(i)) * h[i];
-      pyy += real(c9y(i) * c9y(i)) * h[i];
-    }
-    const real rs = real(1) + drs;
-    // P(g) - P_eq from the deviations (P(g) = c_s^2 I + sum h c c, P_eq = rho_S (c_s^2 I + U U)),
-    // then P(f) - rho_S c_s^2 I = [2 tau2 (P(g) - P_eq) + tau2 (F U + U F)] / (2 tau2 + 1) + rho_S U U
-    const real dxx = pxx - drs * cs2 - rs * Ux * Ux, dxy = pxy - rs * Ux * Uy;
-    const real dyy = pyy - drs * cs2 - rs * Uy * Uy;
-    const real fxx = (a.c2 * dxx + a.tau2 * real(2) * force * Ux) * a.inv_c2p1 + rs * Ux * Ux;
-    const real fxy = (a.c2 * dxy + a.tau2 * force * Uy) * a.inv_c2p1 + rs * Ux * Uy;
-    const real fyy = a.c2 * dyy * a.inv_c2p1 + rs * Uy * Uy;
-    const real usq = Ux * Ux + Uy * Uy;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const real cx = real(c9x(i)), cy = real(c9y(i));
-      const real cu = cx * Ux + cy * Uy;
-      const real pneq = fxx * (cx * cx - cs2) + real(2) * fxy * cx * cy + fyy * (cy * cy - cs2);
-      const real fss_dev = real(w9(i)) * (drs + real(3) * rs * cu + real(4.5) * pneq);
-      const real feq_dev = real(w9(i)) * (drs + rs * (real(3) * cu + real(4.5) * cu * cu - real(1.5) * usq));
-      const real srcterm = real(w9(i)) * (real(3) * (cx - Ux) + real(9) * cu * cx) * force;
-      sdst[(size_t)i * P + n] =
-          to_store<SS>(a.om2b * h[i] + a.tb * (omr * fss_dev + rmix * feq_dev) + a.omb * srcterm);
-    }
-  }
-
-  // ---- polymer, one Q-node at a time; the populations (and psi neighbours) of
-  // Q-node q + 1 are loaded while Q-node q is collided
-  const size_t nxm = off.o[3], nxp = off.o[5], nym = off.o[1], nyp = off.o[7];
-  auto pull = [&](int q, int i) {
-    const V4 c = c25(i);
-    const int e = s_pull[q * 25 + i];
-    const size_t o = e >= 0 ? off.o[shift_index(-c.rx, -c.ry)] : off.o[4];
-    return from_store<real>(src[(size_t)(e >= 0 ? e : ~e) * P + o]);
-  };
-  real h[25], mn[4];
-  if (nq > 0) {
-#pragma unroll
-    for (int i = 0; i < 25; ++i) h[i] = pull(0, i);
-    mn[0] = a.M[nxp];
-    mn[1] = a.M[nxm];
-    mn[2] = a.M[nyp];
-    mn[3] = a.M[nym];
-  }
-  for (int q = 0; q < nq; ++q) {
-    const bool more = q + 1 < nq;
-    const real dpx = real(0.5) * (mn[0] - mn[1]);
-    const real dpy = real(0.5) * (mn[2] - mn[3]);
-    if (more) {
-      const real* Mq = a.M + (size_t)(q + 1) * P;
-      mn[0] = Mq[nxp];
-      mn[1] = Mq[nxm];
-      mn[2] = Mq[nyp];
-      mn[3] = Mq[nym];
-    }
-    real dpsi = 0;
-    // second moments of the deviations: vv (3), v Qdot (4), Qdot Qdot (3)
-    real rxx = 0, rxy = 0, ryy = 0, cxx = 0, cxy = 0, cyx = 0, cyy = 0, qxx = 0, qxy = 0, qyy = 0;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      const V4 c = c25(i);
-      h[i] = h[i] * a.pinv + s_delta[q * 25 + i];
-      dpsi += h[i];
-      rxx += real(c.rx * c.rx) * h[i];
-      rxy += real(c.rx * c.ry) * h[i];
-      ryy += real(c.ry * c.ry) * h[i];
-      cxx += real(c.rx * c.qx) * h[i];
-      cxy += real(c.rx * c.qy) * h[i];
-      cyx += real(c.ry * c.qx) * h[i];
-      cyy += real(c.ry * c.qy) * h[i];
-      qxx += real(c.qx * c.qx) * h[i];
-      qxy += real(c.qx * c.qy) * h[i];
-      qyy += real(c.qy * c.qy) * h[i];
-    }
-    const real Qx = a.tab.qx[q], Qy = a.tab.qy[q], Fx = a.tab.fx[q], Fy = a.tab.fy[q];
-    const real psi = a.tab.psi0[q] + dpsi;
-    const real qg = Qx * dpx + Qy * dpy;
-    const real jrex = psi * Ux + a.tau_m * a.hl2h * Fx * qg;
-    const real jrey = psi * Uy + a.tau_m * a.hl2h * Fy * qg;
-    const real jqex = psi * (Qx * G00 + Qy * G10 - a.kappa * Fx);
-    const real jqey = psi * (Qx * G01 + Qy * G11 - a.kappa * Fy);
-    // P(g) - P_eq = (the deviations' moments) - dpsi c_s^2 I on the diagonal blocks (P_eq =
-    // psi c_s^2 I), so P(f) - P_eq = 2 tau2 (P(g) - P_eq) / (2 tau2 + 1)
-    auto dg = [&](real m) { return a.c2 * (m - dpsi * cs2) * a.inv_c2p1; };
-    auto od = [&](real m) { return a.c2 * m * a.inv_c2p1; };
-    const real Rxx = dg(rxx), Rxy = od(rxy), Ryy = dg(ryy);
-    const real Qxx = dg(qxx), Qxy = od(qxy), Qyy = dg(qyy);
-    const real Cxx = od(cxx), Cxy = od(cxy), Cyx = od(cyx), Cyy = od(cyy);
-    S* dq = dst + (size_t)(9 + 25 * q) * P + n;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      const V4 c = c25(i);
-      const real vx = real(c.rx), vy = real(c.ry), wx = real(c.qx), wy = real(c.qy);
-      const real lin = dpsi + real(3) * (jrex * vx + jrey * vy + jqex * wx + jqey * wy);
-      const real sdiag = Rxx * (vx * vx - cs2) + real(2) * Rxy * vx * vy + Ryy * (vy * vy - cs2) +
-                         Qxx * (wx * wx - cs2) + real(2) * Qxy * wx * wy + Qyy * (wy * wy - cs2);
-      const real scross = Cxx * vx * wx + Cxy * vx * wy + Cyx * vy * wx + Cyy * vy * wy;
-      const real fss_dev = real(w25(i)) * (lin + real(4.5) * sdiag + real(9) * scross);
-      const real feq_dev = real(w25(i)) * lin;
-      dq[(size_t)i * P] = to_store<S>((a.om2b * h[i] + a.tb * (omr * fss_dev + rmix * feq_dev)) * a.pscale);
-      if (more) h[i] = pull(q + 1, i);
-    }
-  }
 }
 
 // ------------------------------------------------------------- observers
@@ -812,37 +419,6 @@ cudaError_t launch_init(const KernelArgs<real>& a, cudaStream_t s) {
   init_kernel<real, S><<<node_grid(a.nx, a.ny), dim3(TX, TY), 0, s>>>(a);
   return cudaGetLastError();
 }
-template <typename real, typename S>
-cudaError_t launch_moments(const KernelArgs<real>& a, cudaStream_t s) {
-  const size_t smem = (sizeof(real) + sizeof(int)) * (size_t)a.nq * 25;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(moments_kernel<real, S>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  moments_kernel<real, S><<<node_grid(a.nx, a.ny), dim3(TX, TY), smem, s>>>(a);
-  return cudaGetLastError();
-}
-template <typename real, typename S>
-cudaError_t launch_step(const KernelArgs<real>& a, cudaStream_t s) {
-  const size_t smem = (sizeof(real) + sizeof(int)) * (size_t)a.nq * 25;   // pull tables
-  if (a.qe == TFKT_QE_STRESS) {
-    if (smem > 40 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(step_stress_kernel<real, S>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    step_stress_kernel<real, S><<<node_grid(a.nx, a.ny), dim3(TX, TY), smem, s>>>(a);
-  } else {
-    if (smem > 40 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(step_kernel<real, S>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    step_kernel<real, S><<<node_grid(a.nx, a.ny), dim3(TX, TY), smem, s>>>(a);
-  }
-  return cudaGetLastError();
-}
 template <typename real>
 cudaError_t launch_velocity(const KernelArgs<real>& a, cudaStream_t s) {
   velocity_kernel<real><<<node_grid(a.nx, a.ny), dim3(TX, TY), 0, s>>>(a);
@@ -878,8 +454,6 @@ cudaError_t launch_diag(const KernelArgs<real>& a, double* partials, int nblocks
 
 #define TFKT_INSTANTIATE_POP(real, S)                                                          \
   template cudaError_t launch_init<real, S>(const KernelArgs<real>&, cudaStream_t);           \
-  template cudaError_t launch_moments<real, S>(const KernelArgs<real>&, cudaStream_t);        \
-  template cudaError_t launch_step<real, S>(const KernelArgs<real>&, cudaStream_t);           \
   template cudaError_t launch_populations<real, S>(const KernelArgs<real>&, double*,          \
                                                    cudaStream_t);
 #define TFKT_INSTANTIATE(real)                                                                 \

@@ -64,10 +64,10 @@ tfkt_status moments_noalloc(const tfkt_params& p, const Lattice& L, const void* 
   o = align_up(o + (size_t)L.nm * L.plane * sz, A);
   const size_t off_U = o;
   o = align_up(o + 2 * L.plane * sz, A);
-  constexpr int NT = 9, KPULL = 5;
+  constexpr int NT = 8, KROW = 5;
   size_t off_t[NT];
-  const size_t tsz[NT] = {nq * sz, nq * sz, nq * sz, nq * sz, nq * sz, nq * 25 * sizeof(int),
-                          nq * 25 * sz, (size_t)L.ny * sz, (size_t)L.ny * sz};
+  const size_t tsz[NT] = {nq * sz, nq * sz, nq * sz, nq * sz, nq * sz, nq * sizeof(QRow<real>),
+                          (size_t)L.ny * sz, (size_t)L.ny * sz};
   for (int k = 0; k < NT; ++k) {
     off_t[k] = o;
     o = align_up(o + tsz[k], A);
@@ -93,12 +93,13 @@ tfkt_status moments_noalloc(const tfkt_params& p, const Lattice& L, const void* 
     if (!g_tables_valid[dev] || !same_params(g_tables_of[dev], p)) {
       g_tables_valid[dev] = false;
       const HostTables t = build_tables(L);
-      const std::vector<double>* src[NT] = {&t.qx,    &t.qy,    &t.fx,   &t.fy,  &t.psi0,
-                                            nullptr, &t.delta, &t.arow, &t.urow};
+      const std::vector<double>* src[NT] = {&t.qx,   &t.qy,   &t.fx,   &t.fy,
+                                            &t.psi0, nullptr, &t.arow, &t.urow};
       std::vector<real> conv[NT];
+      const std::vector<QRow<real>> rows = build_rows<real>(L, t);
       for (int k = 0; k < NT; ++k) {
-        if (k == KPULL) {
-          e = cudaMemcpyAsync(b + off_t[k], t.pull.data(), tsz[k], cudaMemcpyHostToDevice, stream);
+        if (k == KROW) {
+          e = cudaMemcpyAsync(b + off_t[k], rows.data(), tsz[k], cudaMemcpyHostToDevice, stream);
         } else {
           conv[k].assign(src[k]->begin(), src[k]->end());
           e = cudaMemcpyAsync(b + off_t[k], conv[k].data(), tsz[k], cudaMemcpyHostToDevice, stream);
@@ -121,6 +122,7 @@ tfkt_status moments_noalloc(const tfkt_params& p, const Lattice& L, const void* 
   a.nx = L.nx;
   a.ny = L.ny;
   a.nq = L.nq;
+  a.mom_warps = moment_warps(L);
   a.pitch = L.pitch;
   a.plane = L.plane;
   a.tau2 = (real)L.tau2;
@@ -139,10 +141,9 @@ tfkt_status moments_noalloc(const tfkt_params& p, const Lattice& L, const void* 
   a.tab.fx = (const real*)(b + off_t[2]);
   a.tab.fy = (const real*)(b + off_t[3]);
   a.tab.psi0 = (const real*)(b + off_t[4]);
-  a.tab.pull = (const int*)(b + off_t[5]);
-  a.tab.delta = (const real*)(b + off_t[6]);
-  a.tab.arow = (const real*)(b + off_t[7]);
-  a.tab.urow = (const real*)(b + off_t[8]);
+  a.tab.row = (const QRow<real>*)(b + off_t[5]);
+  a.tab.arow = (const real*)(b + off_t[6]);
+  a.tab.urow = (const real*)(b + off_t[7]);
   // every plane read below is written first by these kernels: the moments
   // kernel writes all M planes of every node, the velocity kernel both U
   // planes of every node, so nothing needs clearing between calls (the tables

@@ -1,0 +1,95 @@
+"""Kernel paths of the step at the sizes where they can go wrong, against the oracle:
+the Q-split kernels (small grids, ragged grids, FP64) at node counts around a group
+of 32 nodes, Q-node counts around the warps of a block and grids on both sides of
+the line to the fused kernel, and the fused kernel just above that line.
+Tolerances are those of tests/test_gpu_parity.py: FP64 1e-12, FP32 2e-5, FP16
+storage 3e-3 of the field's scale."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"FP64": 1e-12, "FP32": 2e-5, "FP16": 3e-3}
+SCALE = {"ux": "u", "uy": "u", "cxx": "c", "cxy": "c", "cyy": "c", "thxx": "t", "thxy": "t",
+         "thyy": "t", "rho_s": "rho_s", "psi_tot": "psi_tot"}
+
+
+@pytest.fixture(scope="module")
+def T():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2201_10132_gb300 import build, tfkt
+    build.build()
+    return tfkt
+
+
+def _params(T, nx, ny, S, R, prec, stress=False, fene=0.0):
+    return T.Params(nx, ny, S, R, 5.0, 2.0 if stress or fene else 0.5, 0.5 if stress else 0.2, 0.05, 1,
+                    0.03 if stress else 0.0, 0.0, 1, getattr(T, prec), fene, int(stress))
+
+
+def _check(T, O, p, steps, prec):
+    from paper_2201_10132_gb300.inputs import perturbation
+    pert = perturbation(p.nx, p.ny, 7, 0.05, 0.05) if p.nx * p.ny > 1 else None
+    o = O.Oracle(O.map_params(p.nx, p.ny, p.q_side, p.q_radius, p.re, p.wi, p.beta, p.u0,
+                              p.k_periods, p.tau2, 0.0, p.fene_b, p.qe_model))
+    o.init(pert, p.ic_mode)
+    o.step(steps)
+    f = o.fields()
+    with T.Solver(p, pert) as s:
+        s.step(steps)
+        g = s.moments(list(SCALE))
+    scale = {}
+    for k, t in SCALE.items():
+        scale[t] = max(scale.get(t, 0.0), np.abs(f[k]).max())
+    for k, t in SCALE.items():
+        err = np.abs(g[k] - f[k]).max() / max(scale[t], 1e-300)
+        assert err < TOL[prec], (k, err)
+
+
+# 1, 4, 5 and 9 Q-nodes, then 12, 32, 29 and 52
+SIZES = [(1, 33, 1, 1.0), (31, 1, 2, 1.0), (32, 8, 3, 1.0), (11, 3, 3, 1.5),
+         (33, 31, 4, 2.0), (5, 13, 6, 3.0), (97, 50, 7, 3.0), (72, 72, 8, 4.0)]
+
+
+# (FP16 storage leaves out the one-row grid: its viscous length is 1/(2 pi) node, its stress
+# mode hardly damped, and the rounding of the stored populations reaches 1e-2 of the
+# velocity with any of the kernels.)
+@pytest.mark.parametrize("prec,nx,ny,S,R", [(prec,) + c for prec in TOL for c in SIZES
+                                            if not (prec == "FP16" and c[1] == 1)])
+def test_q_split_sizes(T, oracle_mod, nx, ny, S, R, prec):
+    _check(T, oracle_mod, _params(T, nx, ny, S, R, prec), 6, prec)
+
+
+@pytest.mark.parametrize("prec,stress,fene", [("FP32", False, 0.0), ("FP16", False, 0.0),
+                                              ("FP32", True, 0.0), ("FP16", True, 0.0),
+                                              ("FP32", False, 3.1), ("FP32", True, 3.1)])
+@pytest.mark.parametrize("nx,ny", [(160, 160), (416, 64)])   # 100 and 104 tiles of 32 x 8
+def test_both_sides_of_the_tile_line(T, oracle_mod, nx, ny, prec, stress, fene):
+    _check(T, oracle_mod, _params(T, nx, ny, 6, 3.0, prec, stress, fene), 4, prec)
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(64, 32, "FP32"), (40, 24, "FP32"), (416, 64, "FP16")])
+def test_steps_captured_in_a_graph(T, nx, ny, prec):
+    """tfkt_step under the caller's stream capture: three replays of two captured steps
+    leave the state of six plain steps."""
+    import torch
+    from paper_2201_10132_gb300.inputs import perturbation
+    p = _params(T, nx, ny, 6, 3.0, prec)
+    pert = perturbation(nx, ny, 3, 0.05, 0.05)
+    with T.Solver(p, pert) as s:
+        s.step(6)
+        ref = s.moments()
+    st = torch.cuda.Stream()
+    with T.Solver(p, pert, stream=st.cuda_stream) as s:
+        s.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            s.step(2)
+        with torch.cuda.stream(st):
+            for _ in range(3):
+                g.replay()
+        st.synchronize()
+        got = s.moments()
+    for k in ref:
+        assert np.array_equal(got[k], ref[k], equal_nan=True), k
