@@ -91,8 +91,8 @@ typedef struct {
                             anti-diffusive in r, make the step unstable; keep the disk
                             well inside Q0. */
   int32_t qe_model;      /* tfkt_qe_model: which variables the collision holds
-                            quasi-conserved (Sec. V); both models take the fused
-                            kernel on grids of 32 x 8 tiles */
+                            quasi-conserved (Sec. V); both models run on
+                               every kernel path */
 } tfkt_params;
 
 /* Derived lattice parameters and layout of a context. */
@@ -118,7 +118,9 @@ typedef struct tfkt_ctx tfkt_ctx;
 /* Kernels timed by tfkt_step_profiled. */
 enum {
   TFKT_K_MOMENTS = 0,  /* pull-read of all populations -> moment planes */
-  TFKT_K_STEP,         /* two-pass path: pull, collide and write of all populations */
+  TFKT_K_STEP,         /* two-pass path (FP64 and up to 100 tiles where the grid is no multiple
+                          of the 32 x 8 tile, or too many Q-nodes for the fused kernel): pull,
+                          collide and write of all populations */
   TFKT_K_FUSED,        /* fused path: pull, collide, write and next-step moments (the moments
                           excepted in FP64 and on grids of up to 100 tiles) */
   TFKT_K_FIXUP,        /* fused path: completion of the next step's moments (of the tiles'
@@ -369,11 +371,11 @@ tfkt_status tfkt_batch_destroy(tfkt_batch* b);
    slab k+1's TFKT_SLAB_LOW unpack and slab k's TFKT_SLAB_LOW pack to slab
    k-1's TFKT_SLAB_HIGH unpack (periodic: the last slab's high neighbour is
    the first slab). The ghost width is one row of the fused path's 32 x 8
-   tiles: with y0 and ny_local multiples of 8 (and nx of 32) every slab takes
-   the fused path on tiles that are the single-domain run's tiles, so every
-   owned node sums its arrivals in the same order and the owned rows are bit-
-   identical to the single-domain run (the two-pass path is bit-identical for
-   any split). The learned block does not run on a slab context (EINVAL). */
+   tiles, and a slab's tile rows are those of the single-domain run, so every
+   owned node sums its arrivals in the same order. The owned rows are bit-
+   identical to the single-domain run: for any split in FP64, on runs of up to
+   100 tiles and on runs whose nx is no multiple of 32 or whose ny is none of 8,
+   and on the others with y0 and ny_local multiples of 8. The learned block does not run on a slab context (EINVAL). */
 #define TFKT_SLAB_GHOST 8
 enum { TFKT_SLAB_LOW = 0, TFKT_SLAB_HIGH = 1 };
 

@@ -146,9 +146,7 @@ double polymer_scale(const Lattice& L) {
 // whole run does, so the whole run's size decides.
 constexpr size_t SPLIT_TILES = 100;
 bool split_path(const Lattice& L) {
-  if (L.precision == TFKT_FP64) return true;
-  const size_t ny = L.ny_global > 0 ? L.ny_global : L.ny;
-  return (size_t)(L.nx / TX) * (ny / TY) <= SPLIT_TILES;
+  return L.precision == TFKT_FP64 || run_tiles(L) <= SPLIT_TILES;
 }
 
 size_t store_size(const Lattice& L) {
@@ -194,9 +192,10 @@ size_t layout(const Lattice& L, Workspace* w) {
     w->off_M2 = o;
     o = align_up(o + (size_t)L.nm * L.plane * sz, A);
     w->off_exp = o;
-    o = align_up(o + fused_export_capacity(L.nx, L.ny, L.nq) * sz, A);
+    o = align_up(o + fused_export_capacity(L) * sz, A);
     w->off_ftab = o;
-    o = align_up(o + (size_t)L.nq * (9 * sizeof(int) + sz + 25 * sizeof(long long)) + 2 * A, A);
+    o = align_up(o + (size_t)L.nq * (9 * sizeof(int) + sz + 25 * sizeof(long long)) +
+                     max_tile_rows(L) * sizeof(int2) + 3 * A, A);
   }
   return o;
 }
@@ -345,6 +344,8 @@ FusedArgs<real> make_fused(const Ctx* c) {
   f.tgt = (const int*)(base + c->ws.off_ftab);
   f.dpsi = (const real*)(base + c->ws.off_ftab + align_up((size_t)L.nq * 9 * sizeof(int), 256));
   f.poff = (const long long*)((const char*)f.dpsi + align_up((size_t)L.nq * sizeof(real), 256));
+  f.trow = (const int2*)((const char*)f.poff + align_up((size_t)L.nq * 25 * sizeof(long long), 256));
+  f.ntrow = c->ntrow;
   f.dvx = (real)c->dvx;
   f.dvy = (real)c->dvy;
   return f;
@@ -356,7 +357,12 @@ tfkt_status upload_fused_tables(Ctx* c, const HostTables& t) {
   std::vector<double> dpsi;
   std::vector<long long> poff;
   fused_tables(c->L, t, tgt, dpsi, c->dvx, c->dvy, poff);
+  const std::vector<int2> trow = tile_rows(c->L);
+  c->ntrow = (int)trow.size();
   FusedArgs<real> f = make_fused<real>(c);
+  if (c->ntrow)
+    TFKT_CUDA(c, cudaMemcpy((void*)f.trow, trow.data(), trow.size() * sizeof(int2),
+                            cudaMemcpyHostToDevice));
   std::vector<real> d(dpsi.begin(), dpsi.end());
   TFKT_CUDA(c, cudaMemcpy((void*)f.poff, poff.data(), poff.size() * sizeof(long long),
                           cudaMemcpyHostToDevice));
@@ -437,6 +443,18 @@ tfkt_status ensure_moments(Ctx* c) {
 // learned-block increment rides on the pull of the fused kernel only.
 inline bool step_split(const Ctx* c) { return c->split && !c->lpm_pending; }
 
+// The fused kernel and its fix-up (FP64 contexts step with the Q-split kernels).
+template <typename real, typename S>
+cudaError_t fused_kernel(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+  if constexpr (std::is_same<real, float>::value) return launch_step_fused<real, S>(a, f, s);
+  else return cudaErrorInvalidValue;
+}
+template <typename real>
+cudaError_t fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+  if constexpr (std::is_same<real, float>::value) return launch_fixup<real>(a, f, s);
+  else return cudaErrorInvalidValue;
+}
+
 // One step. Fused path: the step kernel also produces the next state's
 // moment planes (completed at tile borders by the fix-up kernel), or, where the
 // Q-split kernels are faster (split_path), the collision and then the moments
@@ -463,8 +481,8 @@ tfkt_status do_step(Ctx* c, int64_t n) {
         TFKT_CUDA(c, launch_moments<real, S>(next_moments_args(a, f), c->stream, dep));
       } else {
         if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
-        TFKT_CUDA(c, launch_step_fused<real, S>(a, f, c->stream));
-        TFKT_CUDA(c, launch_fixup<real>(a, f, c->stream));
+        TFKT_CUDA(c, (fused_kernel<real, S>(a, f, c->stream)));
+        TFKT_CUDA(c, fixup<real>(a, f, c->stream));
       }
       c->lpm_pending = false;
       c->mcur ^= 1;
@@ -535,13 +553,13 @@ tfkt_status do_step_profiled(Ctx* c, int64_t n, double* ms, int64_t* launches) {
       const bool split = step_split(c);
       if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
       tfkt_status s = timed(TFKT_K_FUSED, [&] {
-        return split ? launch_step<real, S>(a, c->stream) : launch_step_fused<real, S>(a, f, c->stream);
+        return split ? launch_step<real, S>(a, c->stream) : fused_kernel<real, S>(a, f, c->stream);
       });
       if (s != TFKT_OK) return s;
       c->lpm_pending = false;
       s = timed(TFKT_K_FIXUP, [&] {
         return split ? launch_moments<real, S>(next_moments_args(a, f), c->stream)
-                     : launch_fixup<real>(a, f, c->stream);
+                     : fixup<real>(a, f, c->stream);
       });
       if (s != TFKT_OK) return s;
       c->mcur ^= 1;

@@ -13,6 +13,11 @@
 // which the fix-up kernel adds in a fixed order. No atomics: results do not
 // depend on scheduling.
 //
+// Grids that are no multiples of the tile end in partial tiles (template parameter
+// RAGGED; whole tiles keep their own instantiation). The partial tiles' idle threads
+// cost what their share of the tiles is: 1000 x 750 nodes in FP32 run at 4.95 TB/s of
+// population traffic, 1024 x 768 nodes, the same tiles filled, at 5.2.
+//
 // M planes written for step n+1: interior nodes get final values (delta psi,
 // delta rho, J, delta Theta); border nodes get the tile's raw partial sums in
 // the delta psi, delta rho and J planes, completed by the fix-up kernel.
@@ -123,7 +128,11 @@ __host__ __device__ constexpr int axis_vel(int g, int k) {
 // quasi-conserved (Sec. V, Eq. quasieq2; f*_S and f**_P of Sec. VI), whose
 // targets carry the equilibrium momenta and the current stresses of f; it needs
 // the second moments of every Q-node's populations (single-run kernel only).
-template <typename real, typename S, bool RESHAPE, int H, bool LEAN, bool STRESS = false>
+// RAGGED: the tile may be partial (tile_box). Its idle threads repeat the loads of the
+// nearest node of the tile and write nothing, so their cells of the exchange buffer
+// stay zero like the halo, and the ring moves in to the tile's last column and row.
+template <typename real, typename S, bool RESHAPE, int H, bool LEAN, bool STRESS = false,
+          bool RAGGED = false>
 __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const FusedArgs<real>& fa,
                                            int btx, int bty, int ntx, int nty,
                                            unsigned char* smem_raw) {
@@ -133,8 +142,11 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   const int nq = a.nq;
   Smem<real> sm = carve<real, H>(smem_raw, nq);
   const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * TX + lx;
-  const int x0 = btx * TX, y0 = bty * TY;
-  const int x = x0 + lx, y = y0 + ly;
+  TileBox box{btx * TX, bty * TY, TX, TY};
+  if constexpr (RAGGED) box = tile_box(a.nx, fa.trow, btx, bty, ntx);
+  const int x0 = box.x0, y0 = box.y0;
+  const bool live = !RAGGED || (lx < box.w && ly < box.h);
+  const int x = x0 + (RAGGED ? min(lx, box.w - 1) : lx), y = y0 + (RAGGED ? min(ly, box.h - 1) : ly);
   const size_t P = a.plane;
   const real* __restrict__ Min = fa.Min;
   real* __restrict__ Mout = fa.Mout;
@@ -180,6 +192,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   for (int k = tid; k < nq * RING; k += NT) sm.Ar[k] = real(0);
   for (int k = tid; k < (TX + 2) * (TY + 2); k += NT) {
     const int hx = k % (TX + 2), hy = k / (TX + 2);
+    if (RAGGED && (hx > box.w + 1 || hy > box.h + 1)) continue;
     int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
     gx = gx < 0 ? gx + a.nx : (gx >= a.nx ? gx - a.nx : gx);
     gy = gy < 0 ? gy + a.ny : (gy >= a.ny ? gy - a.ny : gy);
@@ -190,7 +203,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   }
   __syncthreads();
 
-  const int c = (ly + 1) * (TX + 2) + (lx + 1);
+  const int c = (y - y0 + 1) * (TX + 2) + (x - x0 + 1);
   const real Ux = sm.Ux[c], Uy = sm.Uy[c];
   const real G00 = real(0.5) * (sm.Ux[c + 1] - sm.Ux[c - 1]);                    // d_x U_x
   const real G01 = real(0.5) * (sm.Uy[c + 1] - sm.Uy[c - 1]);                    // d_x U_y
@@ -203,6 +216,8 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   const bool ring_thread = tid < RING;
   int rex = 0, rey = 0;
   if (ring_thread) ring_coords<H>(tid, rex, rey);
+  if (RAGGED && rex == TX) rex = box.w;   // the right column and the bottom row close up
+  if (RAGGED && rey == TY) rey = box.h;   // to a partial tile
   const int rcell = (rey + 1) * HX + (rex + 1);
 
   const real rho = a.rho0 + Min[(size_t)(nq + M_DRHO) * P + n];
@@ -290,9 +305,9 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
       const real feq_dev = real(w9(i)) * (drs + rs * (real(3) * cu + real(4.5) * cu * cu - real(1.5) * usq));
       const real srcterm = real(w9(i)) * (real(3) * (cx - Ux) + real(9) * cu * cx) * force;
       const real hp = a.om2b * hs[i] + a.tb * (a.omr * fss_dev + a.r * feq_dev) + a.omb * srcterm;
-      sdst[(size_t)i * P + n] = to_store<SS>(hp);
+      if (live) sdst[(size_t)i * P + n] = to_store<SS>(hp);
       if constexpr (i == 0) ms_arr += hp;
-      else sm.hb[(i - 1) * HSZ + hcell] = hp;
+      else if (live) sm.hb[(i - 1) * HSZ + hcell] = hp;
     });
   } else
   {
@@ -324,9 +339,9 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
                                                       real(4.5) * (a.omr * cus * cus + a.r * cu * cu) -
                                                       real(1.5) * sq));
       const real hp = a.om2b * hs[i] + a.tb * feq_dev + a.omb * real(w9(i)) * gx * force;
-      sdst[(size_t)i * P + n] = to_store<SS>(hp);
+      if (live) sdst[(size_t)i * P + n] = to_store<SS>(hp);
       if constexpr (i == 0) ms_arr += hp;
-      else sm.hb[(i - 1) * HSZ + hcell] = hp;
+      else if (live) sm.hb[(i - 1) * HSZ + hcell] = hp;
     });
   }
   __syncthreads();
@@ -345,6 +360,17 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
       acc<c9x(i)>(jx_r, v);
       acc<c9y(i)>(jy_r, v);
     });
+  }
+  // With partial tiles the polymer's momentum is summed apart from the solvent's: its
+  // 20 nq terms are 1e-4 of that and, added to it one by one, cost it half a digit
+  // (velocity error against FP64 on 1000 x 750 nodes 1.7e-6 instead of 8e-7; the two-pass
+  // kernels, which such grids took before, 1.1e-6). The four registers it takes are
+  // not there without a cost in the other instantiations.
+  constexpr bool APART = RAGGED;
+  real jx_s = 0, jy_s = 0, jx_rs = 0, jy_rs = 0;
+  if constexpr (APART) {
+    jx_s = jx_arr; jy_s = jy_arr; jx_rs = jx_r; jy_rs = jy_r;
+    jx_arr = jy_arr = jx_r = jy_r = real(0);
   }
   __syncthreads();
   // every thread has read the staged velocity (it shares A's space): clear
@@ -525,12 +551,15 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
         }
       }
       const real hp = a.om2b * h[i] + d;
-      if constexpr (std::is_same<S, real>::value) dq[(size_t)i * P] = hp;
-      else dq[(size_t)i * P] = to_store<S>(hp * a.pscale);
+      if (live) {
+        if constexpr (std::is_same<S, real>::value) dq[(size_t)i * P] = hp;
+        else dq[(size_t)i * P] = to_store<S>(hp * a.pscale);
+      }
       // an r-moving value goes through the exchange buffer (whether it bounces is
       // settled where the arrivals are summed); the others stay on this r-node
-      if constexpr (moves_r(i)) sm.hb[(i - 1) * HSZ + hcell] = hp;
-      else grp[qgroup(c25(i))] += hp;
+      if constexpr (moves_r(i)) {
+        if (live) sm.hb[(i - 1) * HSZ + hcell] = hp;
+      } else grp[qgroup(c25(i))] += hp;
       if (more) {
         long long e;
         if constexpr (i % 2 == 0) {
@@ -615,8 +644,10 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   }
 
   // ---- flush the next step's moments
-  const bool border = lx == 0 || lx == TX - 1 || ly == 0 || ly == TY - 1;
-  if (!border) {
+  const bool border = lx == 0 || lx == box.w - 1 || ly == 0 || ly == box.h - 1;
+  if (!live) {
+    // an idle thread of a partial tile
+  } else if (!border) {
     real drho = ms_arr, txx = 0, txy = 0, tyy = 0;
     for (int p = 0; p < nq; ++p) {
       const real d = sm.A[p * NT + tid] + fa.dpsi[p];
@@ -628,16 +659,16 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
       tyy += d * Fy * Qy;
     }
     Mout[(size_t)(nq + M_DRHO) * P + n] = drho;
-    Mout[(size_t)(nq + M_JX) * P + n] = jx_arr + fa.dvx;
-    Mout[(size_t)(nq + M_JY) * P + n] = jy_arr + fa.dvy;
+    Mout[(size_t)(nq + M_JX) * P + n] = jx_s + (jx_arr + fa.dvx);
+    Mout[(size_t)(nq + M_JY) * P + n] = jy_s + (jy_arr + fa.dvy);
     Mout[(size_t)(nq + M_THXX) * P + n] = a.hl2h * txx;
     Mout[(size_t)(nq + M_THXY) * P + n] = a.hl2h * txy;
     Mout[(size_t)(nq + M_THYY) * P + n] = a.hl2h * tyy;
   } else {
     for (int p = 0; p < nq; ++p) Mout[(size_t)p * P + n] = sm.A[p * NT + tid];
     Mout[(size_t)(nq + M_DRHO) * P + n] = ms_arr;
-    Mout[(size_t)(nq + M_JX) * P + n] = jx_arr;
-    Mout[(size_t)(nq + M_JY) * P + n] = jy_arr;
+    Mout[(size_t)(nq + M_JX) * P + n] = jx_s + jx_arr;
+    Mout[(size_t)(nq + M_JY) * P + n] = jy_s + jy_arr;
   }
   if (ring_thread) {
     const size_t ntiles = (size_t)ntx * nty;
@@ -645,17 +676,17 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
     real* ex = fa.exports;
     for (int p = 0; p < nq; ++p) ex[((size_t)p * ntiles + tile) * RING + tid] = sm.Ar[p * RING + tid];
     ex[((size_t)(nq + 0) * ntiles + tile) * RING + tid] = ms_r;
-    ex[((size_t)(nq + 1) * ntiles + tile) * RING + tid] = jx_r;
-    ex[((size_t)(nq + 2) * ntiles + tile) * RING + tid] = jy_r;
+    ex[((size_t)(nq + 1) * ntiles + tile) * RING + tid] = jx_rs + jx_r;
+    ex[((size_t)(nq + 2) * ntiles + tile) * RING + tid] = jy_rs + jy_r;
   }
 }
 
-template <typename real, typename S, bool RESHAPE, bool STRESS = false>
+template <typename real, typename S, bool RESHAPE, bool STRESS = false, bool RAGGED = false>
 __global__ void __launch_bounds__(Geo<TY>::NT, 2)
 step_fused_kernel(KernelArgs<real> a, FusedArgs<real> fa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fused_body<real, S, RESHAPE, TY, false, STRESS>(a, fa, blockIdx.x, blockIdx.y, gridDim.x,
-                                                  gridDim.y, smem_raw);
+  fused_body<real, S, RESHAPE, TY, false, STRESS, RAGGED>(a, fa, blockIdx.x, blockIdx.y, gridDim.x,
+                                                          gridDim.y, smem_raw);
 }
 
 
@@ -677,14 +708,22 @@ constexpr int fix_nodes() { return 2 * TX + 2 * (H - 2); }
 template <typename real, int H>
 size_t fix_smem_bytes(int nq) { return (size_t)(nq + 1) * fix_nodes<H>() * sizeof(real); }
 
-template <typename real, int H>
+template <typename real, int H, bool RAGGED = false>
 __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const FusedArgs<real>& fa,
                                            int tx, int ty, int ntx, int nty, real* s_d) {
   constexpr int TY = H, RING = Geo<H>::RING;
-  constexpr int NB = fix_nodes<H>();
-  __shared__ uint32_t s_n[NB];        // node offset within a plane
-  __shared__ uint32_t s_nc[NB];       // contributing neighbour tiles (1 to 3)
-  __shared__ size_t s_e[3][NB];       // their export positions (tile * RING + ring position)
+  constexpr int MAXNB = fix_nodes<H>();
+  // contributing neighbour tiles of a node: 1 to 3, and up to 8 where a partial tile
+  // is one node wide or high
+  constexpr int MAXC = RAGGED ? 8 : 3;
+  __shared__ uint32_t s_n[MAXNB];     // node offset within a plane
+  __shared__ uint32_t s_nc[MAXNB];    // contributing neighbour tiles
+  __shared__ size_t s_e[MAXC][MAXNB]; // their export positions (tile * RING + ring position)
+  TileBox box{tx * TX, ty * TY, TX, TY};
+  if constexpr (RAGGED) box = tile_box(a.nx, fa.trow, tx, ty, ntx);
+  const int W = box.w, h = box.h;
+  const int top = h > 1 ? 2 * W : W;  // nodes of the first and the last row
+  const int NB = RAGGED ? top + (h > 2 ? (W > 1 ? 2 : 1) * (h - 2) : 0) : MAXNB;
   const int tid = threadIdx.x;
   const size_t ntiles = (size_t)ntx * nty;
   const int nq = a.nq;
@@ -692,27 +731,28 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
   if (tid < NB) {
     const int k = tid;
     int lx, ly;
-    if (k < TX) { lx = k; ly = 0; }
-    else if (k < 2 * TX) { lx = k - TX; ly = TY - 1; }
-    else if (k < 2 * TX + TY - 2) { lx = 0; ly = 1 + (k - 2 * TX); }
-    else { lx = TX - 1; ly = 1 + (k - 2 * TX - (TY - 2)); }
-    s_n[k] = (uint32_t)((size_t)(ty * TY + ly) * a.pitch + (tx * TX + lx));
-    int ctile[3] = {0, 0, 0}, cpos[3] = {0, 0, 0}, nc = 0;
+    if (k < W) { lx = k; ly = 0; }
+    else if (k < top) { lx = k - W; ly = h - 1; }
+    else if (k < top + h - 2) { lx = 0; ly = 1 + (k - top); }
+    else { lx = W - 1; ly = 1 + (k - top - (h - 2)); }
+    s_n[k] = (uint32_t)((size_t)(box.y0 + ly) * a.pitch + (box.x0 + lx));
+    int ctile[MAXC] = {}, cpos[MAXC] = {}, nc = 0;
     auto tile_of = [&](int dx, int dy) {
       const int ax = (tx + dx + ntx) % ntx, ay = (ty + dy + nty) % nty;
       return ay * ntx + ax;
     };
+    // (the ring's right column is at TX and its bottom row at TY whatever the tile's size)
     if (lx == 0) { ctile[nc] = tile_of(-1, 0); cpos[nc++] = ring_pos<H>(TX, ly); }
-    if (lx == TX - 1) { ctile[nc] = tile_of(1, 0); cpos[nc++] = ring_pos<H>(-1, ly); }
+    if (lx == W - 1) { ctile[nc] = tile_of(1, 0); cpos[nc++] = ring_pos<H>(-1, ly); }
     if (ly == 0) { ctile[nc] = tile_of(0, -1); cpos[nc++] = ring_pos<H>(lx, TY); }
-    if (ly == TY - 1) { ctile[nc] = tile_of(0, 1); cpos[nc++] = ring_pos<H>(lx, -1); }
+    if (ly == h - 1) { ctile[nc] = tile_of(0, 1); cpos[nc++] = ring_pos<H>(lx, -1); }
     if (lx == 0 && ly == 0) { ctile[nc] = tile_of(-1, -1); cpos[nc++] = ring_pos<H>(TX, TY); }
-    if (lx == TX - 1 && ly == 0) { ctile[nc] = tile_of(1, -1); cpos[nc++] = ring_pos<H>(-1, TY); }
-    if (lx == 0 && ly == TY - 1) { ctile[nc] = tile_of(-1, 1); cpos[nc++] = ring_pos<H>(TX, -1); }
-    if (lx == TX - 1 && ly == TY - 1) { ctile[nc] = tile_of(1, 1); cpos[nc++] = ring_pos<H>(-1, -1); }
+    if (lx == W - 1 && ly == 0) { ctile[nc] = tile_of(1, -1); cpos[nc++] = ring_pos<H>(-1, TY); }
+    if (lx == 0 && ly == h - 1) { ctile[nc] = tile_of(-1, 1); cpos[nc++] = ring_pos<H>(TX, -1); }
+    if (lx == W - 1 && ly == h - 1) { ctile[nc] = tile_of(1, 1); cpos[nc++] = ring_pos<H>(-1, -1); }
     s_nc[k] = nc;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) s_e[c][k] = (size_t)ctile[c] * RING + cpos[c];
+    for (int c = 0; c < MAXC; ++c) s_e[c][k] = (size_t)ctile[c] * RING + cpos[c];
   }
   __syncthreads();
   real* M = fa.Mout;
@@ -731,7 +771,7 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
         real w = M[(size_t)j * P + s_n[k]];
         const uint32_t nc = s_nc[k];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < MAXC; ++c)
           if (c < (int)nc) w += ex[(size_t)j * estride + s_e[c][k]];
         v[u] = w;
       }
@@ -772,10 +812,10 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
   }
 }
 
-template <typename real>
+template <typename real, bool RAGGED = false>
 __global__ void __launch_bounds__(FIX_T) fixup_kernel(KernelArgs<real> a, FusedArgs<real> fa) {
   extern __shared__ __align__(16) unsigned char fix_raw[];
-  fixup_body<real, TY>(a, fa, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y, (real*)fix_raw);
+  fixup_body<real, TY, RAGGED>(a, fa, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y, (real*)fix_raw);
 }
 
 // ---------------------------------------------------------------- batches
@@ -857,15 +897,21 @@ size_t fused_smem_bytes(int nq, size_t real_bytes, int ty) {
   }
 }
 
-size_t fused_export_elems(int nx, int ny, int nq, int ty) {
-  const size_t ring = 2 * (TX + 2) + 2 * (size_t)ty;
-  return (size_t)(nx / TX) * (ny / ty) * ring * (size_t)(nq + 3);
+static bool whole_tiles(const Lattice& L) { return L.nx % TX == 0 && L.ny % TY == 0; }
+
+static size_t export_elems(size_t tiles, int nq, int ty) {
+  return tiles * (2 * (TX + 2) + 2 * (size_t)ty) * (size_t)(nq + 3);
 }
 
-size_t fused_export_capacity(int nx, int ny, int nq) {
+size_t fused_export_capacity(const Lattice& L) {
+  const size_t ntx = (L.nx + TX - 1) / TX;
   size_t m = 0;
-  for (int ty : {4, 8, 16})
-    if (ny % ty == 0) m = std::max(m, fused_export_elems(nx, ny, nq, ty));
+  if (L.precision == TFKT_FP64 || whole_tiles(L)) {
+    for (int ty : {4, 8, 16})
+      if (L.ny % ty == 0) m = std::max(m, export_elems(ntx * (L.ny / ty), L.nq, ty));
+  }
+  if (L.precision != TFKT_FP64 && (!whole_tiles(L) || L.ny_global > 0))
+    m = std::max(m, export_elems(ntx * max_tile_rows(L), L.nq, TY));
   return m;
 }
 
@@ -874,50 +920,90 @@ bool fused_supported(int nx, int ny, int nq, size_t real_bytes, int ty) {
          fused_smem_bytes(nq, real_bytes, ty) <= 227 * 1024;
 }
 
+// Tiles of the whole run that a context belongs to.
+size_t run_tiles(const Lattice& L) {
+  const size_t ny = L.ny_global > 0 ? L.ny_global : L.ny;
+  return (size_t)((L.nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
+}
+
+// Grids of whole tiles, and in FP32 and FP16 storage any grid that does not take the
+// Q-split kernels: with partial tiles the fused kernel and its fix-up take 979 us per
+// step on 1000 x 750 nodes with 32 Q-nodes in FP32 (1026 in FP16 storage, 993 on 999 x 751
+// with the stress quasi-equilibrium), the Q-split kernels, which read the populations
+// twice, 1426 (1193, 1437); with 9 Q-nodes on 333 x 777 nodes 134 against 174.
 bool fused_path(const Lattice& L) {
-  return fused_supported(L.nx, L.ny, L.nq, L.precision == TFKT_FP64 ? 8 : 4);
+  if (fused_smem_bytes(L.nq, L.precision == TFKT_FP64 ? 8 : 4) > 227 * 1024) return false;
+  return whole_tiles(L) || (L.precision != TFKT_FP64 && !split_path(L));
+}
+
+// First row and height of every tile row, or none where they are the whole tiles that
+// the ordinary kernel assumes. Tile rows start at the whole run's multiples of TY and
+// end at its last row, also in a slab whose rows start elsewhere, so that a node
+// sums its arrivals in the same order in every decomposition.
+std::vector<int2> tile_rows(const Lattice& L) {
+  const int nyg = L.ny_global > 0 ? L.ny_global : L.ny;
+  std::vector<int2> rows;
+  if (L.precision == TFKT_FP64 || (whole_tiles(L) && nyg % TY == 0 && L.y_origin % TY == 0)) return rows;
+  for (int y = 0; y < L.ny; ++y) {
+    const int yg = ((L.y_origin + y) % nyg + nyg) % nyg;
+    if (y == 0 || yg % TY == 0) rows.push_back(make_int2(y, 0));
+    ++rows.back().y;
+  }
+  return rows;
+}
+
+// At most so many tile rows, wherever a slab of this height starts.
+size_t max_tile_rows(const Lattice& L) {
+  const int nyg = L.ny_global > 0 ? L.ny_global : L.ny;
+  return (size_t)(L.ny / TY + 2) + (nyg % TY ? 2 * (size_t)(L.ny / nyg + 1) : 0);
+}
+
+template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED>
+static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+  const size_t smem = fused_smem_bytes(a.nq, sizeof(real), TY);
+  cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
+  step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED><<<grid, dim3(TX, TY), smem, s>>>(a, f);
+  return cudaGetLastError();
 }
 
 template <typename real, typename S>
 cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
-  const size_t smem = fused_smem_bytes(a.nq, sizeof(real), TY);
-  const dim3 grid(a.nx / TX, a.ny / TY), block(TX, TY);
   if (f.rshp) {
-    // a learned block's increment rides on this step's pull (FP32 storage only)
+    // a learned block's increment rides on this step's pull (FP32 storage, whole tiles)
     if constexpr (std::is_same<real, float>::value && std::is_same<S, float>::value) {
-      cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<real, S, true>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      step_fused_kernel<real, S, true><<<grid, block, smem, s>>>(a, f);
-      return cudaGetLastError();
+      if (f.ntrow) return cudaErrorInvalidValue;
+      return launch_fused<real, S, true, false, false>(a, f, s);
     } else {
       return cudaErrorInvalidValue;
     }
   }
-  if (a.qe == TFKT_QE_STRESS) {
-    cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<real, S, false, true>,
+  const bool stress = a.qe == TFKT_QE_STRESS;
+  if (f.ntrow)
+    return stress ? launch_fused<real, S, false, true, true>(a, f, s)
+                  : launch_fused<real, S, false, false, true>(a, f, s);
+  return stress ? launch_fused<real, S, false, true, false>(a, f, s)
+                : launch_fused<real, S, false, false, false>(a, f, s);
+}
+
+template <typename real, bool RAGGED>
+static cudaError_t launch_fix(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+  const size_t smem = fix_smem_bytes<real, TY>(a.nq);
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(fixup_kernel<real, RAGGED>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    step_fused_kernel<real, S, false, true><<<grid, block, smem, s>>>(a, f);
-    return cudaGetLastError();
   }
-  cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<real, S, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  step_fused_kernel<real, S, false><<<grid, block, smem, s>>>(a, f);
+  const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
+  fixup_kernel<real, RAGGED><<<grid, FIX_T, smem, s>>>(a, f);
   return cudaGetLastError();
 }
 
 template <typename real>
 cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
-  const size_t smem = fix_smem_bytes<real, TY>(a.nq);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fixup_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  fixup_kernel<real><<<dim3(a.nx / TX, a.ny / TY), FIX_T, smem, s>>>(a, f);
-  return cudaGetLastError();
+  return f.ntrow ? launch_fix<real, true>(a, f, s) : launch_fix<real, false>(a, f, s);
 }
 
 // Batches that launch each run's own single-run kernels (graph branches): the
@@ -1026,14 +1112,10 @@ void fused_tables(const Lattice& L, const HostTables& t, std::vector<int>& tgt,
     }
 }
 
-template cudaError_t launch_step_fused<double, double>(const KernelArgs<double>&,
-                                                        const FusedArgs<double>&, cudaStream_t);
 template cudaError_t launch_step_fused<float, float>(const KernelArgs<float>&,
                                                       const FusedArgs<float>&, cudaStream_t);
 template cudaError_t launch_step_fused<float, __half>(const KernelArgs<float>&,
                                                        const FusedArgs<float>&, cudaStream_t);
-template cudaError_t launch_fixup<double>(const KernelArgs<double>&, const FusedArgs<double>&,
-                                          cudaStream_t);
 template cudaError_t launch_fixup<float>(const KernelArgs<float>&, const FusedArgs<float>&,
                                          cudaStream_t);
 

@@ -34,6 +34,16 @@ struct Geo {
   static constexpr int MINB = NT >= 512 ? 1 : 512 / NT;   // blocks per SM at 128 registers
 };
 
+// A tile of a grid whose last tile column, and in y any tile row, may be partial: its
+// first node, width and height. The tile rows come from a table, so that a slab has
+// the tile rows of its whole run.
+struct TileBox {
+  int x0, y0, w, h;
+};
+__device__ __forceinline__ TileBox tile_box(int nx, const int2* trow, int tx, int ty, int ntx) {
+  return {tx * TX, trow[ty].x, tx == ntx - 1 ? nx - tx * TX : TX, trow[ty].y};
+}
+
 // Ring position of frame coordinates (ex, ey) in [-1, TX] x [-1, H] \ tile.
 template <int H>
 __host__ __device__ constexpr int ring_pos(int ex, int ey) {

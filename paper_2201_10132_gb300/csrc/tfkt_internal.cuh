@@ -200,6 +200,8 @@ struct FusedArgs {
   const int* tgt;       // [nq][9] target Q-node per Q-displacement group, -1: bounce-back
   const real* dpsi;     // [nq] sum over i of the pull shift differences of Q-node q
   const long long* poff;  // [nq*25] element offset of each pull's source plane
+  const int2* trow;     // [ntrow] first row and height of every tile row
+  int ntrow;            // 0: whole tiles throughout
   real dvx, dvy;        // r-momentum of all pull shift differences
   // Pending increment of a learned block (or null): per node the coefficients
   // B0..B3 (4 planes) of dpsi(q) = p0(q) (B0 Qx^2 + B1 Qx Qy + B2 Qy^2 + B3), added to
@@ -244,7 +246,8 @@ struct Ctx {
   bool poisoned = false;
   int64_t step = 0;
   int diag_blocks = 0;
-  bool fused = false;     // grid fits the fused single-pass kernel (double-buffered moments)
+  bool fused = false;     // the fused path (double-buffered moment planes)
+  int ntrow = 0;          // tile rows of a fused-path context with partial tiles
   bool split = false;     // a fused-path context that steps with the Q-split kernels
   int mcur = 0;           // moment buffer (0: off_M, 1: off_M2) of the current state
   double dvx = 0, dvy = 0;  // r-momentum of all pull shift differences (fused path)
@@ -305,10 +308,13 @@ cudaError_t launch_diag(const KernelArgs<real>& a, double* partials, int nblocks
 
 // Fused single-pass step (tfkt_fused.cu).
 size_t fused_smem_bytes(int nq, size_t real_bytes, int ty = TY);
-size_t fused_export_elems(int nx, int ny, int nq, int ty = TY);
-// ring-export elements enough for every tile height the grid allows (4, 8, 16)
-size_t fused_export_capacity(int nx, int ny, int nq);
+// ring-export elements of a context, enough for every tile height a batch may choose
+// (4, 8, 16)
+size_t fused_export_capacity(const Lattice& L);
 bool fused_supported(int nx, int ny, int nq, size_t real_bytes, int ty = TY);
+size_t run_tiles(const Lattice& L);
+std::vector<int2> tile_rows(const Lattice& L);
+size_t max_tile_rows(const Lattice& L);
 void fused_tables(const Lattice& L, const HostTables& t, std::vector<int>& tgt,
                   std::vector<double>& dpsi, double& dvx, double& dvy,
                   std::vector<long long>& poff);
@@ -316,10 +322,11 @@ template <typename real, typename S>
 cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s);
 template <typename real>
 cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s);
-// Whether a context of this lattice takes the fused path (tile multiples and the
-// kernel's shared memory; either quasi-equilibrium).
+// Whether a context of this lattice takes the fused path, with double-buffered moment
+// planes (either quasi-equilibrium).
 bool fused_path(const Lattice& L);
-// Whether a fused-path context steps with the Q-split kernels instead (tfkt_api.cu).
+// Whether the run steps with the Q-split kernels where it could take the fused kernel
+// (tfkt_api.cu).
 bool split_path(const Lattice& L);
 
 // Each run's single-run FP32 kernels (fused step + fix-up) without API calls

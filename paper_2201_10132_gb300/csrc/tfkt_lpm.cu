@@ -592,7 +592,8 @@ tfkt_status lpm_err(cudaError_t e, const char* what) {
 tfkt_status check(Ctx* c, int K) {
   const Lattice& L = c->L;
   if (L.precision != TFKT_FP32) return fail(TFKT_EINVAL, "the learned block needs an FP32 context");
-  if (!c->fused) return fail(TFKT_EINVAL, "the learned block needs nx % 32 == 0 and ny % 8 == 0");
+  if (!c->fused || L.nx % TX || L.ny % TY)
+    return fail(TFKT_EINVAL, "the learned block needs nx % 32 == 0 and ny % 8 == 0");
   if (!(L.psi_tot > 0)) return fail(TFKT_EINVAL, "the learned block needs a polymer (beta < 1)");
   if (L.fene_b != 0) return fail(TFKT_EINVAL, "the learned block is for Hookean springs");
   if (L.qe_model != TFKT_QE_MOMENTUM)

@@ -1,7 +1,8 @@
 """Kernel paths of the step at the sizes where they can go wrong, against the oracle:
 the Q-split kernels (small grids, ragged grids, FP64) at node counts around a group
 of 32 nodes, Q-node counts around the warps of a block and grids on both sides of
-the line to the fused kernel, and the fused kernel just above that line.
+the line to the fused kernel, and the fused kernel just above that line and with
+partial tiles, also split into slabs.
 Tolerances are those of tests/test_gpu_parity.py: FP64 1e-12, FP32 2e-5, FP16
 storage 3e-3 of the field's scale."""
 import numpy as np
@@ -67,6 +68,49 @@ def test_q_split_sizes(T, oracle_mod, nx, ny, S, R, prec):
 @pytest.mark.parametrize("nx,ny", [(160, 160), (416, 64)])   # 100 and 104 tiles of 32 x 8
 def test_both_sides_of_the_tile_line(T, oracle_mod, nx, ny, prec, stress, fene):
     _check(T, oracle_mod, _params(T, nx, ny, 6, 3.0, prec, stress, fene), 4, prec)
+
+
+# Partial tiles of the fused kernel (more than 100 tiles): last tiles of 1, 3, 31 and 30 by 1, 7
+# and 2 nodes, and grids of one tile column or row, whose tile is its own neighbour.
+PARTIAL = [(33, 409), (99, 207), (415, 63), (1, 801), (3330, 5), (62, 402)]
+
+
+# (the stress model refuses this momentum relaxation time on five rows)
+@pytest.mark.parametrize("nx,ny,prec,stress,fene", [
+    c + k for c in PARTIAL for k in (("FP32", False, 0.0), ("FP16", False, 0.0), ("FP32", True, 0.0),
+                                     ("FP16", True, 3.1)) if not (k[1] and c[1] == 5)])
+def test_fused_partial_tiles(T, oracle_mod, nx, ny, prec, stress, fene):
+    p = _params(T, nx, ny, 4, 1.6, prec, stress, fene)
+    with T.Solver(p) as s:
+        k, ms = np.zeros(len(T.KERNELS), np.int64), np.zeros(len(T.KERNELS))
+        s.step_profiled(1, ms, k)
+    assert k[T.KERNELS.index("fused")] == 1     # the fused kernel ran
+    _check(T, oracle_mod, p, 3, prec)
+
+
+@pytest.mark.parametrize("nx,ny,parts,prec", [(415, 70, 3, "FP32"), (415, 70, 2, "FP16"),
+                                              (416, 65, 4, "FP32"), (33, 420, 5, "FP32")])
+def test_slabs_of_partial_tiles_are_bit_identical(T, nx, ny, parts, prec):
+    """Slabs keep the whole run's tile rows wherever they start."""
+    import torch
+    from paper_2201_10132_gb300 import slabs as S
+    from paper_2201_10132_gb300.inputs import perturbation
+    p = _params(T, nx, ny, 4, 1.6, prec)
+    pert = perturbation(nx, ny, 9, 0.05, 0.05)
+    with T.Solver(p, pert) as s:
+        s.step(9)
+        ref = s.populations()
+    slabs = [T.Slab(p, y0, n, S.local_perturbation(pert, y0, n)) for y0, n in S.partition(ny, parts)]
+    bufs = [[torch.empty(s.halo_bytes(), dtype=torch.uint8, device="cuda") for _ in (0, 1)] for s in slabs]
+    S.exchange_local(slabs, bufs)
+    for _ in range(9):
+        for s in slabs:
+            s.step(1)
+        S.exchange_local(slabs, bufs)
+    got = np.concatenate([s.owned(s.populations()) for s in slabs], axis=1)
+    for s in slabs:
+        s.close()
+    assert np.array_equal(got, ref)
 
 
 @pytest.mark.parametrize("nx,ny,prec", [(64, 32, "FP32"), (40, 24, "FP32"), (416, 64, "FP16")])
