@@ -11,6 +11,8 @@
 // Moment planes M: delta psi(q) (q < nq), then delta rho (total), J_x, J_y
 // (total momentum of g), and delta Theta_xx, xy, yy = (H ell^2 / 2) sum_q
 // delta psi phi_q Q Q, all of the pulled (pre-collision) state.
+#include <type_traits>
+
 #include "tfkt_internal.cuh"
 
 namespace tfkt {
@@ -161,79 +163,236 @@ __global__ void __launch_bounds__(256) velocity_kernel(KernelArgs<real> a) {
   a.U[a.plane + n] = uy;
 }
 
-// Per-node observables (Sec. VII): rho_S, psi_tot, U, C, Theta, Q_rms, vorticity,
-// the ones in `mask` (others are left unset). The sums over the Q-nodes run in
-// FP64 (the second moments behind C_xy and Theta_xy cancel between Q-nodes of
-// opposite sign, which FP32 sums would resolve only to ~1e-7 of the diagonal
-// ones) and only as far as the requested fields need them.
+// Per-node observables (Sec. VII): rho_S, psi_tot, U, C, Theta, Q_rms, vorticity, the
+// ones in `mask`. The sums over the Q-nodes need more than FP32: the second moments
+// behind C_xy and Theta_xy cancel between Q-nodes of opposite sign, which FP32 sums
+// would resolve only to ~1e-7 of the diagonal ones. FP64 contexts sum in FP64.
+// FP32 contexts sum in pairs of floats without any FP64 operation: each term's
+// product and each sum keep their rounding error (Dekker 1971; Dot2 of Ogita, Rump
+// and Oishi 2005), so a sum is as if formed in 48 bits, far below the rounding of the
+// planes themselves; quotient, root and differences follow in such pairs, and a node
+// with a non-finite or overflowing value is formed again in FP64. FP64 arithmetic, 2
+// lanes per clock and SM, bound the kernel: rho_s, U and C of 1024 x 1024 nodes with 32
+// Q-nodes took 767 us (the velocity pass included), now 161; with 9 Q-nodes 284 and 75.
+// What is left is the FP32 issue rate, about 50 instructions per Q-node.
 constexpr uint32_t FIELDS_PSUM = (1u << TFKT_F_RHO_S) | (1u << TFKT_F_PSI_TOT) | (1u << TFKT_F_CXX) |
                                  (1u << TFKT_F_CXY) | (1u << TFKT_F_CYY) | (1u << TFKT_F_QRMS);
 constexpr uint32_t FIELDS_CONF = (1u << TFKT_F_CXX) | (1u << TFKT_F_CXY) | (1u << TFKT_F_CYY) |
                                  (1u << TFKT_F_QRMS);
 constexpr uint32_t FIELDS_STRESS = (1u << TFKT_F_THXX) | (1u << TFKT_F_THXY) | (1u << TFKT_F_THYY);
 
-template <typename real>
-__device__ void node_fields(const KernelArgs<real>& a, int x, int y, uint32_t mask,
-                            double f[TFKT_NFIELDS]) {
+// A sum kept as a pair of floats: add (p + pl) (w + wl), p and w the leading parts.
+struct PairSum {
+  float hi = 0, lo = 0;
+  __device__ __forceinline__ void add(float p, float pl, float w, float wl) {
+    const float x = __fmul_rn(p, w);
+    const float e = __fmaf_rn(p, w, -x);
+    const float s = __fadd_rn(hi, x);
+    const float b = __fsub_rn(s, hi);
+    const float r = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
+    hi = s;
+    lo = __fadd_rn(lo, __fmaf_rn(pl, w, __fmaf_rn(p, wl, __fadd_rn(e, r))));
+  }
+};
+
+// Arithmetic on such pairs (about 46 bits), as far as the fields need it.
+struct Two {
+  float h, l;
+  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+__device__ __forceinline__ Two two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Two two_add(Two a, Two b) {
+  const Two s = two_sum(a.h, b.h);
+  return two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Two two_scale(Two a, float f) {
+  const float p = __fmul_rn(a.h, f);
+  return {p, __fmaf_rn(a.l, f, __fmaf_rn(a.h, f, -p))};
+}
+__device__ __forceinline__ Two two_div(Two a, Two b) {
+  const float q = a.h / b.h;
+  const float r = __fmaf_rn(-q, b.l, __fadd_rn(__fmaf_rn(-q, b.h, a.h), a.l));
+  return {q, r / b.h};
+}
+__device__ __forceinline__ Two two_sqrt(Two a) {   // a.h > 0
+  const float q = sqrtf(a.h);
+  return {q, __fadd_rn(__fmaf_rn(-q, q, a.h), a.l) / __fadd_rn(q, q)};
+}
+
+// Weights of a Q-node in the pair sums, staged once per block: Q Q and F Q (xx, xy,
+// yy) and what their rounding leaves.
+struct FieldRow {
+  float psi0, w[6], wl[6];
+};
+
+__device__ __forceinline__ void stage_field_rows(const KernelArgs<float>& a, FieldRow* row) {
+  for (int q = threadIdx.y * TX + threadIdx.x; q < a.nq; q += TX * TY) {
+    const float Q[2] = {a.tab.qx[q], a.tab.qy[q]}, F[2] = {a.tab.fx[q], a.tab.fy[q]};
+    FieldRow& r = row[q];
+    r.psi0 = a.tab.psi0[q];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {   // xx, xy, yy
+      const float q1 = Q[j / 2], f1 = F[j / 2], q2 = Q[(j + 1) / 2];
+      r.w[j] = __fmul_rn(q1, q2);
+      r.wl[j] = __fmaf_rn(q1, q2, -r.w[j]);
+      r.w[3 + j] = __fmul_rn(f1, q2);
+      r.wl[3 + j] = __fmaf_rn(f1, q2, -r.w[3 + j]);
+    }
+  }
+}
+
+// s: psi_tot, then sum psi Q Q and sum psi F Q (xx, xy, yy), the latter two where asked.
+template <bool CONF, bool STRESS>
+__device__ __forceinline__ void pair_sums(const KernelArgs<float>& a, const FieldRow* row, size_t n,
+                                          PairSum (&s)[7]) {
   const size_t P = a.plane;
-  const size_t n = (size_t)y * a.pitch + x;
-  const int nq = a.nq;
-  double pt = 0, sxx = 0, sxy = 0, syy = 0, fxx = 0, fxy = 0, fyy = 0;
-  if (mask & (FIELDS_PSUM | FIELDS_STRESS)) {
-    const bool conf = mask & FIELDS_CONF, stress = mask & FIELDS_STRESS;
-    for (int q = 0; q < nq; ++q) {
-      const double p = double(a.tab.psi0[q]) + double(a.M[(size_t)q * P + n]);
-      const double Qx = a.tab.qx[q], Qy = a.tab.qy[q];
-      pt += p;
-      if (conf) {
-        sxx += p * Qx * Qx;
-        sxy += p * Qx * Qy;
-        syy += p * Qy * Qy;
-      }
-      if (stress) {
-        const double Fx = a.tab.fx[q], Fy = a.tab.fy[q];
-        fxx += p * Fx * Qx;
-        fxy += p * Fx * Qy;
-        fyy += p * Fy * Qy;
+  const float* mp = a.M + n;
+  // the planes four at a time, so that several loads are in flight
+  for (int q0 = 0; q0 < a.nq; q0 += 4) {
+    float m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = mp[(size_t)(q0 + k < a.nq ? q0 + k : q0) * P];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (q0 + k >= a.nq) break;
+      const FieldRow& r = row[q0 + k];
+      const float p = __fadd_rn(r.psi0, m[k]);
+      const float b = __fsub_rn(p, r.psi0);
+      const float pl = __fadd_rn(__fsub_rn(r.psi0, __fsub_rn(p, b)), __fsub_rn(m[k], b));
+      s[0].add(p, pl, 1.0f, 0.0f);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        if (CONF) s[1 + j].add(p, pl, r.w[j], r.wl[j]);
+        if (STRESS) s[4 + j].add(p, pl, r.w[3 + j], r.wl[3 + j]);
       }
     }
   }
-  const double ptd = pt;
-  const double rho = double(a.rho0) + double(a.M[(size_t)(nq + M_DRHO) * P + n]);
-  const double l2 = a.l2, hh = 0.5 * double(a.H) * l2;
-  f[TFKT_F_RHO_S] = rho - ptd;
-  f[TFKT_F_PSI_TOT] = ptd;
-  f[TFKT_F_UX] = a.U[n];
-  f[TFKT_F_UY] = a.U[P + n];
-  const double cxx = ptd != 0 ? l2 * double(sxx) / ptd : 0, cxy = ptd != 0 ? l2 * double(sxy) / ptd : 0,
-               cyy = ptd != 0 ? l2 * double(syy) / ptd : 0;
-  f[TFKT_F_CXX] = cxx;
-  f[TFKT_F_CXY] = cxy;
-  f[TFKT_F_CYY] = cyy;
-  f[TFKT_F_THXX] = hh * double(fxx);
-  f[TFKT_F_THXY] = hh * double(fxy);
-  f[TFKT_F_THYY] = hh * double(fyy);
-  f[TFKT_F_QRMS] = sqrt(cxx + cyy);
-  if (mask & (1u << TFKT_F_VORT)) {
-    const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
-    const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y == a.ny - 1 ? 0 : y + 1;
-    const double duy_dx = 0.5 * (double(a.U[P + (size_t)y * a.pitch + xp]) -
-                                 double(a.U[P + (size_t)y * a.pitch + xm]));
-    const double dux_dy =
-        0.5 * (double(a.U[(size_t)yp * a.pitch + x]) - double(a.U[(size_t)ym * a.pitch + x]));
-    f[TFKT_F_VORT] = duy_dx - dux_dy;
+}
+
+template <typename real>
+__device__ __forceinline__ void fp64_sums(const KernelArgs<real>& a, size_t n, bool conf, bool stress,
+                                       double (&s)[7]) {
+  for (int j = 0; j < 7; ++j) s[j] = 0;
+  for (int q = 0; q < a.nq; ++q) {
+    const double p = double(a.tab.psi0[q]) + double(a.M[(size_t)q * a.plane + n]);
+    const double Qx = a.tab.qx[q], Qy = a.tab.qy[q];
+    s[0] += p;
+    if (conf) {
+      s[1] += p * Qx * Qx;
+      s[2] += p * Qx * Qy;
+      s[3] += p * Qy * Qy;
+    }
+    if (stress) {
+      const double Fx = a.tab.fx[q], Fy = a.tab.fy[q];
+      s[4] += p * Fx * Qx;
+      s[5] += p * Fx * Qy;
+      s[6] += p * Fy * Qy;
+    }
   }
 }
 
 template <typename real>
 __global__ void __launch_bounds__(256) fields_kernel(KernelArgs<real> a, uint32_t mask,
                                                      double* out) {
+  extern __shared__ __align__(16) unsigned char field_smem[];
+  const bool sums = mask & (FIELDS_PSUM | FIELDS_STRESS);
+  const bool conf = mask & FIELDS_CONF, stress = mask & FIELDS_STRESS;
+  const int nq = a.nq;
+  if constexpr (std::is_same<real, float>::value)
+    if (sums) {
+      stage_field_rows(a, reinterpret_cast<FieldRow*>(field_smem));
+      __syncthreads();
+    }
   const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
   if (x >= a.nx || y >= a.ny) return;
-  double f[TFKT_NFIELDS];
-  node_fields(a, x, y, mask, f);
+  const size_t P = a.plane, n = (size_t)y * a.pitch + x;
   const size_t N = (size_t)a.nx * a.ny, k = (size_t)y * a.nx + x;
+  double f[TFKT_NFIELDS];
+  f[TFKT_F_UX] = a.U[n];
+  f[TFKT_F_UY] = a.U[P + n];
+  const real drho = a.M[(size_t)(nq + M_DRHO) * P + n];
+  const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
+  const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y == a.ny - 1 ? 0 : y + 1;
+  const bool vort = mask & (1u << TFKT_F_VORT);
+  bool done = false;
+  if constexpr (std::is_same<real, float>::value) {
+    // FP32 contexts: pairs of floats to the end, one FP64 addition per field
+    const FieldRow* row = reinterpret_cast<const FieldRow*>(field_smem);
+    PairSum ps[7];
+    if (conf && stress) pair_sums<true, true>(a, row, n, ps);
+    else if (conf) pair_sums<true, false>(a, row, n, ps);
+    else if (stress) pair_sums<false, true>(a, row, n, ps);
+    else if (sums) pair_sums<false, false>(a, row, n, ps);
+    Two s[7];
+    done = true;   // unless a sum left the range of FP32 or met a non-finite value
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+      s[j] = two_sum(ps[j].hi, ps[j].lo);
+      done = done && isfinite(ps[j].hi);
+    }
+    if (sums) {
+      f[TFKT_F_PSI_TOT] = s[0].value();
+      f[TFKT_F_RHO_S] = two_add(two_sum(a.rho0, drho), {-s[0].h, -s[0].l}).value();
+    }
+    if (conf) {
+      Two c[3] = {};
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (s[0].h != 0.0f) c[j] = two_div(two_scale(s[1 + j], a.l2), s[0]);
+      f[TFKT_F_CXX] = c[0].value();
+      f[TFKT_F_CXY] = c[1].value();
+      f[TFKT_F_CYY] = c[2].value();
+      if (mask & (1u << TFKT_F_QRMS)) {
+        const Two t = two_add(c[0], c[2]);
+        f[TFKT_F_QRMS] = t.h > 0.0f ? two_sqrt(t).value() : sqrt(t.value());
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j) done = done && isfinite(c[j].h);
+    }
+    if (stress) {
+      const double hh = 0.5 * double(a.H) * double(a.l2);
+      f[TFKT_F_THXX] = hh * s[4].value();
+      f[TFKT_F_THXY] = hh * s[5].value();
+      f[TFKT_F_THYY] = hh * s[6].value();
+    }
+    if (vort) {
+      const Two d1 = two_sum(a.U[P + (size_t)y * a.pitch + xp], -a.U[P + (size_t)y * a.pitch + xm]);
+      const Two d2 = two_sum(a.U[(size_t)ym * a.pitch + x], -a.U[(size_t)yp * a.pitch + x]);
+      const Two w = two_add(d1, d2);
+      f[TFKT_F_VORT] = 0.5 * w.value();
+      done = done && isfinite(w.h);
+    }
+  }
+  if (!done) {
+    double s[7] = {};
+    if (sums) fp64_sums(a, n, conf, stress, s);
+    const double pt = s[0], l2 = a.l2, hh = 0.5 * double(a.H) * l2;
+    f[TFKT_F_RHO_S] = double(a.rho0) + double(drho) - pt;
+    f[TFKT_F_PSI_TOT] = pt;
+    if (conf) {
+      const double cxx = pt != 0 ? l2 * s[1] / pt : 0, cxy = pt != 0 ? l2 * s[2] / pt : 0,
+                   cyy = pt != 0 ? l2 * s[3] / pt : 0;
+      f[TFKT_F_CXX] = cxx;
+      f[TFKT_F_CXY] = cxy;
+      f[TFKT_F_CYY] = cyy;
+      if (mask & (1u << TFKT_F_QRMS)) f[TFKT_F_QRMS] = sqrt(cxx + cyy);
+    }
+    f[TFKT_F_THXX] = hh * s[4];
+    f[TFKT_F_THXY] = hh * s[5];
+    f[TFKT_F_THYY] = hh * s[6];
+    if (vort) {
+      const double duy_dx = 0.5 * (double(a.U[P + (size_t)y * a.pitch + xp]) -
+                                   double(a.U[P + (size_t)y * a.pitch + xm]));
+      const double dux_dy =
+          0.5 * (double(a.U[(size_t)yp * a.pitch + x]) - double(a.U[(size_t)ym * a.pitch + x]));
+      f[TFKT_F_VORT] = duy_dx - dux_dy;
+    }
+  }
   int slot = 0;
+#pragma unroll
   for (int j = 0; j < TFKT_NFIELDS; ++j)
     if (mask & (1u << j)) out[(size_t)(slot++) * N + k] = f[j];
 }
@@ -426,7 +585,13 @@ cudaError_t launch_velocity(const KernelArgs<real>& a, cudaStream_t s) {
 }
 template <typename real>
 cudaError_t launch_fields(const KernelArgs<real>& a, uint32_t mask, double* out, cudaStream_t s) {
-  fields_kernel<real><<<node_grid(a.nx, a.ny), dim3(TX, TY), 0, s>>>(a, mask, out);
+  const size_t smem = sizeof(real) == 4 ? (size_t)a.nq * sizeof(FieldRow) : 0;   // at most 213 KB
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(fields_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  fields_kernel<real><<<node_grid(a.nx, a.ny), dim3(TX, TY), smem, s>>>(a, mask, out);
   return cudaGetLastError();
 }
 template <typename real>

@@ -113,6 +113,29 @@ def test_slabs_of_partial_tiles_are_bit_identical(T, nx, ny, parts, prec):
     assert np.array_equal(got, ref)
 
 
+@pytest.mark.parametrize("prec", ["FP32", "FP16"])
+@pytest.mark.parametrize("S,R", [(1, 1.0), (3, 1.0), (3, 1.5), (6, 3.0), (7, 3.0)])
+def test_field_sums_of_fp32_contexts(T, S, R, prec):
+    """psi_tot, C and Q_rms, summed in pairs of floats, against FP64 sums over the same
+    psi(r, q): pairs hold about 46 bits, so within 1e-12 of psi_tot and of the trace."""
+    from paper_2201_10132_gb300.inputs import perturbation
+    p = _params(T, 45, 19, S, R, prec)
+    with T.Solver(p, perturbation(45, 19, 5, 0.05, 0.05)) as s:
+        s.step(4)
+        psi, f = s.psi(), s.moments(["psi_tot", "cxx", "cxy", "cyy", "qrms"])
+    h = 0.5 * (S - 1)
+    Q = np.array([(i - h, j - h) for j in range(S) for i in range(S)
+                  if (i - h) ** 2 + (j - h) ** 2 <= R * R + 1e-9])
+    pt = psi.sum(-1)
+    c = {k: 2.0 * (psi * w).sum(-1) / pt for k, w in
+         (("cxx", Q[:, 0] ** 2), ("cxy", Q[:, 0] * Q[:, 1]), ("cyy", Q[:, 1] ** 2))}
+    tr = c["cxx"] + c["cyy"]
+    assert np.abs(f["psi_tot"] - pt).max() <= 1e-12 * np.abs(pt).max()
+    for k in c:
+        assert np.abs(f[k] - c[k]).max() <= 1e-12 * np.abs(tr).max(), k
+    assert np.abs(f["qrms"] ** 2 - tr).max() <= 2e-12 * np.abs(tr).max()
+
+
 @pytest.mark.parametrize("nx,ny,prec", [(64, 32, "FP32"), (40, 24, "FP32"), (416, 64, "FP16")])
 def test_steps_captured_in_a_graph(T, nx, ny, prec):
     """tfkt_step under the caller's stream capture: three replays of two captured steps
