@@ -195,7 +195,7 @@ size_t layout(const Lattice& L, Workspace* w) {
     o = align_up(o + fused_export_capacity(L) * sz, A);
     w->off_ftab = o;
     o = align_up(o + (size_t)L.nq * (9 * sizeof(int) + sz + 25 * sizeof(long long)) +
-                     max_tile_rows(L) * sizeof(int2) + 3 * A, A);
+                     max_tile_rows(L) * sizeof(int2) + 2 * fused_image_size(L.nq) + 5 * A, A);
   }
   return o;
 }
@@ -346,6 +346,8 @@ FusedArgs<real> make_fused(const Ctx* c) {
   f.poff = (const long long*)((const char*)f.dpsi + align_up((size_t)L.nq * sizeof(real), 256));
   f.trow = (const int2*)((const char*)f.poff + align_up((size_t)L.nq * 25 * sizeof(long long), 256));
   f.ntrow = c->ntrow;
+  f.image = (const char*)f.trow + align_up(max_tile_rows(L) * sizeof(int2), 256) +
+            (c->cur ? align_up(fused_image_size(L.nq), 256) : 0);
   f.dvx = (real)c->dvx;
   f.dvy = (real)c->dvy;
   return f;
@@ -363,6 +365,16 @@ tfkt_status upload_fused_tables(Ctx* c, const HostTables& t) {
   if (c->ntrow)
     TFKT_CUDA(c, cudaMemcpy((void*)f.trow, trow.data(), trow.size() * sizeof(int2),
                             cudaMemcpyHostToDevice));
+  if constexpr (std::is_same<real, float>::value) {
+    const int cur = c->cur;
+    for (c->cur = 0; c->cur < 2; ++c->cur) {
+      const std::vector<char> img = fused_image(c->L, t, tgt, poff, (const char*)c->ws.base + c->ws.off_pop[c->cur],
+                                                store_size(c->L));
+      cudaError_t e = cudaMemcpy((void*)make_fused<real>(c).image, img.data(), img.size(), cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) return cuda_fail(c, e, "table image");
+    }
+    c->cur = cur;
+  }
   std::vector<real> d(dpsi.begin(), dpsi.end());
   TFKT_CUDA(c, cudaMemcpy((void*)f.poff, poff.data(), poff.size() * sizeof(long long),
                           cudaMemcpyHostToDevice));
@@ -445,13 +457,15 @@ inline bool step_split(const Ctx* c) { return c->split && !c->lpm_pending; }
 
 // The fused kernel and its fix-up (FP64 contexts step with the Q-split kernels).
 template <typename real, typename S>
-cudaError_t fused_kernel(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
-  if constexpr (std::is_same<real, float>::value) return launch_step_fused<real, S>(a, f, s);
+cudaError_t fused_kernel(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                         bool dependent = false) {
+  if constexpr (std::is_same<real, float>::value) return launch_step_fused<real, S>(a, f, s, dependent);
   else return cudaErrorInvalidValue;
 }
 template <typename real>
-cudaError_t fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
-  if constexpr (std::is_same<real, float>::value) return launch_fixup<real>(a, f, s);
+cudaError_t fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                  bool dependent = false) {
+  if constexpr (std::is_same<real, float>::value) return launch_fixup<real>(a, f, s, dependent);
   else return cudaErrorInvalidValue;
 }
 
@@ -465,8 +479,7 @@ tfkt_status do_step(Ctx* c, int64_t n) {
   // Under a stream capture no programmatic serialisation (the node before may be no
   // kernel), and a two-pass context's first step takes its own moments, so that
   // every replay does.
-  const bool q_split = n > 0 && (c->split || !c->fused);
-  const bool cap = q_split && capturing(c->stream), dep = q_split && !cap;
+  const bool cap = n > 0 && capturing(c->stream), dep = n > 0 && !cap;
   if (cap && !c->fused) c->m_valid = false;
   for (int64_t k = 0; k < n; ++k) {
     KernelArgs<real> a = make_args<real>(c);
@@ -481,8 +494,8 @@ tfkt_status do_step(Ctx* c, int64_t n) {
         TFKT_CUDA(c, launch_moments<real, S>(next_moments_args(a, f), c->stream, dep));
       } else {
         if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
-        TFKT_CUDA(c, (fused_kernel<real, S>(a, f, c->stream)));
-        TFKT_CUDA(c, fixup<real>(a, f, c->stream));
+        TFKT_CUDA(c, (fused_kernel<real, S>(a, f, c->stream, dep)));
+        TFKT_CUDA(c, fixup<real>(a, f, c->stream, dep));
       }
       c->lpm_pending = false;
       c->mcur ^= 1;

@@ -54,8 +54,13 @@ struct Smem {
   uint32_t* bmask;   // [nq] bit g set when displacement group g leaves the disk
 };
 
+// The tables behind Ar, in this order: one block of memory (fused_image on the host).
 constexpr int PQ = 26;   // per-Q-node stride of the pull table (entry pairs 16-byte aligned)
 constexpr int AQ = 12;   // per-Q-node stride of the target table (three 16-byte loads)
+
+__host__ __device__ constexpr uint32_t fused_image_bytes(int nq) {
+  return ((uint32_t)nq * (PQ * 8 + DG * 4 + AQ * 4 + 4) + 15u) & ~15u;
+}
 
 template <typename real, int H>
 __host__ __device__ constexpr size_t smem_layout(int nq, size_t* o_A, size_t* o_Ar, size_t* o_poff,
@@ -77,7 +82,7 @@ __host__ __device__ constexpr size_t smem_layout(int nq, size_t* o_A, size_t* o_
   o += sizeof(int) * (size_t)nq * AQ;
   *o_bm = o;
   o += sizeof(uint32_t) * (size_t)nq;
-  return o;
+  return (o + 15) & ~(size_t)15;   // the image is copied in 16-byte words
 }
 
 template <typename real, int H>
@@ -166,29 +171,60 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   off[6] = yp * pitch + xm; off[7] = yp * pitch + x; off[8] = yp * pitch + xp;
   const uint32_t n = off[4];
 
-  // ---- stage: tables, zeroed accumulators and exchange halo, U on the tile and its ring
-  for (int k = tid; k < nq; k += NT) {
-    uint32_t m = 0;
-    for (int g = 0; g < 9; ++g)
-      if (fa.tgt[k * 9 + g] < 0) m |= 1u << g;
-    sm.bmask[k] = m;
+  let_successor_start();
+  wait_for_predecessor();
+  // this node's density, and the solvent's pulls where their registers are free (FP16 storage
+  // and the stress collision spill with them)
+  const real rho = a.rho0 + Min[(size_t)(nq + M_DRHO) * P + n];
+  const real force = rho * a.tab.arow[y];
+  constexpr bool EARLY = std::is_same<S, real>::value && !STRESS;
+  real hs[9];
+  auto pull_solvent = [&] {
+    static_for<0, 9>([&](auto I) {
+      constexpr int i = I;
+      hs[i] = from_store<real>(ssrc[(size_t)i * P + off[shift_index(-c9x(i), -c9y(i))]]);
+    });
+  };
+  if constexpr (EARLY) pull_solvent();
+
+  // ---- stage: tables, zeroed accumulators and exchange halo, U on the tile and its ring.
+  // The single-run kernel copies the image of its tables (fused_image) asynchronously,
+  // all of it in flight while U is formed; built from the separate tables, each with
+  // its own round trip, and with the solvent's pulls behind them, a tile took 2 to 3 us
+  // more (us per step before and now, with the launches' overlap: 2048 x 512 nodes and
+  // one Q-node 136 and 124, 1024 x 1024 with 9 428 and 411, 512 x 512 with 32 367 and 355,
+  // 2048 x 2048 5099 and 5056; 256 x 256 with 9 37 and 32).
+  if constexpr (!LEAN) {
+    const char* img = static_cast<const char*>(fa.image);
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(sm.ptab);
+    for (uint32_t k = tid * 16; k < fused_image_bytes(nq); k += NT * 16)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(to + k), "l"(img + k) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  } else {
+    for (int k = tid; k < nq; k += NT) {
+      uint32_t m = 0;
+      for (int g = 0; g < 9; ++g)
+        if (fa.tgt[k * 9 + g] < 0) m |= 1u << g;
+      sm.bmask[k] = m;
+    }
+    for (int k = tid; k < nq * AQ; k += NT) {
+      const int q = k / AQ, g = k % AQ;
+      const int t = g < 9 ? fa.tgt[q * 9 + g] : -1;
+      sm.aoff[k] = (t >= 0 ? t : q) * (int)AROW;
+    }
+    for (int k = tid; k < nq * PQ; k += NT) {
+      const int q = k / PQ, i = k % PQ;
+      const long long e = i < 25 ? fa.poff[q * 25 + i] : 0;
+      sm.ptab[k] = e;
+    }
+    for (int k = tid; k < nq * DG; k += NT) {
+      const int q = k / DG, s = k % DG;
+      sm.delta[k] = a.tab.delta[q * 25 + group_member(s < 4 ? s : s + 1)];
+    }
   }
-  for (int k = tid; k < nq * AQ; k += NT) {
-    const int q = k / AQ, g = k % AQ;
-    const int t = g < 9 ? fa.tgt[q * 9 + g] : -1;
-    sm.aoff[k] = (t >= 0 ? t : q) * (int)AROW;
-  }
-  for (int k = tid; k < nq * PQ; k += NT) {
-    const int q = k / PQ, i = k % PQ;
-    const long long e = i < 25 ? fa.poff[q * 25 + i] : 0;
-    if constexpr (LEAN) sm.ptab[k] = e;
-    else sm.ptab[k] = reinterpret_cast<long long>(src + e);
-  }
-  for (int k = tid; k < nq * DG; k += NT) {
-    const int q = k / DG, s = k % DG;
-    sm.delta[k] = a.tab.delta[q * 25 + group_member(s < 4 ? s : s + 1)];
-  }
-  for (int k = tid; k < 20 * HSZ + 2 * HPAD; k += NT) sm.hb[k - HPAD] = real(0);
+  static_assert((20 * HSZ + 2 * HPAD) % 4 == 0 && sizeof(real) == 4, "zeroed in 16-byte words");
+  for (int k = tid; k < (20 * HSZ + 2 * HPAD) / 4; k += NT)
+    reinterpret_cast<float4*>(sm.hb - HPAD)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int k = tid; k < nq * RING; k += NT) sm.Ar[k] = real(0);
   for (int k = tid; k < (TX + 2) * (TY + 2); k += NT) {
     const int hx = k % (TX + 2), hy = k / (TX + 2);
@@ -201,6 +237,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
     sm.Ux[k] = ux;
     sm.Uy[k] = uy;
   }
+  if constexpr (!LEAN) asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
 
   const int c = (y - y0 + 1) * (TX + 2) + (x - x0 + 1);
@@ -220,8 +257,6 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   if (RAGGED && rey == TY) rey = box.h;   // to a partial tile
   const int rcell = (rey + 1) * HX + (rex + 1);
 
-  const real rho = a.rho0 + Min[(size_t)(nq + M_DRHO) * P + n];
-  const real force = rho * a.tab.arow[y];
   real jx_arr = 0, jy_arr = 0, ms_arr = 0;    // own-node arrivals (momentum, solvent mass)
   real jx_r = 0, jy_r = 0, ms_r = 0;          // ring-node arrivals
 
@@ -275,14 +310,13 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   }
 
   // ---- solvent
+  if constexpr (!EARLY) pull_solvent();
   if constexpr (STRESS) {
     // stress quasi-equilibrium: f*_S carries rho_S U and the stress of f,
     // P(f) - rho_S c_s^2 I = [2 tau2 (P(g) - P_eq) + tau2 (F U + U F)] / (2 tau2 + 1) + rho_S U U
-    real hs[9];
     real drs = 0, pxx = 0, pxy = 0, pyy = 0;
     static_for<0, 9>([&](auto I) {
       constexpr int i = I;
-      hs[i] = from_store<real>(ssrc[(size_t)i * P + off[shift_index(-c9x(i), -c9y(i))]]);
       drs += hs[i];
       acc<c9x(i) * c9x(i)>(pxx, hs[i]);
       acc<c9x(i) * c9y(i)>(pxy, hs[i]);
@@ -311,11 +345,9 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
     });
   } else
   {
-    real hs[9];
     real drs = 0, jsx = 0, jsy = 0;
     static_for<0, 9>([&](auto I) {
       constexpr int i = I;
-      hs[i] = from_store<real>(ssrc[(size_t)i * P + off[shift_index(-c9x(i), -c9y(i))]]);
       drs += hs[i];
       acc<c9x(i)>(jsx, hs[i]);
       acc<c9y(i)>(jsy, hs[i]);
@@ -388,21 +420,25 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   }
   char* const Acol = reinterpret_cast<char*>(sm.A) + tid * sizeof(real);
 
-  // ---- polymer, one Q-node at a time
+  // ---- polymer, one Q-node at a time. FP16 storage is worked on in stored units (the
+  // deviation times a power of two), so that no population is unscaled or scaled; the
+  // solvent's momentum joins them in those units, and the flush returns from them (1%
+  // of the instructions; with the staging above 2048 x 2048 nodes 4370 -> 4280 us per step).
+  if constexpr (!RAW) {
+    jx_arr *= a.pscale;
+    jy_arr *= a.pscale;
+    jx_r *= a.pscale;
+    jy_r *= a.pscale;
+  }
   for (int q = 0; q < nq; ++q) {
     const uint32_t bm = sm.bmask[q];
     {
       real dl[DG];
       load_vec<DG>(dl, sm.delta + q * DG);
-      static_for<0, 25>([&](auto I) {   // unscale (FP16 storage), shift to this Q-node
+      static_for<0, 25>([&](auto I) {   // shift to this Q-node
         constexpr int i = I, g = qgroup(c25(i));
-        if constexpr (g == 4) {
-          if constexpr (!RAW) h[i] = from_store<real>(hr[i]) * a.pinv;
-        } else {
-          constexpr int sl = g < 4 ? g : g - 1;
-          if constexpr (RAW) h[i] += dl[sl];
-          else h[i] = from_store<real>(hr[i]) * a.pinv + dl[sl];
-        }
+        if constexpr (!RAW) h[i] = from_store<real>(hr[i]);
+        if constexpr (g != 4) h[i] += dl[g < 4 ? g : g - 1];
       });
     }
     if constexpr (RESHAPE) {
@@ -481,8 +517,8 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
       });
     }
     const real Qx = a.tab.qx[q], Qy = a.tab.qy[q], Fx = a.tab.fx[q], Fy = a.tab.fy[q];
-    const real psi = a.tab.psi0[q] + dpsi;
-    const real qg = Qx * dpx + Qy * dpy;
+    const real psi = RAW ? a.tab.psi0[q] + dpsi : a.tab.psi0[q] * a.pscale + dpsi;
+    const real qg = RAW ? Qx * dpx + Qy * dpy : (Qx * dpx + Qy * dpy) * a.pscale;
     const real jrex = psi * Ux + a.tau_m * a.hl2h * Fx * qg;
     const real jrey = psi * Uy + a.tau_m * a.hl2h * Fy * qg;
     const real jqex = psi * (Qx * G00 + Qy * G10 - a.kappa * Fx);
@@ -551,10 +587,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
         }
       }
       const real hp = a.om2b * h[i] + d;
-      if (live) {
-        if constexpr (std::is_same<S, real>::value) dq[(size_t)i * P] = hp;
-        else dq[(size_t)i * P] = to_store<S>(hp * a.pscale);
-      }
+      if (live) dq[(size_t)i * P] = to_store<S>(hp);
       // an r-moving value goes through the exchange buffer (whether it bounces is
       // settled where the arrivals are summed); the others stay on this r-node
       if constexpr (moves_r(i)) {
@@ -644,13 +677,20 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   }
 
   // ---- flush the next step's moments
+  const real unit = RAW ? real(1) : a.pinv;   // of the polymer's sums
+  if constexpr (!RAW) {
+    jx_arr *= unit;
+    jy_arr *= unit;
+    jx_r *= unit;
+    jy_r *= unit;
+  }
   const bool border = lx == 0 || lx == box.w - 1 || ly == 0 || ly == box.h - 1;
   if (!live) {
     // an idle thread of a partial tile
   } else if (!border) {
     real drho = ms_arr, txx = 0, txy = 0, tyy = 0;
     for (int p = 0; p < nq; ++p) {
-      const real d = sm.A[p * NT + tid] + fa.dpsi[p];
+      const real d = RAW ? sm.A[p * NT + tid] + fa.dpsi[p] : sm.A[p * NT + tid] * unit + fa.dpsi[p];
       Mout[(size_t)p * P + n] = d;
       drho += d;
       const real Qx = a.tab.qx[p], Qy = a.tab.qy[p], Fx = a.tab.fx[p], Fy = a.tab.fy[p];
@@ -665,7 +705,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
     Mout[(size_t)(nq + M_THXY) * P + n] = a.hl2h * txy;
     Mout[(size_t)(nq + M_THYY) * P + n] = a.hl2h * tyy;
   } else {
-    for (int p = 0; p < nq; ++p) Mout[(size_t)p * P + n] = sm.A[p * NT + tid];
+    for (int p = 0; p < nq; ++p) Mout[(size_t)p * P + n] = sm.A[p * NT + tid] * unit;
     Mout[(size_t)(nq + M_DRHO) * P + n] = ms_arr;
     Mout[(size_t)(nq + M_JX) * P + n] = jx_s + jx_arr;
     Mout[(size_t)(nq + M_JY) * P + n] = jy_s + jy_arr;
@@ -674,7 +714,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
     const size_t ntiles = (size_t)ntx * nty;
     const size_t tile = (size_t)bty * ntx + btx;
     real* ex = fa.exports;
-    for (int p = 0; p < nq; ++p) ex[((size_t)p * ntiles + tile) * RING + tid] = sm.Ar[p * RING + tid];
+    for (int p = 0; p < nq; ++p) ex[((size_t)p * ntiles + tile) * RING + tid] = sm.Ar[p * RING + tid] * unit;
     ex[((size_t)(nq + 0) * ntiles + tile) * RING + tid] = ms_r;
     ex[((size_t)(nq + 1) * ntiles + tile) * RING + tid] = jx_rs + jx_r;
     ex[((size_t)(nq + 2) * ntiles + tile) * RING + tid] = jy_rs + jy_r;
@@ -728,6 +768,7 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
   const size_t ntiles = (size_t)ntx * nty;
   const int nq = a.nq;
   const size_t P = a.plane;
+  let_successor_start();
   if (tid < NB) {
     const int k = tid;
     int lx, ly;
@@ -754,6 +795,7 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
 #pragma unroll
     for (int c = 0; c < MAXC; ++c) s_e[c][k] = (size_t)ctile[c] * RING + cpos[c];
   }
+  wait_for_predecessor();
   __syncthreads();
   real* M = fa.Mout;
   const real* ex = fa.exports;
@@ -959,37 +1001,40 @@ size_t max_tile_rows(const Lattice& L) {
 }
 
 template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED>
-static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                                bool dependent) {
   const size_t smem = fused_smem_bytes(a.nq, sizeof(real), TY);
   cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
-  step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED><<<grid, dim3(TX, TY), smem, s>>>(a, f);
-  return cudaGetLastError();
+  return launch(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, grid, dim3(TX, TY), smem, s,
+                dependent, a, f);
 }
 
 template <typename real, typename S>
-cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                              bool dependent) {
   if (f.rshp) {
     // a learned block's increment rides on this step's pull (FP32 storage, whole tiles)
     if constexpr (std::is_same<real, float>::value && std::is_same<S, float>::value) {
       if (f.ntrow) return cudaErrorInvalidValue;
-      return launch_fused<real, S, true, false, false>(a, f, s);
+      return launch_fused<real, S, true, false, false>(a, f, s, dependent);
     } else {
       return cudaErrorInvalidValue;
     }
   }
   const bool stress = a.qe == TFKT_QE_STRESS;
   if (f.ntrow)
-    return stress ? launch_fused<real, S, false, true, true>(a, f, s)
-                  : launch_fused<real, S, false, false, true>(a, f, s);
-  return stress ? launch_fused<real, S, false, true, false>(a, f, s)
-                : launch_fused<real, S, false, false, false>(a, f, s);
+    return stress ? launch_fused<real, S, false, true, true>(a, f, s, dependent)
+                  : launch_fused<real, S, false, false, true>(a, f, s, dependent);
+  return stress ? launch_fused<real, S, false, true, false>(a, f, s, dependent)
+                : launch_fused<real, S, false, false, false>(a, f, s, dependent);
 }
 
 template <typename real, bool RAGGED>
-static cudaError_t launch_fix(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
+static cudaError_t launch_fix(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                              bool dependent) {
   const size_t smem = fix_smem_bytes<real, TY>(a.nq);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(fixup_kernel<real, RAGGED>,
@@ -997,13 +1042,13 @@ static cudaError_t launch_fix(const KernelArgs<real>& a, const FusedArgs<real>& 
     if (e != cudaSuccess) return e;
   }
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
-  fixup_kernel<real, RAGGED><<<grid, FIX_T, smem, s>>>(a, f);
-  return cudaGetLastError();
+  return launch(fixup_kernel<real, RAGGED>, grid, dim3(FIX_T), smem, s, dependent, a, f);
 }
 
 template <typename real>
-cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s) {
-  return f.ntrow ? launch_fix<real, true>(a, f, s) : launch_fix<real, false>(a, f, s);
+cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                         bool dependent) {
+  return f.ntrow ? launch_fix<real, true>(a, f, s, dependent) : launch_fix<real, false>(a, f, s, dependent);
 }
 
 // Batches that launch each run's own single-run kernels (graph branches): the
@@ -1112,11 +1157,37 @@ void fused_tables(const Lattice& L, const HostTables& t, std::vector<int>& tgt,
     }
 }
 
+// The single-run kernel's tables as they lie in its shared memory: pull pointers into
+// the population buffer at `src` (storage elements of es bytes), shift differences
+// (in stored units) of the groups that move in Q, byte offsets of the groups' target rows in A (the
+// Q-node's own row where a group leaves the disk), bounce masks.
+size_t fused_image_size(int nq) { return fused_image_bytes(nq); }
+std::vector<char> fused_image(const Lattice& L, const HostTables& t, const std::vector<int>& tgt,
+                              const std::vector<long long>& poff, const void* src, size_t es) {
+  std::vector<char> img(fused_image_bytes(L.nq), 0);
+  long long* ptab = (long long*)img.data();
+  float* delta = (float*)(ptab + (size_t)L.nq * PQ);
+  int* aoff = (int*)(delta + (size_t)L.nq * DG);
+  uint32_t* bmask = (uint32_t*)(aoff + (size_t)L.nq * AQ);
+  for (int q = 0; q < L.nq; ++q) {
+    for (int i = 0; i < PQ; ++i)
+      ptab[q * PQ + i] = (long long)(uintptr_t)src + (i < 25 ? poff[(size_t)q * 25 + i] * (long long)es : 0);
+    for (int s = 0; s < DG; ++s)
+      delta[q * DG + s] = (float)(polymer_scale(L) * t.delta[(size_t)q * 25 + group_member(s < 4 ? s : s + 1)]);
+    for (int g = 0; g < AQ; ++g) {
+      const int to = g < 9 ? tgt[(size_t)q * 9 + g] : -1;
+      aoff[q * AQ + g] = (to >= 0 ? to : q) * (int)(Geo<TY>::NT * sizeof(float));
+      if (g < 9 && to < 0) bmask[q] |= 1u << g;
+    }
+  }
+  return img;
+}
+
 template cudaError_t launch_step_fused<float, float>(const KernelArgs<float>&,
-                                                      const FusedArgs<float>&, cudaStream_t);
+                                                      const FusedArgs<float>&, cudaStream_t, bool);
 template cudaError_t launch_step_fused<float, __half>(const KernelArgs<float>&,
-                                                       const FusedArgs<float>&, cudaStream_t);
+                                                       const FusedArgs<float>&, cudaStream_t, bool);
 template cudaError_t launch_fixup<float>(const KernelArgs<float>&, const FusedArgs<float>&,
-                                         cudaStream_t);
+                                         cudaStream_t, bool);
 
 }  // namespace tfkt

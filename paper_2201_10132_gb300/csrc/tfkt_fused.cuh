@@ -22,6 +22,31 @@ __device__ __forceinline__ void static_for(F&& f) {
   static_for_impl<B>(f, std::make_integer_sequence<int, N>{});
 }
 
+// Programmatic dependent launch: a kernel lets the next one start its index
+// arithmetic and table loads early, and reads or writes nothing of the state
+// before the kernels in front of it have completed. (Both are no-ops in a launch
+// without the attribute.)
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+// A launch that may start while the stream's previous kernel finishes (dependent),
+// or an ordinary one.
+template <typename... Args>
+cudaError_t launch(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                   bool dependent, const Args&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = at;
+  c.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // Tile geometry for a tile height H (the width is one warp, TX): threads /
 // nodes per tile, ring nodes around it, the exchange buffer's rows and plane.
 // The single-run path uses H = TY; batches pick H by timing (tfkt_batch.cu).

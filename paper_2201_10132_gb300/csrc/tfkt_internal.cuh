@@ -200,6 +200,7 @@ struct FusedArgs {
   const int* tgt;       // [nq][9] target Q-node per Q-displacement group, -1: bounce-back
   const real* dpsi;     // [nq] sum over i of the pull shift differences of Q-node q
   const long long* poff;  // [nq*25] element offset of each pull's source plane
+  const void* image;    // the single-run kernel's tables for the current source buffer
   const int2* trow;     // [ntrow] first row and height of every tile row
   int ntrow;            // 0: whole tiles throughout
   real dvx, dvy;        // r-momentum of all pull shift differences
@@ -318,10 +319,15 @@ size_t max_tile_rows(const Lattice& L);
 void fused_tables(const Lattice& L, const HostTables& t, std::vector<int>& tgt,
                   std::vector<double>& dpsi, double& dvx, double& dvy,
                   std::vector<long long>& poff);
+size_t fused_image_size(int nq);
+std::vector<char> fused_image(const Lattice& L, const HostTables& t, const std::vector<int>& tgt,
+                              const std::vector<long long>& poff, const void* src, size_t es);
 template <typename real, typename S>
-cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s);
+cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                              bool dependent = false);
 template <typename real>
-cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s);
+cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
+                         bool dependent = false);
 // Whether a context of this lattice takes the fused path, with double-buffered moment
 // planes (either quasi-equilibrium).
 bool fused_path(const Lattice& L);

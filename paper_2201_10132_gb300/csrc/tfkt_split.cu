@@ -196,13 +196,6 @@ struct Pair {
 template <int PR>
 using PairOf = Pair<(PR < 3 ? 0 : (PR < 5 ? 1 : 2)), (PR == 0 ? 1 : (PR == 1 || PR == 3 ? 2 : 3))>;
 
-// Programmatic dependent launch: a kernel lets the next one start its index
-// arithmetic and table loads early, and reads or writes nothing of the state
-// before the kernels in front of it have completed. (Both are no-ops in a launch
-// without the attribute.)
-__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;"); }
-
 // ------------------------------------------------------------------ moments
 // Whether the shift differences are folded into the moments and the equilibria (see
 // above) or added to every pulled population.
@@ -596,25 +589,6 @@ std::vector<QRow<real>> build_rows(const Lattice& L, const HostTables& t) {
   return rows;
 }
 
-namespace {
-// A launch that may start while the stream's previous kernel finishes (dependent),
-// or an ordinary one.
-template <typename real>
-cudaError_t launch(void (*kernel)(KernelArgs<real>), dim3 grid, dim3 block, cudaStream_t s,
-                   const KernelArgs<real>& a, bool dependent) {
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = grid;
-  c.blockDim = block;
-  c.stream = s;
-  c.attrs = at;
-  c.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&c, kernel, a);
-}
-}  // namespace
-
 // `n` tasks over at most `most` warps in as few rounds as possible, the warps
 // equally loaded.
 static int even_warps(int n, int most) {
@@ -648,8 +622,8 @@ cudaError_t launch_moments(const KernelArgs<real>& a, cudaStream_t s, bool depen
   auto go = [&](auto MW) {
     constexpr int mw = decltype(MW)::value;
     const int w = a.mom_warps, g = mw / w;
-    return launch<real>(moments_kernel<real, S, mw>, node_blocks(a.nx, a.ny, g), dim3(QN, w, g), s, a,
-                        dependent);
+    return launch(moments_kernel<real, S, mw>, node_blocks(a.nx, a.ny, g), dim3(QN, w, g), 0, s, dependent,
+                  a);
   };
   if (a.mom_warps <= 8) return go(std::integral_constant<int, 8>());
   if constexpr (sizeof(real) == 4)
@@ -685,8 +659,8 @@ cudaError_t launch_step(const KernelArgs<real>& a, cudaStream_t s, bool dependen
   }
   const dim3 grid(nb, split), block(QN, w, g);
   if (a.qe == TFKT_QE_STRESS)
-    return launch<real>(collide_kernel<real, S, true>, grid, block, s, a, dependent);
-  return launch<real>(collide_kernel<real, S, false>, grid, block, s, a, dependent);
+    return launch(collide_kernel<real, S, true>, grid, block, 0, s, dependent, a);
+  return launch(collide_kernel<real, S, false>, grid, block, 0, s, dependent, a);
 }
 
 #define TFKT_INSTANTIATE_SPLIT(real, S)                                                   \
