@@ -34,6 +34,16 @@ tfkt_status cuda_fail(Ctx* c, cudaError_t e, const char* where) {
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Whether the caller is capturing a stream (or that cannot be told).
+bool stream_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // Physical -> lattice parameters (Sec. VII definitions Re = U0 l / nu,
 // Wi = U0 lambda_H / l, beta = eta_s / (eta_s + eta_p), F = eta U0 / l^2):
 // nu_s = c_s^2 tau1 (trapezoidal scheme), lambda_H = zeta / (4 H) with
@@ -432,16 +442,6 @@ tfkt_status init_state(Ctx* c, const double* perturb) {
   return TFKT_OK;
 }
 
-// Whether the caller is capturing a stream (or that cannot be told).
-bool capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-    cudaGetLastError();
-    return true;
-  }
-  return st != cudaStreamCaptureStatusNone;
-}
-
 template <typename real, typename S>
 tfkt_status ensure_moments(Ctx* c) {
   if (c->m_valid) return TFKT_OK;
@@ -479,7 +479,7 @@ tfkt_status do_step(Ctx* c, int64_t n) {
   // Under a stream capture no programmatic serialisation (the node before may be no
   // kernel), and a two-pass context's first step takes its own moments, so that
   // every replay does.
-  const bool cap = n > 0 && capturing(c->stream), dep = n > 0 && !cap;
+  const bool cap = n > 0 && stream_capturing(c->stream), dep = n > 0 && !cap;
   if (cap && !c->fused) c->m_valid = false;
   for (int64_t k = 0; k < n; ++k) {
     KernelArgs<real> a = make_args<real>(c);

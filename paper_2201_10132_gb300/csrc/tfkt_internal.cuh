@@ -264,6 +264,7 @@ struct Ctx {
 // Host helpers (tfkt_api.cu).
 tfkt_status fail(tfkt_status s, const std::string& msg);
 size_t align_up(size_t v, size_t a);
+bool stream_capturing(cudaStream_t s);   // or cannot be told
 tfkt_status map_params(const tfkt_params* p, Lattice* L);
 size_t real_size(const Lattice& L);   // bytes of the compute type (moment planes, tables)
 size_t store_size(const Lattice& L);  // bytes of the population storage type

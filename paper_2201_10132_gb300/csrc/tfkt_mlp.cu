@@ -12,18 +12,11 @@
 #include <string>
 #include <vector>
 
-#include "tfkt_internal.cuh"
+#include "tfkt_fused.cuh"
 #include "tfkt_mlp.cuh"
 
 namespace tfkt {
 namespace {
-
-constexpr int TB = 128;          // samples (threads) per training block
-
-__device__ __forceinline__ float gelu_grad(float z) {
-  return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) +
-         z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
 
 // Inference on raw samples: one warp per TC_ROWS samples, the network on the
 // tensor cores (mlp_warp_tc).
@@ -56,23 +49,41 @@ __global__ void __launch_bounds__(128) forward_kernel(const float* __restrict__ 
 }
 
 // ---- training: forward and backward on the tensor cores
-// Per block TB = 128 samples (4 warps of 32). The forward pass is the inference
-// routine's (standardised inputs and GELU activations as bfloat16 high part plus
-// remainder, bfloat16 weights, FP32 accumulation), keeping pre-activations and
-// activations per sample. Backward: the output layer, the bias sums and the
-// GELU derivatives on the CUDA cores; the weight gradients dW2 = dz2^T h1 and
-// dW1 = dz1^T x (sums over the block's samples) and the propagated error
-// dz2 W2 as mma.sync, both FP32 operands split into high part and remainder
-// (three products per pair: high x high, high x remainder, remainder x high).
-constexpr int TR_LD = 68;   // FP32 row stride of the per-sample tables (float2-aligned)
+// A block of 8 warps takes TB = 128 samples at a time, one 16-row tile per warp, and
+// the grid is at most one block per SM, so that a larger batch adds tiles to a block
+// and no partials. The forward pass is the inference routine's (standardised inputs
+// and GELU activations as bfloat16 high part plus remainder, bfloat16 weights, FP32
+// accumulation), keeping activations and GELU derivatives per sample (the derivative
+// shares its erff with the activation). Backward: the output layer, the bias sums and
+// the GELU derivatives on the CUDA cores; the weight gradients dW2 = dz2^T h1 and
+// dW1 = dz1^T x (sums over samples, in registers over all tiles of the block) and the
+// propagated error dz2 W2 as mma.sync, both FP32 operands split into high part and
+// remainder (three products per pair: high x high, high x remainder, remainder x high).
+//
+// Up to one tile per SM the launches, the wait for the loss and the chain through one
+// tile (14 us, two warps per scheduler, a third of it the GELUs) bound a call, beyond
+// that the tiles. 16384 samples took 72 us for loss, gradient and an Adam step with
+// four warps per block, sums of 128 terms in one thread each (biases, output layer,
+// loss, and the partials of all blocks per weight), strided loads of the samples and
+// separate copies of loss and gradient; now 39. 65536 samples 196 and 81.
+constexpr int TB = 128;          // samples of a tile
+constexpr int TW = 8;            // warps of a block
+constexpr int TT = 32 * TW;      // threads
+constexpr int TR_LD = 68;        // FP32 row stride of the per-sample tables (float2-aligned)
+constexpr int TQ = TT / NH;      // threads that share a column's sum over a tile's samples
+constexpr int MAX_TRAIN_BLOCKS = 152;   // one per SM
+static_assert(TB == 16 * TW && TT == 4 * NH, "tiling of the training kernel");
 
 struct TrainTc {
   MlpTc net;                         // forward weights ([out][in] bfloat16) and normalisation
   __nv_bfloat16 w2t[NH * TC_W2LD];   // W2 transposed ([in][out]) for the propagated error
   float xs[TB * TC_XLD];             // standardised inputs; columns NIN .. TC_K1 - 1 zero
-  float z1[TB * TR_LD], h1[TB * TR_LD], z2[TB * TR_LD], h2[TB * TR_LD];
+  // activations; GELU derivatives, then in their place dz1 and dz2
+  float d1[TB * TR_LD], h1[TB * TR_LD], d2[TB * TR_LD], h2[TB * TR_LD];
   float o[TB * 4], dO[TB * 4];
-  double lsum[TB];
+  float part[TQ][5][NH];             // column sums of the threads that share a column
+  float part3[TW][4];
+  double lsum[TW];
 };
 
 // Fragment pair (p, q) of an FP32 table split into bfloat16 high part and remainder.
@@ -80,98 +91,90 @@ __device__ __forceinline__ void tr_split2(const float* p, const float* q, uint32
   tc_split(*p, *q, hi, lo);
 }
 
-// Forward pass of the warp's 32 samples (rows wb .. wb + 31 of the tables).
-__device__ __forceinline__ void train_forward_warp(TrainTc& sh, int wb, int lane) {
-  const MlpTc& s = sh.net;
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll 1
-  for (int m = 0; m < 2; ++m) {
-    const int r0 = wb + 16 * m + g, r1 = r0 + 8;
-    const float* x0 = sh.xs + r0 * TC_XLD;
-    const float* x1 = sh.xs + r1 * TC_XLD;
-    uint32_t ah1[3][4], al1[3][4];
+// GELU(z) = z Phi(z) and its derivative Phi(z) + z phi(z).
+__device__ __forceinline__ float gelu_and_grad(float z, float& d) {
+  const float e = 1.0f + erff(z * 0.70710678118654752f);
+  d = 0.5f * e + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+  return 0.5f * z * e;
+}
+
+// One hidden layer's activations and derivatives of the warp's rows r0 and r1 from
+// its accumulators, kept in the tables h and d, and the next layer's operands.
+__device__ __forceinline__ void train_activate(const float (&c)[8][4], float* h, float* d, int r0, int r1,
+                                               int t, uint32_t (&ah)[4][4], uint32_t (&al)[4][4]) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int c0 = 16 * k + 2 * t;
-      tc_split(x0[c0], x0[c0 + 1], ah1[k][0], al1[k][0]);
-      tc_split(x1[c0], x1[c0 + 1], ah1[k][1], al1[k][1]);
-      tc_split(x0[c0 + 8], x0[c0 + 9], ah1[k][2], al1[k][2]);
-      tc_split(x1[c0 + 8], x1[c0 + 9], ah1[k][3], al1[k][3]);
-    }
-    float c[8][4];
+  for (int n = 0; n < 8; ++n) {
+    const int col = 8 * n + 2 * t;
+    float a[4], g[4];
 #pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      c[n][0] = c[n][2] = s.b1[8 * n + 2 * t];
-      c[n][1] = c[n][3] = s.b1[8 * n + 2 * t + 1];
-    }
-    tc_layer<3, 8, TC_W1LD>(c, ah1, al1, s.w1, g, t);
-    uint32_t ah[4][4], al[4][4];
-    // keep z1, h1; the next layer's operands from h1
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      const int col = 8 * n + 2 * t;
-      float a[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) a[e] = gelu(c[n][e]);
-      sh.z1[r0 * TR_LD + col] = c[n][0];
-      sh.z1[r0 * TR_LD + col + 1] = c[n][1];
-      sh.z1[r1 * TR_LD + col] = c[n][2];
-      sh.z1[r1 * TR_LD + col + 1] = c[n][3];
-      sh.h1[r0 * TR_LD + col] = a[0];
-      sh.h1[r0 * TR_LD + col + 1] = a[1];
-      sh.h1[r1 * TR_LD + col] = a[2];
-      sh.h1[r1 * TR_LD + col + 1] = a[3];
-      const int k = n >> 1, half = (n & 1) * 2;
-      tc_split(a[0], a[1], ah[k][half], al[k][half]);
-      tc_split(a[2], a[3], ah[k][half + 1], al[k][half + 1]);
-    }
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      c[n][0] = c[n][2] = s.b2[8 * n + 2 * t];
-      c[n][1] = c[n][3] = s.b2[8 * n + 2 * t + 1];
-    }
-    tc_layer<4, 8, TC_W2LD>(c, ah, al, s.w2, g, t);
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      const int col = 8 * n + 2 * t;
-      float a[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) a[e] = gelu(c[n][e]);
-      sh.z2[r0 * TR_LD + col] = c[n][0];
-      sh.z2[r0 * TR_LD + col + 1] = c[n][1];
-      sh.z2[r1 * TR_LD + col] = c[n][2];
-      sh.z2[r1 * TR_LD + col + 1] = c[n][3];
-      sh.h2[r0 * TR_LD + col] = a[0];
-      sh.h2[r0 * TR_LD + col + 1] = a[1];
-      sh.h2[r1 * TR_LD + col] = a[2];
-      sh.h2[r1 * TR_LD + col + 1] = a[3];
-      const int k = n >> 1, half = (n & 1) * 2;
-      tc_split(a[0], a[1], ah[k][half], al[k][half]);
-      tc_split(a[2], a[3], ah[k][half + 1], al[k][half + 1]);
-    }
-    float c3[1][4] = {{s.b3[2 * t], s.b3[2 * t + 1], s.b3[2 * t], s.b3[2 * t + 1]}};
-    tc_layer<4, 1, TC_W2LD>(c3, ah, al, s.w3, g, t);
-    if (2 * t < NOUT) {
-      sh.o[r0 * 4 + 2 * t] = c3[0][0];
-      sh.o[r1 * 4 + 2 * t] = c3[0][2];
-    }
-    if (2 * t + 1 < NOUT) {
-      sh.o[r0 * 4 + 2 * t + 1] = c3[0][1];
-      sh.o[r1 * 4 + 2 * t + 1] = c3[0][3];
-    }
+    for (int e = 0; e < 4; ++e) a[e] = gelu_and_grad(c[n][e], g[e]);
+    *reinterpret_cast<float2*>(d + r0 * TR_LD + col) = make_float2(g[0], g[1]);
+    *reinterpret_cast<float2*>(d + r1 * TR_LD + col) = make_float2(g[2], g[3]);
+    *reinterpret_cast<float2*>(h + r0 * TR_LD + col) = make_float2(a[0], a[1]);
+    *reinterpret_cast<float2*>(h + r1 * TR_LD + col) = make_float2(a[2], a[3]);
+    const int k = n >> 1, half = (n & 1) * 2;
+    tc_split(a[0], a[1], ah[k][half], al[k][half]);
+    tc_split(a[2], a[3], ah[k][half + 1], al[k][half + 1]);
   }
 }
 
-// G[o][i] = sum over the block's TB samples s of D[s][o] B[s][i] for o in this
-// warp's 16 rows (o0 ..) and i < ni (NN n-tiles of 8), written to P[o * ld + i].
-template <int NN>
-__device__ __forceinline__ void train_weight_grad(const float* D, const float* B, int bld, int o0,
-                                                  int ni, float* P, int ld, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  float c[NN][4];
+// Operand fragments of rows r0 and r1 of an FP32 table, NK k-steps of 16 columns.
+template <int NK, int LD>
+__device__ __forceinline__ void train_rows(const float* x, int r0, int r1, int t, uint32_t (&ah)[NK][4],
+                                           uint32_t (&al)[NK][4]) {
+  const float* x0 = x + r0 * LD;
+  const float* x1 = x + r1 * LD;
 #pragma unroll
-  for (int n = 0; n < NN; ++n) c[n][0] = c[n][1] = c[n][2] = c[n][3] = 0.f;
-#pragma unroll 1
+  for (int k = 0; k < NK; ++k) {
+    const int c0 = 16 * k + 2 * t;
+    tc_split(x0[c0], x0[c0 + 1], ah[k][0], al[k][0]);
+    tc_split(x1[c0], x1[c0 + 1], ah[k][1], al[k][1]);
+    tc_split(x0[c0 + 8], x0[c0 + 9], ah[k][2], al[k][2]);
+    tc_split(x1[c0 + 8], x1[c0 + 9], ah[k][3], al[k][3]);
+  }
+}
+
+// Forward pass of the warp's 16 samples (rows wb .. wb + 15 of the tables).
+__device__ __forceinline__ void train_forward_warp(TrainTc& sh, int wb, int lane) {
+  const MlpTc& s = sh.net;
+  const int g = lane >> 2, t = lane & 3;
+  const int r0 = wb + g, r1 = r0 + 8;
+  uint32_t ah1[3][4], al1[3][4], ah[4][4], al[4][4];
+  train_rows<3, TC_XLD>(sh.xs, r0, r1, t, ah1, al1);
+  float c[8][4];
+#pragma unroll
+  for (int n = 0; n < 8; ++n) {
+    c[n][0] = c[n][2] = s.b1[8 * n + 2 * t];
+    c[n][1] = c[n][3] = s.b1[8 * n + 2 * t + 1];
+  }
+  tc_layer<3, 8, TC_W1LD>(c, ah1, al1, s.w1, g, t);
+  train_activate(c, sh.h1, sh.d1, r0, r1, t, ah, al);
+#pragma unroll
+  for (int n = 0; n < 8; ++n) {
+    c[n][0] = c[n][2] = s.b2[8 * n + 2 * t];
+    c[n][1] = c[n][3] = s.b2[8 * n + 2 * t + 1];
+  }
+  tc_layer<4, 8, TC_W2LD>(c, ah, al, s.w2, g, t);
+  train_activate(c, sh.h2, sh.d2, r0, r1, t, ah, al);
+  float c3[1][4] = {{s.b3[2 * t], s.b3[2 * t + 1], s.b3[2 * t], s.b3[2 * t + 1]}};
+  tc_layer<4, 1, TC_W2LD>(c3, ah, al, s.w3, g, t);
+  if (2 * t < NOUT) {
+    sh.o[r0 * 4 + 2 * t] = c3[0][0];
+    sh.o[r1 * 4 + 2 * t] = c3[0][2];
+  }
+  if (2 * t + 1 < NOUT) {
+    sh.o[r0 * 4 + 2 * t + 1] = c3[0][1];
+    sh.o[r1 * 4 + 2 * t + 1] = c3[0][3];
+  }
+}
+
+// c += sum over the tile's samples s of D[s][o] B[s][i] for o in 16 rows (o0 ..) and
+// NN n-tiles of 8 columns i (i0 ..).
+template <int NN>
+__device__ __forceinline__ void train_weight_grad(float (&c)[NN][4], const float* D, const float* B,
+                                                  int bld, int o0, int i0, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll 2
   for (int k = 0; k < TB / 16; ++k) {
     const int s0 = 16 * k + 2 * t;
     uint32_t ah[4], al[4];
@@ -181,7 +184,7 @@ __device__ __forceinline__ void train_weight_grad(const float* D, const float* B
     tr_split2(D + (s0 + 8) * TR_LD + o0 + g + 8, D + (s0 + 9) * TR_LD + o0 + g + 8, ah[3], al[3]);
 #pragma unroll
     for (int n = 0; n < NN; ++n) {
-      const int i = 8 * n + g;
+      const int i = i0 + 8 * n + g;
       uint32_t bh0, bl0, bh1, bl1;
       tr_split2(B + s0 * bld + i, B + (s0 + 1) * bld + i, bh0, bl0);
       tr_split2(B + (s0 + 8) * bld + i, B + (s0 + 9) * bld + i, bh1, bl1);
@@ -190,9 +193,16 @@ __device__ __forceinline__ void train_weight_grad(const float* D, const float* B
       tc_mma(c[n], al, bh0, bh1);
     }
   }
+}
+
+// P[o * ld + i] = c for the columns i < ni.
+template <int NN>
+__device__ __forceinline__ void train_store(const float (&c)[NN][4], int o0, int i0, int ni, float* P, int ld,
+                                            int lane) {
+  const int g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int n = 0; n < NN; ++n) {
-    const int i = 8 * n + 2 * t;
+    const int i = i0 + 8 * n + 2 * t;
     if (i < ni) {
       P[(o0 + g) * ld + i] = c[n][0];
       P[(o0 + g + 8) * ld + i] = c[n][2];
@@ -204,8 +214,8 @@ __device__ __forceinline__ void train_weight_grad(const float* D, const float* B
   }
 }
 
-// Loss and gradient partials of one block of TB samples; partial[b][NWEIGHTS].
-__global__ void __launch_bounds__(TB) loss_grad_kernel(const float* __restrict__ master,
+// Loss and gradient partials of a block's tiles of TB samples; partial[b][NWEIGHTS].
+__global__ void __launch_bounds__(TT) loss_grad_kernel(const float* __restrict__ master,
                                                        const __nv_bfloat16* __restrict__ wmat,
                                                        const float* __restrict__ X,
                                                        const float* __restrict__ T, int64_t n,
@@ -214,129 +224,186 @@ __global__ void __launch_bounds__(TB) loss_grad_kernel(const float* __restrict__
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainTc& sh = *reinterpret_cast<TrainTc*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  mlp_stage_tc(sh.net, master, wmat, tid, TB);
-  for (int k = tid; k < NH * TC_W2LD; k += TB) {
-    const int i = k / TC_W2LD, o = k % TC_W2LD;
-    sh.w2t[k] = o < NH ? wmat[NH * NIN + o * NH + i] : __float2bfloat16(0.0f);
+  const int g = lane >> 2, t = lane & 3, wb = 16 * warp;
+  let_successor_start();
+  wait_for_predecessor();
+  mlp_stage_tc(sh.net, master, wmat, tid, TT);
+  for (int k = tid; k < NH * NH; k += TT) {   // (columns >= NH of w2t are never read)
+    const int o = k / NH, i = k % NH;
+    sh.w2t[i * TC_W2LD + o] = wmat[NH * NIN + k];
   }
+  for (int k = tid; k < TB * (TC_XLD - NIN); k += TT)
+    sh.xs[k / (TC_XLD - NIN) * TC_XLD + NIN + k % (TC_XLD - NIN)] = 0.0f;
   __syncthreads();
   const MlpTc& s = sh.net;
-  const int64_t k = (int64_t)blockIdx.x * TB + tid;
-  const bool valid = k < n;
   const float inv_n = 1.0f / (float)n;
-  // ---- forward, keeping what the backward pass needs
-  float* xs = sh.xs + tid * TC_XLD;
-#pragma unroll
-  for (int i = 0; i < NIN; ++i) xs[i] = valid ? (X[k * NIN + i] - s.mx[i]) * s.rsx[i] : 0.0f;
-#pragma unroll
-  for (int i = NIN; i < TC_XLD; ++i) xs[i] = 0.0f;
-  __syncwarp();
-  train_forward_warp(sh, warp * 32, lane);
-  __syncwarp();
+  // sums over the block's tiles: this warp's part of the matrices' gradients, and for
+  // column `col` a quarter of the samples of db1, db2 and the three rows of dW3
+  float cw1[3][4] = {}, cw2[4][4] = {};
+  const int o0 = 16 * (warp & 3), half = warp >> 2;
+  const int col = tid % NH, quarter = tid / NH;
+  float sb1 = 0.0f, sb2 = 0.0f, sw3[NOUT] = {}, sb3[NOUT] = {};
   double lsq = 0.0;
-  for (int j = 0; j < NOUT; ++j) {
-    float d = 0.0f;
-    if (valid) {
-      const float tj = (T[k * NOUT + j] - s.mt[j]) / s.st[j];
-      const float r = sh.o[tid * 4 + j] - tj;
-      lsq += (double)r * (double)r;
-      d = 2.0f * r * inv_n;
+  const int64_t ntiles = (n + TB - 1) / TB;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    // ---- standardised inputs
+    const int64_t k0 = tile * TB;
+    const int rows = (int)(n - k0 < TB ? n - k0 : TB);
+    for (int k = tid; k < TB * NIN; k += TT) {
+      const int r = k / NIN, i = k % NIN;
+      sh.xs[r * TC_XLD + i] = r < rows ? (X[k0 * NIN + k] - s.mx[i]) * s.rsx[i] : 0.0f;
     }
-    sh.dO[tid * 4 + j] = d;
-  }
-  sh.lsum[tid] = lsq;
-  __syncthreads();
-  float* P = partial + (size_t)blockIdx.x * TFKT_MLP_NWEIGHTS;
-  // ---- output layer: dW3 = sum_s dO h2^T, db3 = sum_s dO (invalid samples carry dO = 0)
-  for (int e = tid; e < NOUT * NH + NOUT; e += TB) {
-    float acc = 0.0f;
-    if (e < NOUT * NH) {
-      const int j = e / NH, i = e % NH;
-      for (int r = 0; r < TB; ++r) acc = fmaf(sh.dO[r * 4 + j], sh.h2[r * TR_LD + i], acc);
-      P[OW3 + e] = acc;
-    } else {
-      const int j = e - NOUT * NH;
-      for (int r = 0; r < TB; ++r) acc += sh.dO[r * 4 + j];
-      P[OB3 + j] = acc;
-    }
-  }
-  // ---- dz2 = (W3^T dO) GELU'(z2) for this thread's sample, in place of z2
-  for (int o = 0; o < NH; ++o) {
-    float acc = 0.0f;
-    for (int j = 0; j < NOUT; ++j)
-      acc = fmaf(__bfloat162float(s.w3[j * TC_W2LD + o]), sh.dO[tid * 4 + j], acc);
-    sh.z2[tid * TR_LD + o] = acc * gelu_grad(sh.z2[tid * TR_LD + o]);
-  }
-  __syncthreads();
-  // ---- layer 2: dW2 = dz2^T h1 (warp: 16 output rows), db2 = sum_s dz2
-  train_weight_grad<8>(sh.z2, sh.h1, TR_LD, 16 * warp, NH, P + OW2, NH, lane);
-  if (tid < NH) {
-    float acc = 0.0f;
-    for (int r = 0; r < TB; ++r) acc += sh.z2[r * TR_LD + tid];
-    P[OB2 + tid] = acc;
-  }
-  // ---- dz1 = (dz2 W2) GELU'(z1) for the warp's 32 samples, in place of z1
-  {
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll 1
-    for (int m = 0; m < 2; ++m) {
-      const int r0 = warp * 32 + 16 * m + g, r1 = r0 + 8;
-      uint32_t ah[4][4], al[4][4];
+    __syncthreads();
+    // ---- forward, and the error of the outputs, of the warp's own samples
+    train_forward_warp(sh, wb, lane);
+    __syncwarp();
+    if (lane < 16) {
+      const int r = wb + lane;
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const int c0 = 16 * kk + 2 * t;
-        const float* d0 = sh.z2 + r0 * TR_LD;
-        const float* d1 = sh.z2 + r1 * TR_LD;
-        tc_split(d0[c0], d0[c0 + 1], ah[kk][0], al[kk][0]);
-        tc_split(d1[c0], d1[c0 + 1], ah[kk][1], al[kk][1]);
-        tc_split(d0[c0 + 8], d0[c0 + 9], ah[kk][2], al[kk][2]);
-        tc_split(d1[c0 + 8], d1[c0 + 9], ah[kk][3], al[kk][3]);
+      for (int j = 0; j < NOUT; ++j) {
+        float d = 0.0f;
+        if (r < rows) {
+          const float tj = (T[(k0 + r) * NOUT + j] - s.mt[j]) / s.st[j];
+          const float e = sh.o[r * 4 + j] - tj;
+          lsq += (double)e * (double)e;
+          d = 2.0f * e * inv_n;
+        }
+        sh.dO[r * 4 + j] = d;
+        sb3[j] += d;
       }
-      float c[8][4];
+      sh.dO[r * 4 + 3] = 0.0f;
+    }
+    __syncwarp();
+    // ---- dz2 = (W3^T dO) GELU'(z2), in place of the derivative
 #pragma unroll
-      for (int nn = 0; nn < 8; ++nn) c[nn][0] = c[nn][1] = c[nn][2] = c[nn][3] = 0.f;
+    for (int u = 0; u < 2; ++u) {
+      const int c = lane + 32 * u;
+      float w[NOUT];
+#pragma unroll
+      for (int j = 0; j < NOUT; ++j) w[j] = __bfloat162float(s.w3[j * TC_W2LD + c]);
+#pragma unroll 4
+      for (int r = wb; r < wb + 16; ++r) {
+        const float4 e = *reinterpret_cast<const float4*>(sh.dO + 4 * r);
+        sh.d2[r * TR_LD + c] *= fmaf(w[2], e.z, fmaf(w[1], e.y, w[0] * e.x));
+      }
+    }
+    __syncthreads();
+    // ---- layer 2 and the output layer: dW2 = dz2^T h1, db2, dW3 = dO^T h2
+    train_weight_grad<4>(cw2, sh.d2, sh.h1, TR_LD, o0, 32 * half, lane);
+#pragma unroll 4
+    for (int r = quarter * (TB / TQ); r < (quarter + 1) * (TB / TQ); ++r) {
+      const float h = sh.h2[r * TR_LD + col];
+      const float4 e = *reinterpret_cast<const float4*>(sh.dO + 4 * r);
+      sw3[0] = fmaf(e.x, h, sw3[0]);
+      sw3[1] = fmaf(e.y, h, sw3[1]);
+      sw3[2] = fmaf(e.z, h, sw3[2]);
+      sb2 += sh.d2[r * TR_LD + col];
+    }
+    // ---- dz1 = (dz2 W2) GELU'(z1) for the warp's samples, in place of the derivative
+    {
+      const int r0 = wb + g, r1 = r0 + 8;
+      uint32_t ah[4][4], al[4][4];
+      train_rows<4, TR_LD>(sh.d2, r0, r1, t, ah, al);
+      float c[8][4] = {};
       tc_layer<4, 8, TC_W2LD>(c, ah, al, sh.w2t, g, t);
 #pragma unroll
       for (int nn = 0; nn < 8; ++nn) {
-        const int col = 8 * nn + 2 * t;
-        float* z0 = sh.z1 + r0 * TR_LD + col;
-        float* z1r = sh.z1 + r1 * TR_LD + col;
-        z0[0] = c[nn][0] * gelu_grad(z0[0]);
-        z0[1] = c[nn][1] * gelu_grad(z0[1]);
-        z1r[0] = c[nn][2] * gelu_grad(z1r[0]);
-        z1r[1] = c[nn][3] * gelu_grad(z1r[1]);
+        float2* z0 = reinterpret_cast<float2*>(sh.d1 + r0 * TR_LD + 8 * nn + 2 * t);
+        float2* z1 = reinterpret_cast<float2*>(sh.d1 + r1 * TR_LD + 8 * nn + 2 * t);
+        const float2 a = *z0, b = *z1;
+        *z0 = make_float2(c[nn][0] * a.x, c[nn][1] * a.y);
+        *z1 = make_float2(c[nn][2] * b.x, c[nn][3] * b.y);
       }
     }
+    __syncthreads();
+    // ---- layer 1: dW1 = dz1^T x (inputs padded to 48), db1
+    train_weight_grad<3>(cw1, sh.d1, sh.xs, TC_XLD, o0, 24 * half, lane);
+#pragma unroll 8
+    for (int r = quarter * (TB / TQ); r < (quarter + 1) * (TB / TQ); ++r) sb1 += sh.d1[r * TR_LD + col];
+    __syncthreads();   // the tables are overwritten by the next tile
+  }
+  // ---- the block's partials; shared sums in a fixed order
+  float* P = partial + (size_t)blockIdx.x * TFKT_MLP_NWEIGHTS;
+  train_store<4>(cw2, o0, 32 * half, NH, P + OW2, NH, lane);
+  train_store<3>(cw1, o0, 24 * half, NIN, P + OW1, NIN, lane);
+  sh.part[quarter][0][col] = sb1;
+  sh.part[quarter][1][col] = sb2;
+#pragma unroll
+  for (int j = 0; j < NOUT; ++j) sh.part[quarter][2 + j][col] = sw3[j];
+#pragma unroll
+  for (int m = 8; m > 0; m >>= 1) {   // over the 16 lanes that hold samples
+    lsq += __shfl_down_sync(0xffffffffu, lsq, m, 16);
+#pragma unroll
+    for (int j = 0; j < NOUT; ++j) sb3[j] += __shfl_down_sync(0xffffffffu, sb3[j], m, 16);
+  }
+  if (lane == 0) {
+    sh.lsum[warp] = lsq;
+#pragma unroll
+    for (int j = 0; j < NOUT; ++j) sh.part3[warp][j] = sb3[j];
   }
   __syncthreads();
-  // ---- layer 1: dW1 = dz1^T x (warp: 16 output rows, inputs padded to 48), db1 = sum_s dz1
-  train_weight_grad<6>(sh.z1, sh.xs, TC_XLD, 16 * warp, NIN, P + OW1, NIN, lane);
-  if (tid < NH) {
-    float acc = 0.0f;
-    for (int r = 0; r < TB; ++r) acc += sh.z1[r * TR_LD + tid];
-    P[OB1 + tid] = acc;
+  for (int k = tid; k < 5 * NH; k += TT) {
+    const int c = k % NH, v = k / NH;
+    float a = sh.part[0][v][c];
+#pragma unroll
+    for (int q = 1; q < TQ; ++q) a += sh.part[q][v][c];
+    P[v == 0 ? OB1 + c : (v == 1 ? OB2 + c : OW3 + (v - 2) * NH + c)] = a;
   }
-  if (tid == 0) {
+  if (tid < NOUT) {
+    float a = 0.0f;
+    for (int w = 0; w < TW; ++w) a += sh.part3[w][tid];
+    P[OB3 + tid] = a;
+  }
+  if (tid == 32) {
     double l = 0.0;
-    for (int r = 0; r < TB; ++r) l += sh.lsum[r];
+    for (int w = 0; w < TW; ++w) l += sh.lsum[w];
     lpart[blockIdx.x] = l;
   }
 }
 
-// grad[w] = sum over blocks of partial[b][w], in block order; loss = sum lpart / n.
-__global__ void reduce_kernel(const float* __restrict__ partial, int nblocks,
-                              float* __restrict__ grad, const double* __restrict__ lpart,
-                              double* __restrict__ loss, int64_t n) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w < TFKT_MLP_NWEIGHTS) {
-    float acc = 0.0f;
-    for (int b = 0; b < nblocks; ++b) acc += partial[(size_t)b * TFKT_MLP_NWEIGHTS + w];
-    grad[w] = acc;
-  }
-  if (w == 0) {
+// grad[w] = sum over blocks of partial[b][w], eight threads per weight with an eighth
+// of the blocks each, in a fixed order; loss = sum lpart / n by the last block. out:
+// the caller's copy of the gradient, or null.
+constexpr int RD_W = 32, RD_S = 8;   // weights and shares of a block
+__global__ void __launch_bounds__(RD_W * RD_S) reduce_kernel(const float* __restrict__ partial, int nblocks,
+                                                             float* __restrict__ grad,
+                                                             float* __restrict__ out,
+                                                             const double* __restrict__ lpart,
+                                                             double* __restrict__ loss, int64_t n) {
+  __shared__ float part[RD_S][RD_W];
+  __shared__ double lp[RD_S];
+  const int lane = threadIdx.x % RD_W, share = threadIdx.x / RD_W;
+  let_successor_start();
+  wait_for_predecessor();
+  if (blockIdx.x == gridDim.x - 1) {   // the loss
     double l = 0.0;
-    for (int b = 0; b < nblocks; ++b) l += lpart[b];
-    *loss = l / (double)n;
+    for (int b = threadIdx.x; b < nblocks; b += RD_W * RD_S) l += lpart[b];
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) l += __shfl_down_sync(0xffffffffu, l, m);
+    if (lane == 0) lp[share] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int k = 0; k < RD_S; ++k) t += lp[k];
+      *loss = t / (double)n;
+    }
+    return;
+  }
+  const int w = blockIdx.x * RD_W + lane;
+  float a = 0.0f;
+  if (w < TFKT_MLP_NWEIGHTS) {
+    const int per = (nblocks + RD_S - 1) / RD_S;
+    const int b1 = min(nblocks, (share + 1) * per);
+#pragma unroll 8
+    for (int b = share * per; b < b1; ++b) a += partial[(size_t)b * TFKT_MLP_NWEIGHTS + w];
+  }
+  part[share][lane] = a;
+  __syncthreads();
+  if (share == 0 && w < TFKT_MLP_NWEIGHTS) {
+#pragma unroll
+    for (int k = 1; k < RD_S; ++k) a += part[k][lane];
+    grad[w] = a;
+    if (out) out[w] = a;
   }
 }
 
@@ -346,6 +413,8 @@ __global__ void adam_kernel(float* __restrict__ master, __nv_bfloat16* __restric
                             const float* __restrict__ grad, float lr, float b1, float b2,
                             float eps, float c1, float c2) {
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  let_successor_start();
+  wait_for_predecessor();
   if (w >= TFKT_MLP_NWEIGHTS) return;
   const float g = grad[w];
   const float mw = b1 * m[w] + (1.0f - b1) * g;
@@ -381,16 +450,29 @@ tfkt_status cuda_err(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_err(e_, #__VA_ARGS__);  \
   } while (0)
 
-tfkt_status ensure_blocks(tfkt_mlp* net, int nblocks) {
-  if (nblocks <= net->max_blocks) return TFKT_OK;
+// What only training needs, on its first use: the partial sums of nb blocks.
+tfkt_status ensure_training(tfkt_mlp* net, int nb) {
+  if (!net->lpart) MLP_CUDA(cudaMalloc(&net->lpart, (MAX_TRAIN_BLOCKS + 1) * sizeof(double)));
+  if (nb <= net->partial_blocks) return TFKT_OK;
   if (net->partial) MLP_CUDA(cudaFree(net->partial));
-  if (net->lpart) MLP_CUDA(cudaFree(net->lpart));
   net->partial = nullptr;
-  net->lpart = nullptr;
-  net->max_blocks = 0;
-  MLP_CUDA(cudaMalloc(&net->partial, (size_t)nblocks * TFKT_MLP_NWEIGHTS * sizeof(float)));
-  MLP_CUDA(cudaMalloc(&net->lpart, (size_t)nblocks * sizeof(double)));
-  net->max_blocks = nblocks;
+  net->partial_blocks = 0;
+  MLP_CUDA(cudaMalloc(&net->partial, (size_t)nb * TFKT_MLP_NWEIGHTS * sizeof(float)));
+  net->partial_blocks = nb;
+  return TFKT_OK;
+}
+
+// Where reduce_kernel leaves the loss that the host reads. From the second read on it
+// is pinned host memory, which saves the copy (6 us of 45 at 16384 samples) but takes
+// 75 us to allocate: a network that is evaluated once goes without.
+tfkt_status loss_target(tfkt_mlp* net, bool read, double** at) {
+  *at = net->loss_host ? net->loss_host : net->lpart + MAX_TRAIN_BLOCKS;
+  if (!read || net->loss_host) return TFKT_OK;
+  if (net->loss_read) {
+    MLP_CUDA(cudaMallocHost(&net->loss_host, sizeof(double)));
+    *at = net->loss_host;
+  }
+  net->loss_read = true;
   return TFKT_OK;
 }
 
@@ -419,8 +501,7 @@ tfkt_status tfkt_mlp_create(const float* params, void* stream, tfkt_mlp** out) {
       (e = cudaMalloc(&net->d.wmat, NMAT * sizeof(__nv_bfloat16))) != cudaSuccess ||
       (e = cudaMalloc(&net->m, TFKT_MLP_NWEIGHTS * sizeof(float))) != cudaSuccess ||
       (e = cudaMalloc(&net->v, TFKT_MLP_NWEIGHTS * sizeof(float))) != cudaSuccess ||
-      (e = cudaMalloc(&net->grad, TFKT_MLP_NWEIGHTS * sizeof(float))) != cudaSuccess ||
-      (e = cudaMalloc(&net->loss_dev, sizeof(double))) != cudaSuccess) {
+      (e = cudaMalloc(&net->grad, TFKT_MLP_NWEIGHTS * sizeof(float))) != cudaSuccess) {
     tfkt_mlp_destroy(net);
     cudaGetLastError();   // clear the allocation error
     return fail(TFKT_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
@@ -441,13 +522,16 @@ tfkt_status tfkt_mlp_create(const float* params, void* stream, tfkt_mlp** out) {
 tfkt_status tfkt_mlp_destroy(tfkt_mlp* net) {
   if (!net) return TFKT_OK;
   cudaError_t e = cudaStreamSynchronize(net->stream);
-  void* ptrs[] = {net->d.master, net->d.wmat, net->m, net->v, net->grad, net->partial, net->lpart,
-                  net->loss_dev};
+  void* ptrs[] = {net->d.master, net->d.wmat, net->m, net->v, net->grad, net->partial, net->lpart};
   for (void* p : ptrs)
     if (p) {
       cudaError_t f = cudaFree(p);
       if (e == cudaSuccess) e = f;
     }
+  if (net->loss_host) {
+    cudaError_t f = cudaFreeHost(net->loss_host);
+    if (e == cudaSuccess) e = f;
+  }
   delete net;
   if (e != cudaSuccess) return cuda_err(e, "destroy");
   return TFKT_OK;
@@ -491,26 +575,28 @@ tfkt_status tfkt_mlp_loss_grad(tfkt_mlp* net, const float* X, const float* T, in
                                double* loss, float* grad) {
   NvtxRange nvtx_range("tfkt_mlp_loss_grad");
   if (!net || n < 1 || !X || !T) return fail(TFKT_EINVAL, "bad argument");
-  const int64_t nb = (n + TB - 1) / TB;
-  if (nb > (1 << 20)) return fail(TFKT_EINVAL, "batch too large (at most 2^27 samples)");
-  tfkt_status s = ensure_blocks(net, (int)nb);
-  if (s != TFKT_OK) return s;
+  const int64_t tiles = (n + TB - 1) / TB;
+  if (tiles > (1 << 20)) return fail(TFKT_EINVAL, "batch too large (at most 2^27 samples)");
+  const int nb = (int)(tiles < MAX_TRAIN_BLOCKS ? tiles : MAX_TRAIN_BLOCKS);
+  tfkt_status st = ensure_training(net, nb);
+  double* at = nullptr;
+  if (st == TFKT_OK) st = loss_target(net, loss != nullptr, &at);
+  if (st != TFKT_OK) return st;
   const size_t smem = sizeof(TrainTc);
   MLP_CUDA(cudaFuncSetAttribute(loss_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem));
-  loss_grad_kernel<<<(unsigned)nb, TB, smem, net->stream>>>(net->d.master, net->d.wmat, X, T, n,
-                                                            net->partial, net->lpart);
-  MLP_CUDA(cudaGetLastError());
-  reduce_kernel<<<(TFKT_MLP_NWEIGHTS + 255) / 256, 256, 0, net->stream>>>(
-      net->partial, (int)nb, net->grad, net->lpart, net->loss_dev, n);
-  MLP_CUDA(cudaGetLastError());
-  if (grad)
-    MLP_CUDA(cudaMemcpyAsync(grad, net->grad, TFKT_MLP_NWEIGHTS * sizeof(float),
-                             cudaMemcpyDeviceToDevice, net->stream));
+  const bool dep = !stream_capturing(net->stream);
+  MLP_CUDA(launch(loss_grad_kernel, dim3(nb), dim3(TT), smem, net->stream, dep,
+                  (const float*)net->d.master, (const __nv_bfloat16*)net->d.wmat, X, T, n,
+                  net->partial, net->lpart));
+  MLP_CUDA(launch(reduce_kernel, dim3((TFKT_MLP_NWEIGHTS + RD_W - 1) / RD_W + 1), dim3(RD_W * RD_S), 0,
+                  net->stream, dep, (const float*)net->partial, nb, net->grad, grad,
+                  (const double*)net->lpart, at, n));
   if (loss) {
-    MLP_CUDA(cudaMemcpyAsync(loss, net->loss_dev, sizeof(double), cudaMemcpyDeviceToHost,
-                             net->stream));
+    if (at != net->loss_host)
+      MLP_CUDA(cudaMemcpyAsync(loss, at, sizeof(double), cudaMemcpyDeviceToHost, net->stream));
     MLP_CUDA(cudaStreamSynchronize(net->stream));
+    if (at == net->loss_host) *loss = *(volatile double*)net->loss_host;
   }
   return TFKT_OK;
 }
@@ -523,9 +609,9 @@ tfkt_status tfkt_mlp_adam(tfkt_mlp* net, float lr, float beta1, float beta2, flo
   net->t += 1;
   const float c1 = (float)(1.0 / (1.0 - std::pow((double)beta1, (double)net->t)));
   const float c2 = (float)(1.0 / (1.0 - std::pow((double)beta2, (double)net->t)));
-  adam_kernel<<<(TFKT_MLP_NWEIGHTS + 255) / 256, 256, 0, net->stream>>>(
-      net->d.master, net->d.wmat, net->m, net->v, net->grad, lr, beta1, beta2, eps, c1, c2);
-  MLP_CUDA(cudaGetLastError());
+  MLP_CUDA(launch(adam_kernel, dim3((TFKT_MLP_NWEIGHTS + 127) / 128), dim3(128), 0, net->stream,
+                  !stream_capturing(net->stream), net->d.master, net->d.wmat, net->m, net->v,
+                  (const float*)net->grad, lr, beta1, beta2, eps, c1, c2));
   return TFKT_OK;
 }
 

@@ -38,9 +38,9 @@ constexpr int TC_ROWS = 32;                 // samples per warp pass
 constexpr int TC_K1 = 48;                   // layer-1 inner size, NIN padded to 3 steps of 16
 constexpr int TC_W1LD = 56, TC_W2LD = 72;   // bfloat16 row strides (padded against bank conflicts)
 constexpr int TC_XLD = 52;                  // FP32 row stride of a warp's standardised samples
-static_assert(NIN <= TC_K1 && NH == 64 && NOUT <= 8, "tensor-core tiling of the network");
+static_assert(NIN <= TC_K1 && NIN % 8 == 0 && NH == 64 && NOUT <= 8, "tensor-core tiling of the network");
 
-struct MlpTc {
+struct alignas(16) MlpTc {
   __nv_bfloat16 w1[NH * TC_W1LD];      // [out][in], in >= NIN zero
   __nv_bfloat16 w2[NH * TC_W2LD];      // [out][in]
   __nv_bfloat16 w3[8 * TC_W2LD];       // [out][in], out >= NOUT zero
@@ -55,18 +55,22 @@ constexpr size_t tc_smem_bytes(int warps) {
 
 __device__ __forceinline__ void mlp_stage_tc(MlpTc& s, const float* master,
                                              const __nv_bfloat16* wmat, int tid, int nthreads) {
-  const __nv_bfloat16 zero = __float2bfloat16(0.0f);
-  for (int k = tid; k < NH * TC_W1LD; k += nthreads) {
-    const int o = k / TC_W1LD, i = k % TC_W1LD;
-    s.w1[k] = i < NIN ? wmat[o * NIN + i] : zero;
+  // 16-byte chunks of eight columns; padding columns that the MMAs read are zero
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  auto chunk = [&](const __nv_bfloat16* p) { return *reinterpret_cast<const uint4*>(p); };
+  constexpr int C1 = TC_K1 / 8, C2 = NH / 8;
+  for (int k = tid; k < NH * C1; k += nthreads) {
+    const int o = k / C1, i = 8 * (k % C1);
+    *reinterpret_cast<uint4*>(s.w1 + o * TC_W1LD + i) = i < NIN ? chunk(wmat + o * NIN + i) : zero;
   }
-  for (int k = tid; k < NH * TC_W2LD; k += nthreads) {
-    const int o = k / TC_W2LD, i = k % TC_W2LD;
-    s.w2[k] = i < NH ? wmat[NH * NIN + o * NH + i] : zero;
+  for (int k = tid; k < NH * C2; k += nthreads) {
+    const int o = k / C2, i = 8 * (k % C2);
+    *reinterpret_cast<uint4*>(s.w2 + o * TC_W2LD + i) = chunk(wmat + NH * NIN + o * NH + i);
   }
-  for (int k = tid; k < 8 * TC_W2LD; k += nthreads) {
-    const int o = k / TC_W2LD, i = k % TC_W2LD;
-    s.w3[k] = (o < NOUT && i < NH) ? wmat[NH * NIN + NH * NH + o * NH + i] : zero;
+  for (int k = tid; k < 8 * C2; k += nthreads) {
+    const int o = k / C2, i = 8 * (k % C2);
+    *reinterpret_cast<uint4*>(s.w3 + o * TC_W2LD + i) =
+        o < NOUT ? chunk(wmat + NH * NIN + NH * NH + o * NH + i) : zero;
   }
   for (int k = tid; k < NH; k += nthreads) {
     s.b1[k] = master[OB1 + k];
@@ -198,10 +202,11 @@ struct tfkt_mlp {
   float* m = nullptr;         // [NWEIGHTS] Adam first moments
   float* v = nullptr;         // [NWEIGHTS] Adam second moments
   float* grad = nullptr;      // [NWEIGHTS] last gradient
-  float* partial = nullptr;   // [max_blocks][NWEIGHTS] per-block gradient partials
-  double* lpart = nullptr;    // [max_blocks] per-block loss partials
-  double* loss_dev = nullptr;
-  int max_blocks = 0;
+  float* partial = nullptr;   // per-block gradient partials
+  int partial_blocks = 0;     // blocks that it holds
+  double* lpart = nullptr;    // per-block loss partials, then the loss
+  double* loss_host = nullptr;  // pinned: the last loss, from its second read on
+  bool loss_read = false;
   int64_t t = 0;              // Adam steps taken
   cudaStream_t stream = nullptr;
 };

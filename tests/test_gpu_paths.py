@@ -160,3 +160,37 @@ def test_steps_captured_in_a_graph(T, nx, ny, prec):
         got = s.moments()
     for k in ref:
         assert np.array_equal(got[k], ref[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128, 152 * 128 + 1, 40000])
+def test_training_gradient_over_tile_counts(T, n):
+    """Loss and gradient for sample counts at the edges of a tile of 128 samples and of one
+    tile per block, against FP64 autograd with the same bfloat16 matrices (1e-4 of each
+    tensor's largest magnitude, as in tests/test_gpu_lpm.py); the caller's copy of the
+    gradient may be at any 4-byte boundary, and so may the samples."""
+    import torch
+    from paper_2201_10132_gb300 import train_lpm
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    vec, _ = train_lpm.load()
+    w = {k: torch.from_numpy(np.array(v)).cuda() for k, v in T.unpack_mlp(vec).items()}
+    X = torch.empty(n * T.MLP_IN + 1, device="cuda")[1:].view(n, T.MLP_IN)
+    X.copy_(torch.randn((n, T.MLP_IN), generator=g, device="cuda") * w["sx"] + w["mx"])
+    Y = torch.randn((n, T.MLP_OUT), generator=g, device="cuda") * w["st"] + w["mt"]
+    grad = torch.empty(T.MLP_NWEIGHTS + 1, device="cuda")[1:]
+    net = T.Mlp(vec)
+    loss = net.loss_grad(X.data_ptr(), Y.data_ptr(), n, grad.data_ptr())
+    net.close()
+    p = [(w[k].bfloat16() if k[0] == "W" else w[k]).double().requires_grad_()
+         for k in ("W1", "b1", "W2", "b2", "W3", "b3")]
+    act = torch.nn.functional.gelu
+    x = (X.double() - w["mx"].double()) / w["sx"].double()
+    t = (Y.double() - w["mt"].double()) / w["st"].double()
+    o = act(act(x @ p[0].T + p[1]) @ p[2].T + p[3]) @ p[4].T + p[5]
+    ref = ((o - t) ** 2).sum() / n
+    assert loss == pytest.approx(float(ref), rel=1e-4)
+    k = 0
+    for r in torch.autograd.grad(ref, p):
+        got = grad[k:k + r.numel()].double().view_as(r)
+        k += r.numel()
+        assert (got - r).abs().max() <= 1e-4 * r.abs().max()
