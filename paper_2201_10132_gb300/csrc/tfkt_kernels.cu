@@ -35,34 +35,6 @@ __device__ __forceinline__ Offsets node_offsets(int x, int y, int nx, int ny, si
   return f;
 }
 
-// Mixture velocity U of f at node n (Sec. VI-C, moments of f): summing the
-// g -> f momentum relations over both species with the body force applied
-// by the same half-step rule gives rho U = J(g) + (E + rho a) / 2, where the
-// elastic force E = div Theta (Sec. III, Eq. IDef) by central differences.
-template <typename real>
-__device__ __forceinline__ void mixture_velocity(const KernelArgs<real>& a, int x, int y,
-                                                 real& ux, real& uy, real& rho) {
-  const int nq = a.nq;
-  const size_t P = a.plane;
-  const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
-  const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y == a.ny - 1 ? 0 : y + 1;
-  const size_t n = (size_t)y * a.pitch + x;
-  const size_t nxm = (size_t)y * a.pitch + xm, nxp = (size_t)y * a.pitch + xp;
-  const size_t nym = (size_t)ym * a.pitch + x, nyp = (size_t)yp * a.pitch + x;
-  const real* M = a.M;
-  const real* Txx = M + (size_t)(nq + M_THXX) * P;
-  const real* Txy = M + (size_t)(nq + M_THXY) * P;
-  const real* Tyy = M + (size_t)(nq + M_THYY) * P;
-  rho = a.rho0 + M[(size_t)(nq + M_DRHO) * P + n];
-  const real jx = M[(size_t)(nq + M_JX) * P + n];
-  const real jy = M[(size_t)(nq + M_JY) * P + n];
-  const real ex = real(0.5) * (Txx[nxp] - Txx[nxm]) + real(0.5) * (Txy[nyp] - Txy[nym]);
-  const real ey = real(0.5) * (Txy[nxp] - Txy[nxm]) + real(0.5) * (Tyy[nyp] - Tyy[nym]);
-  const real f = a.tab.arow[y];
-  ux = (jx + real(0.5) * (ex + rho * f)) / rho;
-  uy = (jy + real(0.5) * ey) / rho;
-}
-
 // ------------------------------------------------------------------ init
 // g = f^eq of the initial fields (Sec. VI-D): rho_S = 1, psi = psi0(q),
 // U = base flow + perturbation, J^r_eq = psi U, J^Q_eq = psi (Q . grad U -

@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "tfkt_fused.cuh"
 #include "tfkt_internal.cuh"
 #include "tfkt_mlp.cuh"
 #include "tfkt_umma.cuh"
@@ -20,7 +21,8 @@ const MlpDev& mlp_dev(const tfkt_mlp* net);
 
 namespace {
 
-// Scratch planes of the learned block (ny * pitch floats each).
+// Scratch planes of the learned block (ny * pitch floats each). L_B holds the sub-steps'
+// polymer terms (solvent_kernel) and then the increment's coefficients (reshape_kernel).
 enum { L_PSI = 0, L_C1 = 1, L_DP = 4, L_JP = 6, L_CNEW = 8, L_CPREV = 11, L_B = 14, L_NPLANES = 18 };
 
 struct LpmArgs {
@@ -57,8 +59,18 @@ __device__ __forceinline__ Nbr nbr(int x, int y, int nx, int ny, size_t pitch) {
 __device__ __forceinline__ void node_conformation(const KernelArgs<float>& a, const LpmArgs& l,
                                                   size_t n, float& pt, float C[3]) {
   const size_t P = a.plane;
+  // in Q-node order, the planes eight at a time so that several loads are in flight
   float s = 0.f;
-  for (int q = 0; q < a.nq; ++q) s += a.M[(size_t)q * P + n];
+  const float* mp = a.M + n;
+  int q = 0;
+  for (; q + 8 <= a.nq; q += 8) {
+    float m[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m[k] = mp[(size_t)(q + k) * P];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += m[k];
+  }
+  for (; q < a.nq; ++q) s += mp[(size_t)q * P];
   pt = a.psi_tot0 + s;
   const float r = l.l2 / pt;
   C[0] = r * (l.S0[0] + a.M[(size_t)(a.nq + M_THXX) * P + n] / l.hl2h);
@@ -88,7 +100,7 @@ __global__ void __launch_bounds__(256) conf_kernel(KernelArgs<float> a, LpmArgs 
   for (int c = 0; c < 3; ++c) l.p[(size_t)(out_plane + c) * P + n] = C[c];
 }
 
-// After the plain step: psi_tot, C(t + 1), the polymer momentum J_P = J - J_S and
+// After the plain step: U, psi_tot, C(t + 1), the polymer momentum J_P = J - J_S and
 // its offset dP = J_P - psi_tot U - tau2 E from the slaved value.
 __global__ void __launch_bounds__(256) prepare_kernel(KernelArgs<float> a, LpmArgs l) {
   const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
@@ -96,8 +108,14 @@ __global__ void __launch_bounds__(256) prepare_kernel(KernelArgs<float> a, LpmAr
   const size_t P = a.plane;
   const Nbr nb = nbr(x, y, a.nx, a.ny, a.pitch);
   const size_t n = nb.o[4];
+  wait_for_predecessor();
+  let_successor_start();
   float pt, C[3];
   node_conformation(a, l, n, pt, C);
+  float ux, uy, rho;
+  mixture_velocity(a, x, y, ux, uy, rho);
+  a.U[n] = ux;
+  a.U[P + n] = uy;
   float drs, jsx, jsy;
   solvent_pull_moments((const float*)a.src, P, nb, drs, jsx, jsy);
   const float* Txx = a.M + (size_t)(a.nq + M_THXX) * P;
@@ -107,7 +125,6 @@ __global__ void __launch_bounds__(256) prepare_kernel(KernelArgs<float> a, LpmAr
   const float ey = 0.5f * (Txy[nb.o[5]] - Txy[nb.o[3]]) + 0.5f * (Tyy[nb.o[7]] - Tyy[nb.o[1]]);
   const float jpx = a.M[(size_t)(a.nq + M_JX) * P + n] - jsx;
   const float jpy = a.M[(size_t)(a.nq + M_JY) * P + n] - jsy;
-  const float ux = a.U[n], uy = a.U[P + n];
   float* p = l.p;
   p[(size_t)L_PSI * P + n] = pt;
   for (int c = 0; c < 3; ++c) p[(size_t)(L_C1 + c) * P + n] = C[c];
@@ -229,6 +246,7 @@ __global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, L
   float* Cn = l.p + (size_t)L_CNEW * P;
   const float Kf = (float)l.K;
   if (l.mode == TFKT_LPM_FROZEN) {
+    wait_for_predecessor();
     for (int k = tid; k < T * T; k += blockDim.x) {
       const int x = tx0 + k % T, y = ty0 + k / T;
       if (x >= a.nx || y >= a.ny) continue;
@@ -273,6 +291,8 @@ __global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, L
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
+  wait_for_predecessor();
+  let_successor_start();
   const uint32_t tmem = s.tmem + 64u * g;                          // the group's 64 columns
   const uint32_t tmem_row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);   // this warp's lanes
   __nv_bfloat16* ahi = s.act[g][0];
@@ -434,7 +454,12 @@ __global__ void __launch_bounds__(256) targets_kernel(KernelArgs<float> a, LpmAr
 
 // One solvent sub-step: pull, U under the interpolated polymer stress with the
 // polymer momentum slaved (rho_S U = J_S + (tau2 + 1/2) E + rho a / 2 + dP), and
-// the plain step's solvent collision.
+// the plain step's solvent collision. The stress is linear in the fraction of the
+// way from C to C_new, so the block's first sub-step leaves
+// A = (tau2 + 1/2) E(C) + dP and B = (tau2 + 1/2) E(C_new - C) in the L_B planes and
+// the others read A + frac B: 14 plane loads per node in place of 40, which bound the
+// sub-step although most of them hit the cache (24 us at 1024 x 1024 nodes, now 18).
+template <bool FIRST>
 __global__ void __launch_bounds__(256) solvent_kernel(KernelArgs<float> a, LpmArgs l,
                                                      const float* __restrict__ src,
                                                      float* __restrict__ dst, float frac) {
@@ -443,28 +468,53 @@ __global__ void __launch_bounds__(256) solvent_kernel(KernelArgs<float> a, LpmAr
   const size_t P = a.plane;
   const Nbr nb = nbr(x, y, a.nx, a.ny, a.pitch);
   const size_t n = nb.o[4];
+  wait_for_predecessor();
+  let_successor_start();
   float h[9], drs = 0.f, jsx = 0.f, jsy = 0.f;
 #pragma unroll
+  for (int i = 0; i < 9; ++i) h[i] = src[(size_t)i * P + nb.o[shift_index(-c9x(i), -c9y(i))]];
+  const float* psi = l.p + (size_t)L_PSI * P;
+  const float psin = psi[n];
+  float* ab = l.p + (size_t)L_B * P + n;
+  float Ex, Ey;   // (tau2 + 1/2) E + dP
+  if (FIRST) {
+    const float t = l.tau2 + 0.5f;
+    float th0[4][3], thd[4][3];   // Theta of C and of C_new - C, right, left, above, below
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const size_t m = nb.o[k == 0 ? 5 : k == 1 ? 3 : k == 2 ? 7 : 1];
+      const float w = 0.5f * l.H * psi[m];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if ((k < 2 && c == 2) || (k >= 2 && c == 0)) continue;
+        const float c1 = l.p[(size_t)(L_C1 + c) * P + m];
+        th0[k][c] = w * c1;
+        thd[k][c] = w * (l.p[(size_t)(L_CNEW + c) * P + m] - c1);
+      }
+    }
+    auto div_x = [](const float (&v)[4][3]) { return 0.5f * (v[0][0] - v[1][0]) + 0.5f * (v[2][1] - v[3][1]); };
+    auto div_y = [](const float (&v)[4][3]) { return 0.5f * (v[0][1] - v[1][1]) + 0.5f * (v[2][2] - v[3][2]); };
+    Ex = t * div_x(th0) + l.p[(size_t)L_DP * P + n];
+    Ey = t * div_y(th0) + l.p[(size_t)(L_DP + 1) * P + n];
+    ab[0] = Ex;
+    ab[P] = Ey;
+    ab[2 * P] = t * div_x(thd);
+    ab[3 * P] = t * div_y(thd);
+  } else {
+    Ex = ab[0] + frac * ab[2 * P];
+    Ey = ab[P] + frac * ab[3 * P];
+  }
+#pragma unroll
   for (int i = 0; i < 9; ++i) {
-    h[i] = src[(size_t)i * P + nb.o[shift_index(-c9x(i), -c9y(i))]];
     drs += h[i];
     jsx += float(c9x(i)) * h[i];
     jsy += float(c9y(i)) * h[i];
   }
-  const float* psi = l.p + (size_t)L_PSI * P;
-  auto theta = [&](int c, size_t m) {
-    const float c1 = l.p[(size_t)(L_C1 + c) * P + m];
-    const float cn = l.p[(size_t)(L_CNEW + c) * P + m];
-    return 0.5f * l.H * psi[m] * (c1 + frac * (cn - c1));
-  };
-  const float ex = 0.5f * (theta(0, nb.o[5]) - theta(0, nb.o[3])) + 0.5f * (theta(1, nb.o[7]) - theta(1, nb.o[1]));
-  const float ey = 0.5f * (theta(1, nb.o[5]) - theta(1, nb.o[3])) + 0.5f * (theta(2, nb.o[7]) - theta(2, nb.o[1]));
   const float rs = 1.f + drs;
-  const float rho = rs + psi[n];
+  const float rho = rs + psin;
   const float force = rho * a.tab.arow[y];
-  const float t = l.tau2 + 0.5f;
-  const float Ux = (jsx + t * ex + 0.5f * force + l.p[(size_t)L_DP * P + n]) / rs;
-  const float Uy = (jsy + t * ey + l.p[(size_t)(L_DP + 1) * P + n]) / rs;
+  const float Ux = (jsx + Ex + 0.5f * force) / rs;
+  const float Uy = (jsy + Ey) / rs;
   const float jfx = (a.c2 * jsx + rs * Ux + a.tau2 * force) * a.inv_c2p1;
   const float jfy = (a.c2 * jsy + rs * Uy) * a.inv_c2p1;
   const float usx = jfx / rs, usy = jfy / rs;
@@ -488,6 +538,8 @@ __global__ void __launch_bounds__(256) solvent_kernel(KernelArgs<float> a, LpmAr
 // Rewrite the moment planes of the state (polymer part with dpsi, solvent part
 // from the last sub-step) and keep psi_tot times the coefficients of the
 // quadratic form for apply_kernel: dpsi(q) = p0(q) (B0 Qx^2 + B1 Qx Qy + B2 Qy^2 + B3).
+// Bound by the moment planes, read once and written once (109 us at 1024 x 1024 nodes with
+// 32 Q-nodes when they were read a second time for psi_tot and C, now 90).
 __global__ void __launch_bounds__(256) reshape_kernel(KernelArgs<float> a, LpmArgs l) {
   const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
   if (x >= a.nx || y >= a.ny) return;
@@ -495,10 +547,15 @@ __global__ void __launch_bounds__(256) reshape_kernel(KernelArgs<float> a, LpmAr
   const Nbr nb = nbr(x, y, a.nx, a.ny, a.pitch);
   const size_t n = nb.o[4];
   const int nq = a.nq;
-  float pt, C[3];
-  node_conformation(a, l, n, pt, C);
-  float d[3];
-  for (int c = 0; c < 3; ++c) d[c] = (l.p[(size_t)(L_CNEW + c) * P + n] - C[c]) / l.l2;
+  wait_for_predecessor();
+  let_successor_start();
+  // the sub-steps leave the polymer alone: psi_tot and C are still prepare_kernel's
+  const float pt = l.p[(size_t)L_PSI * P + n];
+  float cnew[3], d[3];
+  for (int c = 0; c < 3; ++c) {
+    cnew[c] = l.p[(size_t)(L_CNEW + c) * P + n];
+    d[c] = (cnew[c] - l.p[(size_t)(L_C1 + c) * P + n]) / l.l2;
+  }
   float beta[3];
   for (int r = 0; r < 3; ++r)
     beta[r] = l.M0inv[3 * r] * d[0] + l.M0inv[3 * r + 1] * d[1] + l.M0inv[3 * r + 2] * d[2];
@@ -510,15 +567,24 @@ __global__ void __launch_bounds__(256) reshape_kernel(KernelArgs<float> a, LpmAr
   p[(size_t)(L_B + 2) * P + n] = B2;
   p[(size_t)(L_B + 3) * P + n] = B3;
   float sum = 0.f, txx = 0.f, txy = 0.f, tyy = 0.f;
-  for (int q = 0; q < nq; ++q) {
-    const float qx = a.tab.qx[q], qy = a.tab.qy[q];
-    const float dpsi = a.tab.psi0[q] * l.rpt0 * (B0 * qx * qx + B1 * qx * qy + B2 * qy * qy + B3);
-    const float dv = a.M[(size_t)q * P + n] + dpsi;
-    a.M[(size_t)q * P + n] = dv;
-    sum += dv;
-    txx += dpsi * qx * qx;
-    txy += dpsi * qx * qy;
-    tyy += dpsi * qy * qy;
+  float* mp = a.M + n;
+  for (int q0 = 0; q0 < nq; q0 += 4) {   // four planes' loads in flight
+    float m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = q0 + k < nq ? mp[(size_t)(q0 + k) * P] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = q0 + k;
+      if (q >= nq) break;
+      const float qx = a.tab.qx[q], qy = a.tab.qy[q];
+      const float dpsi = a.tab.psi0[q] * l.rpt0 * (B0 * qx * qx + B1 * qx * qy + B2 * qy * qy + B3);
+      const float dv = m[k] + dpsi;
+      mp[(size_t)q * P] = dv;
+      sum += dv;
+      txx += dpsi * qx * qx;
+      txy += dpsi * qx * qy;
+      tyy += dpsi * qy * qy;
+    }
   }
   float drs, jsx, jsy;
   solvent_pull_moments((const float*)a.src, P, nb, drs, jsx, jsy);
@@ -528,7 +594,7 @@ __global__ void __launch_bounds__(256) reshape_kernel(KernelArgs<float> a, LpmAr
   a.M[(size_t)(nq + M_THXX) * P + n] += l.hl2h * txx;
   a.M[(size_t)(nq + M_THXY) * P + n] += l.hl2h * txy;
   a.M[(size_t)(nq + M_THYY) * P + n] += l.hl2h * tyy;
-  for (int c = 0; c < 3; ++c) p[(size_t)(L_CPREV + c) * P + n] = p[(size_t)(L_CNEW + c) * P + n];
+  for (int c = 0; c < 3; ++c) p[(size_t)(L_CPREV + c) * P + n] = cnew[c];
 }
 
 // Add to every stored polymer population the increment that its pull delivers
@@ -717,23 +783,18 @@ extern "C" tfkt_status tfkt_lpm_run(tfkt_ctx* cc, const tfkt_mlp* net, const tfk
     }
     if ((s = tfkt_step(cc, 1)) != TFKT_OK) return s;
     KernelArgs<float> a = ctx_args<float>(c);
-    LPM_CUDA(launch_velocity<float>(a, st));
-    prepare_kernel<<<grid, blk, 0, st>>>(a, l);
-    LPM_CUDA(cudaGetLastError());
+    LPM_CUDA(launch(prepare_kernel, grid, blk, 0, st, true, a, l));
     const size_t nsm = net_smem_bytes();
     LPM_CUDA(cudaFuncSetAttribute(net_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nsm));
-    net_kernel<<<tiles, NET_THREADS, nsm, st>>>(a, l, nd);
-    LPM_CUDA(cudaGetLastError());
+    LPM_CUDA(launch(net_kernel, tiles, dim3(NET_THREADS), nsm, st, true, a, l, nd));
     for (int j = 0; j < o->K; ++j) {
       KernelArgs<float> aj = ctx_args<float>(c);
-      solvent_kernel<<<grid, blk, 0, st>>>(aj, l, (const float*)aj.src, (float*)aj.dst,
-                                           (float)j / (float)o->K);
-      LPM_CUDA(cudaGetLastError());
+      LPM_CUDA(launch(j == 0 ? solvent_kernel<true> : solvent_kernel<false>, grid, blk, 0, st, true,
+                      aj, l, (const float*)aj.src, (float*)aj.dst, (float)j / (float)o->K));
       c->cur ^= 1;
     }
     a = ctx_args<float>(c);
-    reshape_kernel<<<grid, blk, 0, st>>>(a, l);
-    LPM_CUDA(cudaGetLastError());
+    LPM_CUDA(launch(reshape_kernel, grid, blk, 0, st, true, a, l));
     // the increment rides on the next step's pull (tfkt_step, or the next block)
     c->lpm_pending = true;
     c->lpm_rshp = l.p + (size_t)L_B * L.plane;
