@@ -205,9 +205,9 @@ struct NetSmem {
   __nv_bfloat16 w1[NH * NET_K1];                 // K-major operand layout, in >= NIN zero
   __nv_bfloat16 w2[NH * NH];
   __nv_bfloat16 act[NET_GROUPS][2][128 * NH];    // per group: high part and remainder rows
-  float w3[NOUT][NH];
-  float b1[NH], b2[NH], b3[NOUT];
-  float mx[NIN], rsx[NIN], mt[NOUT], st[NOUT];
+  alignas(16) float w3[NOUT][NH];                // (aligned: read four at a time)
+  float b1[NH], b2[NH], mx[NIN], rsx[NIN];
+  float b3[NOUT], mt[NOUT], st[NOUT];
   uint64_t mbar[NET_GROUPS];
   uint32_t tmem;
 };
@@ -219,23 +219,24 @@ __host__ __device__ constexpr uint32_t op_offset(int r, int k, uint32_t sbo) {
          (uint32_t)(k % 8) * 2u;
 }
 
-// Writes 8 values v[8 c .. 8 c + 7] of row r, split into high part and remainder,
-// as one 16-byte chunk of each operand.
+// Writes the values of row r from column 8 c0 on, eight at a time, split into high part
+// and remainder, as one 16-byte chunk of each operand.
 __device__ __forceinline__ void write_row(__nv_bfloat16* hi, __nv_bfloat16* lo, int r, const float* v,
-                                          int nchunks, uint32_t sbo) {
+                                          int c0, int nchunks, uint32_t sbo) {
+#pragma unroll
   for (int c = 0; c < nchunks; ++c) {
     uint32_t h[4], l[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) tc_split(v[8 * c + 2 * j], v[8 * c + 2 * j + 1], h[j], l[j]);
-    const uint32_t off = op_offset(r, 8 * c, sbo);
+    const uint32_t off = op_offset(r, 8 * (c0 + c), sbo);
     *reinterpret_cast<uint4*>(reinterpret_cast<char*>(hi) + off) = make_uint4(h[0], h[1], h[2], h[3]);
     *reinterpret_cast<uint4*>(reinterpret_cast<char*>(lo) + off) = make_uint4(l[0], l[1], l[2], l[3]);
   }
 }
 
-__global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, LpmArgs l, MlpDev net) {
+__global__ void __launch_bounds__(NET_THREADS, 2) net_kernel(KernelArgs<float> a, LpmArgs l, MlpDev net) {
   extern __shared__ __align__(16) unsigned char net_smem[];
-  __shared__ float red[NET_THREADS];
+  __shared__ float red[NET_THREADS / 32];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int g = tid >> 7, r = tid & 127;         // group, row (node) within the group
   const size_t P = a.plane;
@@ -305,9 +306,8 @@ __global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, L
   uint32_t phase = 0;
   bool failed = false;
   float worst = 0.f;
-  const int npass = (T * T + NET_THREADS - 1) / NET_THREADS;      // same count in both groups
-  for (int pass = 0; pass < npass; ++pass) {
-    const int k = pass * NET_THREADS + g * 128 + r;
+  for (int k0 = 128 * g; k0 < T * T; k0 += NET_THREADS) {         // a group goes by itself
+    const int k = k0 + r;
     const int x = tx0 + k % T, y = ty0 + k / T;
     const bool ok = k < T * T && x < a.nx && y < a.ny;
     float f[NET_K1], cdep[3] = {0.f, 0.f, 0.f};
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, L
 #pragma unroll
     for (int i = NIN; i < NET_K1; ++i) f[i] = 0.f;
     // layer 1: [128 x 48] x [48 x 64]
-    write_row(ahi, alo, r, f, NET_K1 / 8, NET_SBO1);
+    write_row(ahi, alo, r, f, 0, NET_K1 / 8, NET_SBO1);
     umma::fence_proxy_async();
     umma::fence_before_sync();
     umma::bar_sync(1 + g, 128);
@@ -340,21 +340,20 @@ __global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, L
     const bool done1 = umma::mbar_wait(&s.mbar[g], phase, polls);
     phase ^= 1u;
     umma::fence_after_sync();
-    float h[NH];
-    if (done1) {
-      float v[32];
+    // layer 2: [128 x 64] x [64 x 64] (the layer-1 operands are consumed: reuse them)
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
+    for (int half = 0; half < 2; ++half) {
+      float v[32];
+      if (done1) {
         umma::ld_x32(tmem_row + 32u * half, v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) h[32 * half + j] = gelu(v[j] + s.b1[32 * half + j]);
-      }
-    } else {
+        for (int j = 0; j < 32; ++j) v[j] = gelu(v[j] + s.b1[32 * half + j]);
+      } else {
 #pragma unroll
-      for (int j = 0; j < NH; ++j) h[j] = 0.f;
+        for (int j = 0; j < 32; ++j) v[j] = 0.f;
+      }
+      write_row(ahi, alo, r, v, 4 * half, 4, NET_SBO2);
     }
-    // layer 2: [128 x 64] x [64 x 64] (the layer-1 operands are consumed: reuse them)
-    write_row(ahi, alo, r, h, NH / 8, NET_SBO2);
     umma::fence_proxy_async();
     umma::fence_before_sync();
     umma::bar_sync(1 + g, 128);
@@ -410,13 +409,14 @@ __global__ void __launch_bounds__(NET_THREADS) net_kernel(KernelArgs<float> a, L
     worst = __int_as_float(0x7f800000);
     if (r == 0) umma::mbar_wait(&s.mbar[g], phase ^ 1u, polls);
   }
-  red[tid] = worst;
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, m));
+  if ((tid & 31) == 0) red[warp] = worst;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (tid < w) red[tid] = fmaxf(red[tid], red[tid + w]);
-    __syncthreads();
-  }
-  if (!(red[0] <= l.threshold)) {      // NaN falls back too
+  worst = red[0];
+#pragma unroll
+  for (int w = 1; w < NET_THREADS / 32; ++w) worst = fmaxf(worst, red[w]);
+  if (!(worst <= l.threshold)) {      // NaN falls back too
     if (tid == 0) atomicAdd(l.counter, 1);
     for (int k = tid; k < T * T; k += blockDim.x) {
       const int x = tx0 + k % T, y = ty0 + k / T;
