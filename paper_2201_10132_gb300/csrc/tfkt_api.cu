@@ -432,10 +432,11 @@ tfkt_status init_state(Ctx* c, const double* perturb) {
   }
   a.perturb = dpert;
   a.dst = (char*)c->ws.base + c->ws.off_pop[0];
-  TFKT_CUDA(c, launch_init<real, S>(a, c->stream));   // populations and their moments
   // the Q-split kernels sum the moments in another order: take theirs from the start,
   // so that a step gives the same bits whether or not its moments were formed again
-  if (!c->fused || c->split) TFKT_CUDA(c, launch_moments<real, S>(a, c->stream));
+  const bool split = !c->fused || c->split;
+  TFKT_CUDA(c, launch_init<real, S>(a, !split, c->stream));
+  if (split) TFKT_CUDA(c, launch_moments<real, S>(a, c->stream));
   c->cur = 0;
   c->m_valid = true;
   TFKT_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -323,7 +323,7 @@ int moment_warps(const Lattice& L);   // KernelArgs::mom_warps of a run
 
 // Launchers (tfkt_kernels.cu). Each returns the launch status.
 template <typename real, typename S>
-cudaError_t launch_init(const KernelArgs<real>& a, cudaStream_t s);
+cudaError_t launch_init(const KernelArgs<real>& a, bool moments, cudaStream_t s);
 template <typename real>
 cudaError_t launch_velocity(const KernelArgs<real>& a, cudaStream_t s);
 template <typename real>

@@ -43,8 +43,9 @@ __device__ __forceinline__ Offsets node_offsets(int x, int y, int nx, int ny, si
 // For the same reason the pulled populations of a node are its own stored
 // values: the kernel also writes the state's moment planes M, rebuilding each
 // value from its stored form, so the moments need no second pass over the
-// populations.
-template <typename real, typename S>
+// populations. Contexts whose steps sum the moments in another order (the Q-split
+// kernels) leave the sums out and run the moments pass.
+template <typename real, typename S, bool MOMENTS>
 __global__ void __launch_bounds__(256) init_kernel(KernelArgs<real> a) {
   using SS = SolventT<S>;
   SS* __restrict__ sdst = solvent_planes<S>(a.dst, a.plane, a.nq);
@@ -77,10 +78,12 @@ __global__ void __launch_bounds__(256) init_kernel(KernelArgs<real> a) {
     const real h = real(w9(i)) * (real(3) * cu + real(4.5) * cu * cu - real(1.5) * usq);
     const SS st = to_store<SS>(h);
     sdst[(size_t)i * P + off.o[shift_index(-c9x(i), -c9y(i))]] = st;
-    const real v = from_store<real>(st);
-    drho += v;
-    jx += real(c9x(i)) * v;
-    jy += real(c9y(i)) * v;
+    if (MOMENTS) {
+      const real v = from_store<real>(st);
+      drho += v;
+      jx += real(c9x(i)) * v;
+      jy += real(c9y(i)) * v;
+    }
   }
   real txx = 0, txy = 0, tyy = 0;
   for (int q = 0; q < a.nq; ++q) {
@@ -100,11 +103,14 @@ __global__ void __launch_bounds__(256) init_kernel(KernelArgs<real> a) {
       const int p = e >= 0 ? e : ~e;
       const S st = to_store<S>((h - a.tab.delta[q * 25 + i]) * a.pscale);
       dst[(size_t)p * P + o] = st;
-      const real v = from_store<real>(st) * a.pinv + a.tab.delta[q * 25 + i];
-      dpsi += v;
-      rx += real(c.rx) * v;
-      ry += real(c.ry) * v;
+      if (MOMENTS) {
+        const real v = from_store<real>(st) * a.pinv + a.tab.delta[q * 25 + i];
+        dpsi += v;
+        rx += real(c.rx) * v;
+        ry += real(c.ry) * v;
+      }
     }
+    if (!MOMENTS) continue;
     a.M[(size_t)q * P + off.o[4]] = dpsi;
     drho += dpsi;
     jx += rx;
@@ -113,6 +119,7 @@ __global__ void __launch_bounds__(256) init_kernel(KernelArgs<real> a) {
     txy += dpsi * Fx * Qy;
     tyy += dpsi * Fy * Qy;
   }
+  if (!MOMENTS) return;
   const size_t n = off.o[4];
   const int nq = a.nq;
   a.M[(size_t)(nq + M_DRHO) * P + n] = drho;
@@ -546,8 +553,10 @@ inline dim3 node_grid(int nx, int ny) { return dim3((nx + TX - 1) / TX, (ny + TY
 }  // namespace
 
 template <typename real, typename S>
-cudaError_t launch_init(const KernelArgs<real>& a, cudaStream_t s) {
-  init_kernel<real, S><<<node_grid(a.nx, a.ny), dim3(TX, TY), 0, s>>>(a);
+cudaError_t launch_init(const KernelArgs<real>& a, bool moments, cudaStream_t s) {
+  const dim3 grid = node_grid(a.nx, a.ny), block(TX, TY);
+  if (moments) init_kernel<real, S, true><<<grid, block, 0, s>>>(a);
+  else init_kernel<real, S, false><<<grid, block, 0, s>>>(a);
   return cudaGetLastError();
 }
 template <typename real>
@@ -590,7 +599,7 @@ cudaError_t launch_diag(const KernelArgs<real>& a, double* partials, int nblocks
 }
 
 #define TFKT_INSTANTIATE_POP(real, S)                                                          \
-  template cudaError_t launch_init<real, S>(const KernelArgs<real>&, cudaStream_t);           \
+  template cudaError_t launch_init<real, S>(const KernelArgs<real>&, bool, cudaStream_t);     \
   template cudaError_t launch_populations<real, S>(const KernelArgs<real>&, double*,          \
                                                    cudaStream_t);
 #define TFKT_INSTANTIATE(real)                                                                 \
