@@ -30,7 +30,7 @@ struct MlpDev {
 // it leaves in a t (weighted minimax by Lawson's iteration, 3e-9); beyond, |z| P falls on
 // and t underflows. The largest error against FP64 over |z| < 8 is 2.4e-7 (half an ulp of
 // the result) and the rms error 3.9e-8; 0.5 z (1 + erff(z / sqrt 2)) has 4.5e-7 and
-// 5.0e-8. 13 instructions where erff with its branch takes over twice as many: net_kernel
+// 5.0e-8. 14 instructions where erff with its branch takes over twice as many: net_kernel
 // at 1024 x 1024 nodes took 253 us with it and takes 203.
 // The derivative (training) needs Phi itself, for which erff is the closer one.
 __device__ constexpr float GELU_P[10] = {
@@ -43,7 +43,7 @@ __device__ __forceinline__ float gelu(float z) {
   for (int k = 8; k >= 0; --k) p = fmaf(p, a, GELU_P[k]);
   float t;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(p, a, -1.0f)));
-  return fmaf(-t, a, fmaxf(z, 0.0f));
+  return fmaf(-t, fminf(a, 3e38f), fmaxf(z, 0.0f));   // 0 infinity is no NaN
 }
 
 // ---- Tensor-core forward pass: mma.sync m16n8k16, bfloat16 operands, FP32
