@@ -143,90 +143,75 @@ __global__ void __launch_bounds__(256) velocity_kernel(KernelArgs<real> a) {
 }
 
 // Per-node observables (Sec. VII): rho_S, psi_tot, U, C, Theta, Q_rms, vorticity, the
-// ones in `mask`. The sums over the Q-nodes need more than FP32: the second moments
-// behind C_xy and Theta_xy cancel between Q-nodes of opposite sign, which FP32 sums
-// would resolve only to ~1e-7 of the diagonal ones. FP64 contexts sum in FP64.
-// FP32 contexts sum in pairs of floats without any FP64 operation: each term's
-// product and each sum keep their rounding error (Dekker 1971; Dot2 of Ogita, Rump
-// and Oishi 2005), so a sum is as if formed in 48 bits, far below the rounding of the
-// planes themselves; quotient, root and differences follow in such pairs, and a node
-// with a non-finite or overflowing value is formed again in FP64. FP64 arithmetic, 2
-// lanes per clock and SM, bound the kernel: rho_s, U and C of 1024 x 1024 nodes with 32
-// Q-nodes took 767 us (the velocity pass included), now 161; with 9 Q-nodes 284 and 75.
-// What is left is the FP32 issue rate, about 50 instructions per Q-node.
+// ones in `mask`, in FP64 from sums over the Q-nodes: the second moments behind C_xy and
+// Theta_xy cancel between Q-nodes of opposite sign, which FP32 sums would resolve only
+// to ~1e-7 of the diagonal ones. FP64 arithmetic, 2 lanes per clock and SM, would bound
+// the kernel of FP32 contexts: rho_s, U and C of 1024 x 1024 nodes with 32 Q-nodes took
+// 767 us (the velocity pass included). There the sums of psi, psi Q Q run over the stored
+// deviations in three floats each, which keep what every product and sum rounds away
+// (two-sum: Knuth; cascaded: Ogita, Rump and Oishi 2005), and meet the sums of psi0 in
+// FP64 at the end: 247 us; with 9 Q-nodes 284 and 159. Two floats per sum (161 and
+// 75 us) leave 2^-48 of a sum, more than FP64 sums do; three leave less (2^-70), so the
+// result is rounded three times where an FP64 sum is at every Q-node. Theta (the spring
+// force is no short binary fraction) and nodes with non-finite or overflowing values are
+// summed in FP64. What bounds it: the FP32 issue rate, about 80 instructions per Q-node,
+// and about 40 FP64 operations per node after the sums.
 constexpr uint32_t FIELDS_PSUM = (1u << TFKT_F_RHO_S) | (1u << TFKT_F_PSI_TOT) | (1u << TFKT_F_CXX) |
                                  (1u << TFKT_F_CXY) | (1u << TFKT_F_CYY) | (1u << TFKT_F_QRMS);
 constexpr uint32_t FIELDS_CONF = (1u << TFKT_F_CXX) | (1u << TFKT_F_CXY) | (1u << TFKT_F_CYY) |
                                  (1u << TFKT_F_QRMS);
 constexpr uint32_t FIELDS_STRESS = (1u << TFKT_F_THXX) | (1u << TFKT_F_THXY) | (1u << TFKT_F_THYY);
 
-// A sum kept as a pair of floats: add (p + pl) (w + wl), p and w the leading parts.
-struct PairSum {
-  float hi = 0, lo = 0;
-  __device__ __forceinline__ void add(float p, float pl, float w, float wl) {
-    const float x = __fmul_rn(p, w);
-    const float e = __fmaf_rn(p, w, -x);
-    const float s = __fadd_rn(hi, x);
-    const float b = __fsub_rn(s, hi);
-    const float r = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
-    hi = s;
-    lo = __fadd_rn(lo, __fmaf_rn(pl, w, __fmaf_rn(p, wl, __fadd_rn(e, r))));
+// A sum kept in three floats.
+struct ExactSum {
+  float hi = 0, lo = 0, rest = 0;
+  // a += x; returns what the addition rounds away (exact)
+  static __device__ __forceinline__ float two_sum(float& a, float x) {
+    const float s = __fadd_rn(a, x), b = __fsub_rn(s, a);
+    const float r = __fadd_rn(__fsub_rn(a, __fsub_rn(s, b)), __fsub_rn(x, b));
+    a = s;
+    return r;
   }
+  __device__ __forceinline__ void add(float x) {
+    rest = __fadd_rn(rest, two_sum(lo, two_sum(hi, x)));
+  }
+  __device__ __forceinline__ void add(float m, float w) {   // m w: a product and its rounding error
+    const float x = __fmul_rn(m, w);
+    add(x);
+    rest = __fadd_rn(rest, two_sum(lo, __fmaf_rn(m, w, -x)));
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + ((double)lo + (double)rest); }
 };
 
-// Arithmetic on such pairs (about 46 bits), as far as the fields need it.
-struct Two {
-  float h, l;
-  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-};
-__device__ __forceinline__ Two two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
-}
-__device__ __forceinline__ Two two_add(Two a, Two b) {
-  const Two s = two_sum(a.h, b.h);
-  return two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ Two two_scale(Two a, float f) {
-  const float p = __fmul_rn(a.h, f);
-  return {p, __fmaf_rn(a.l, f, __fmaf_rn(a.h, f, -p))};
-}
-__device__ __forceinline__ Two two_div(Two a, Two b) {
-  const float q = a.h / b.h;
-  const float r = __fmaf_rn(-q, b.l, __fadd_rn(__fmaf_rn(-q, b.h, a.h), a.l));
-  return {q, r / b.h};
-}
-__device__ __forceinline__ Two two_sqrt(Two a) {   // a.h > 0
-  const float q = sqrtf(a.h);
-  return {q, __fadd_rn(__fmaf_rn(-q, q, a.h), a.l) / __fadd_rn(q, q)};
-}
-
-// Weights of a Q-node in the pair sums, staged once per block: Q Q and F Q (xx, xy,
-// yy) and what their rounding leaves.
+// Staged once per block: the weights Q Q (xx, xy, yy) of the Q-nodes, exact in FP32
+// (quarters of small integers), behind the sums of psi0 with the weights 1, Q Q.
 struct FieldRow {
-  float psi0, w[6], wl[6];
+  float w[3];
 };
+constexpr size_t FIELD_HEAD = 4 * sizeof(double);
 
-__device__ __forceinline__ void stage_field_rows(const KernelArgs<float>& a, FieldRow* row) {
+__device__ __forceinline__ void stage_field_rows(const KernelArgs<float>& a, double* s0, FieldRow* row) {
   for (int q = threadIdx.y * TX + threadIdx.x; q < a.nq; q += TX * TY) {
-    const float Q[2] = {a.tab.qx[q], a.tab.qy[q]}, F[2] = {a.tab.fx[q], a.tab.fy[q]};
-    FieldRow& r = row[q];
-    r.psi0 = a.tab.psi0[q];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {   // xx, xy, yy
-      const float q1 = Q[j / 2], f1 = F[j / 2], q2 = Q[(j + 1) / 2];
-      r.w[j] = __fmul_rn(q1, q2);
-      r.wl[j] = __fmaf_rn(q1, q2, -r.w[j]);
-      r.w[3 + j] = __fmul_rn(f1, q2);
-      r.wl[3 + j] = __fmaf_rn(f1, q2, -r.w[3 + j]);
-    }
+    const float Qx = a.tab.qx[q], Qy = a.tab.qy[q];
+    row[q] = {{Qx * Qx, Qx * Qy, Qy * Qy}};
   }
+  static_assert(TX == 32 && TY >= 4, "one warp per sum of psi0");
+  const int j = threadIdx.y;
+  if (j >= 4) return;
+  double s = 0;
+  for (int q = threadIdx.x; q < a.nq; q += 32) {
+    const float Qx = a.tab.qx[q], Qy = a.tab.qy[q];
+    s += double(a.tab.psi0[q]) * double(j == 0 ? 1.0f : j == 1 ? Qx * Qx : j == 2 ? Qx * Qy : Qy * Qy);
+  }
+#pragma unroll
+  for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  if (threadIdx.x == 0) s0[j] = s;
 }
 
-// s: psi_tot, then sum psi Q Q and sum psi F Q (xx, xy, yy), the latter two where asked.
-template <bool CONF, bool STRESS>
-__device__ __forceinline__ void pair_sums(const KernelArgs<float>& a, const FieldRow* row, size_t n,
-                                          PairSum (&s)[7]) {
+// s: sum of delta psi, then of delta psi Q Q (xx, xy, yy) where asked.
+template <bool CONF>
+__device__ __forceinline__ void exact_sums(const KernelArgs<float>& a, const FieldRow* row, size_t n,
+                                           ExactSum (&s)[4]) {
   const size_t P = a.plane;
   const float* mp = a.M + n;
   // the planes four at a time, so that several loads are in flight
@@ -237,16 +222,10 @@ __device__ __forceinline__ void pair_sums(const KernelArgs<float>& a, const Fiel
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       if (q0 + k >= a.nq) break;
-      const FieldRow& r = row[q0 + k];
-      const float p = __fadd_rn(r.psi0, m[k]);
-      const float b = __fsub_rn(p, r.psi0);
-      const float pl = __fadd_rn(__fsub_rn(r.psi0, __fsub_rn(p, b)), __fsub_rn(m[k], b));
-      s[0].add(p, pl, 1.0f, 0.0f);
+      s[0].add(m[k]);
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        if (CONF) s[1 + j].add(p, pl, r.w[j], r.wl[j]);
-        if (STRESS) s[4 + j].add(p, pl, r.w[3 + j], r.wl[3 + j]);
-      }
+      for (int j = 0; j < 3; ++j)
+        if (CONF) s[1 + j].add(m[k], row[q0 + k].w[j]);
     }
   }
 }
@@ -280,9 +259,11 @@ __global__ void __launch_bounds__(256) fields_kernel(KernelArgs<real> a, uint32_
   const bool sums = mask & (FIELDS_PSUM | FIELDS_STRESS);
   const bool conf = mask & FIELDS_CONF, stress = mask & FIELDS_STRESS;
   const int nq = a.nq;
+  double* s0 = reinterpret_cast<double*>(field_smem);
+  FieldRow* row = reinterpret_cast<FieldRow*>(field_smem + FIELD_HEAD);
   if constexpr (std::is_same<real, float>::value)
-    if (sums) {
-      stage_field_rows(a, reinterpret_cast<FieldRow*>(field_smem));
+    if (sums && !stress) {
+      stage_field_rows(a, s0, row);
       __syncthreads();
     }
   const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
@@ -296,79 +277,41 @@ __global__ void __launch_bounds__(256) fields_kernel(KernelArgs<real> a, uint32_
   const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
   const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y == a.ny - 1 ? 0 : y + 1;
   const bool vort = mask & (1u << TFKT_F_VORT);
-  bool done = false;
-  if constexpr (std::is_same<real, float>::value) {
-    // FP32 contexts: pairs of floats to the end, one FP64 addition per field
-    const FieldRow* row = reinterpret_cast<const FieldRow*>(field_smem);
-    PairSum ps[7];
-    if (conf && stress) pair_sums<true, true>(a, row, n, ps);
-    else if (conf) pair_sums<true, false>(a, row, n, ps);
-    else if (stress) pair_sums<false, true>(a, row, n, ps);
-    else if (sums) pair_sums<false, false>(a, row, n, ps);
-    Two s[7];
-    done = true;   // unless a sum left the range of FP32 or met a non-finite value
+  double s[7] = {};
+  bool done = !sums;
+  if constexpr (std::is_same<real, float>::value)
+    if (sums && !stress) {
+      ExactSum es[4];
+      if (conf) exact_sums<true>(a, row, n, es);
+      else exact_sums<false>(a, row, n, es);
+      done = true;   // unless a sum left the range of FP32 or met a non-finite value
 #pragma unroll
-    for (int j = 0; j < 7; ++j) {
-      s[j] = two_sum(ps[j].hi, ps[j].lo);
-      done = done && isfinite(ps[j].hi);
-    }
-    if (sums) {
-      f[TFKT_F_PSI_TOT] = s[0].value();
-      f[TFKT_F_RHO_S] = two_add(two_sum(a.rho0, drho), {-s[0].h, -s[0].l}).value();
-    }
-    if (conf) {
-      Two c[3] = {};
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        if (s[0].h != 0.0f) c[j] = two_div(two_scale(s[1 + j], a.l2), s[0]);
-      f[TFKT_F_CXX] = c[0].value();
-      f[TFKT_F_CXY] = c[1].value();
-      f[TFKT_F_CYY] = c[2].value();
-      if (mask & (1u << TFKT_F_QRMS)) {
-        const Two t = two_add(c[0], c[2]);
-        f[TFKT_F_QRMS] = t.h > 0.0f ? two_sqrt(t).value() : sqrt(t.value());
+      for (int j = 0; j < 4; ++j) {
+        s[j] = s0[j] + es[j].value();
+        done = done && isfinite(es[j].hi);
       }
-#pragma unroll
-      for (int j = 0; j < 3; ++j) done = done && isfinite(c[j].h);
     }
-    if (stress) {
-      const double hh = 0.5 * double(a.H) * double(a.l2);
-      f[TFKT_F_THXX] = hh * s[4].value();
-      f[TFKT_F_THXY] = hh * s[5].value();
-      f[TFKT_F_THYY] = hh * s[6].value();
-    }
-    if (vort) {
-      const Two d1 = two_sum(a.U[P + (size_t)y * a.pitch + xp], -a.U[P + (size_t)y * a.pitch + xm]);
-      const Two d2 = two_sum(a.U[(size_t)ym * a.pitch + x], -a.U[(size_t)yp * a.pitch + x]);
-      const Two w = two_add(d1, d2);
-      f[TFKT_F_VORT] = 0.5 * w.value();
-      done = done && isfinite(w.h);
-    }
+  if (!done) fp64_sums(a, n, conf, stress, s);
+  const double pt = s[0], l2 = a.l2, hh = 0.5 * double(a.H) * l2;
+  f[TFKT_F_RHO_S] = double(a.rho0) + double(drho) - pt;
+  f[TFKT_F_PSI_TOT] = pt;
+  if (conf) {
+    const double cxx = pt != 0 ? l2 * s[1] / pt : 0, cxy = pt != 0 ? l2 * s[2] / pt : 0,
+                 cyy = pt != 0 ? l2 * s[3] / pt : 0;
+    f[TFKT_F_CXX] = cxx;
+    f[TFKT_F_CXY] = cxy;
+    f[TFKT_F_CYY] = cyy;
+    if (mask & (1u << TFKT_F_QRMS)) f[TFKT_F_QRMS] = sqrt(cxx + cyy);
   }
-  if (!done) {
-    double s[7] = {};
-    if (sums) fp64_sums(a, n, conf, stress, s);
-    const double pt = s[0], l2 = a.l2, hh = 0.5 * double(a.H) * l2;
-    f[TFKT_F_RHO_S] = double(a.rho0) + double(drho) - pt;
-    f[TFKT_F_PSI_TOT] = pt;
-    if (conf) {
-      const double cxx = pt != 0 ? l2 * s[1] / pt : 0, cxy = pt != 0 ? l2 * s[2] / pt : 0,
-                   cyy = pt != 0 ? l2 * s[3] / pt : 0;
-      f[TFKT_F_CXX] = cxx;
-      f[TFKT_F_CXY] = cxy;
-      f[TFKT_F_CYY] = cyy;
-      if (mask & (1u << TFKT_F_QRMS)) f[TFKT_F_QRMS] = sqrt(cxx + cyy);
-    }
-    f[TFKT_F_THXX] = hh * s[4];
-    f[TFKT_F_THXY] = hh * s[5];
-    f[TFKT_F_THYY] = hh * s[6];
-    if (vort) {
-      const double duy_dx = 0.5 * (double(a.U[P + (size_t)y * a.pitch + xp]) -
-                                   double(a.U[P + (size_t)y * a.pitch + xm]));
-      const double dux_dy =
-          0.5 * (double(a.U[(size_t)yp * a.pitch + x]) - double(a.U[(size_t)ym * a.pitch + x]));
-      f[TFKT_F_VORT] = duy_dx - dux_dy;
-    }
+  f[TFKT_F_THXX] = hh * s[4];
+  f[TFKT_F_THXY] = hh * s[5];
+  f[TFKT_F_THYY] = hh * s[6];
+  if (vort) {
+    const double duy_dx = 0.5 * (double(a.U[P + (size_t)y * a.pitch + xp]) -
+                                 double(a.U[P + (size_t)y * a.pitch + xm]));
+    const double dux_dy =
+        0.5 * (double(a.U[(size_t)yp * a.pitch + x]) - double(a.U[(size_t)ym * a.pitch + x]));
+    f[TFKT_F_VORT] = duy_dx - dux_dy;
   }
   int slot = 0;
 #pragma unroll
@@ -566,7 +509,7 @@ cudaError_t launch_velocity(const KernelArgs<real>& a, cudaStream_t s) {
 }
 template <typename real>
 cudaError_t launch_fields(const KernelArgs<real>& a, uint32_t mask, double* out, cudaStream_t s) {
-  const size_t smem = sizeof(real) == 4 ? (size_t)a.nq * sizeof(FieldRow) : 0;   // at most 213 KB
+  const size_t smem = sizeof(real) == 4 ? FIELD_HEAD + (size_t)a.nq * sizeof(FieldRow) : 0;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(fields_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
