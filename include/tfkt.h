@@ -118,7 +118,7 @@ typedef struct tfkt_ctx tfkt_ctx;
 /* Kernels timed by tfkt_step_profiled. */
 enum {
   TFKT_K_MOMENTS = 0,  /* pull-read of all populations -> moment planes */
-  TFKT_K_STEP,         /* two-pass path (FP64 and up to 100 tiles where the grid is no multiple
+  TFKT_K_STEP,         /* two-pass path (FP64 and up to 152 tiles where the grid is no multiple
                           of the 32 x 8 tile, or too many Q-nodes for the fused kernel): pull,
                           collide and write of all populations */
   TFKT_K_FUSED,        /* fused path: pull, collide, write and next-step moments (the moments

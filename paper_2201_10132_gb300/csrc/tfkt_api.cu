@@ -152,11 +152,16 @@ double polymer_scale(const Lattice& L) {
 // step, with 32 Q-nodes: 61.8 against 12.1 at 64 x 64 nodes (16 tiles), 64 against 35
 // at 128 x 128 (64), 71.5 against 60 at 160 x 160 (100), 77.5 against 90 at 192 x 192
 // (144); with 9 Q-nodes 25.4 against 13.8 at 128 x 128, 26.8 against 16.2 at 160 x 160,
-// 36 against 57 at 256 x 256. The line is drawn at 100 tiles. A slab steps as its
-// whole run does, so the whole run's size decides.
-constexpr size_t SPLIT_TILES = 100;
+// 36 against 57 at 256 x 256. The line is drawn at 100 tiles. With partial tiles the
+// fused kernel takes about 90 us up to one tile per SM, whatever the tiles hold, and the
+// line is there: with 32, 52 and 9 Q-nodes 91, 182 and 30.7 against 71, 107 and 16.8 at
+// 161 x 161 nodes (126 tiles), 91, 178 and 31.0 against 84, 123 and 21.8 at 500 x 65
+// (144); 90, 187 and 31.5 against 108, 159 and 25.5 at 200 x 200 (175). A slab steps as
+// its whole run does, so the whole run's size decides.
+constexpr size_t SPLIT_TILES = 100, SPLIT_TILES_PARTIAL = 152;
 bool split_path(const Lattice& L) {
-  return L.precision == TFKT_FP64 || run_tiles(L) <= SPLIT_TILES;
+  const bool partial = L.nx % TX || (L.ny_global > 0 ? L.ny_global : L.ny) % TY;
+  return L.precision == TFKT_FP64 || run_tiles(L) <= (partial ? SPLIT_TILES_PARTIAL : SPLIT_TILES);
 }
 
 size_t store_size(const Lattice& L) {

@@ -65,14 +65,14 @@ def test_q_split_sizes(T, oracle_mod, nx, ny, S, R, prec):
 @pytest.mark.parametrize("prec,stress,fene", [("FP32", False, 0.0), ("FP16", False, 0.0),
                                               ("FP32", True, 0.0), ("FP16", True, 0.0),
                                               ("FP32", False, 3.1), ("FP32", True, 3.1)])
-@pytest.mark.parametrize("nx,ny", [(160, 160), (416, 64)])   # 100 and 104 tiles of 32 x 8
+@pytest.mark.parametrize("nx,ny", [(160, 160), (416, 64), (601, 58), (609, 57)])   # 100, 104, 152, 160 tiles of 32 x 8
 def test_both_sides_of_the_tile_line(T, oracle_mod, nx, ny, prec, stress, fene):
     _check(T, oracle_mod, _params(T, nx, ny, 6, 3.0, prec, stress, fene), 4, prec)
 
 
-# Partial tiles of the fused kernel (more than 100 tiles): last tiles of 1, 3, 31 and 30 by 1, 7
+# Partial tiles of the fused kernel (more than 152 tiles): last tiles of 1, 3, 31 and 30 by 1, 7
 # and 2 nodes, and grids of one tile column or row, whose tile is its own neighbour.
-PARTIAL = [(33, 409), (99, 207), (415, 63), (1, 801), (3330, 5), (62, 402)]
+PARTIAL = [(33, 617), (99, 311), (639, 63), (1, 1225), (4898, 5), (62, 610)]
 
 
 # (the stress model refuses this momentum relaxation time on five rows)
@@ -88,8 +88,8 @@ def test_fused_partial_tiles(T, oracle_mod, nx, ny, prec, stress, fene):
     _check(T, oracle_mod, p, 3, prec)
 
 
-@pytest.mark.parametrize("nx,ny,parts,prec", [(415, 70, 3, "FP32"), (415, 70, 2, "FP16"),
-                                              (416, 65, 4, "FP32"), (33, 420, 5, "FP32")])
+@pytest.mark.parametrize("nx,ny,parts,prec", [(575, 70, 3, "FP32"), (575, 70, 2, "FP16"),
+                                              (576, 65, 4, "FP32"), (33, 620, 5, "FP32")])
 def test_slabs_of_partial_tiles_are_bit_identical(T, nx, ny, parts, prec):
     """Slabs keep the whole run's tile rows wherever they start."""
     import torch
