@@ -156,12 +156,14 @@ double polymer_scale(const Lattice& L) {
 // fused kernel takes about 90 us up to one tile per SM, whatever the tiles hold, and the
 // line is there: with 32, 52 and 9 Q-nodes 91, 182 and 30.7 against 71, 107 and 16.8 at
 // 161 x 161 nodes (126 tiles), 91, 178 and 31.0 against 84, 123 and 21.8 at 500 x 65
-// (144); 90, 187 and 31.5 against 108, 159 and 25.5 at 200 x 200 (175). A slab steps as
+// (144); 90, 187 and 31.5 against 108, 159 and 25.5 at 200 x 200 (175). So it is in FP16
+// storage: 86.6, 150 and 29.8 against 69.5, 105 and 23.2 at 192 x 192 (144). A slab steps as
 // its whole run does, so the whole run's size decides.
-constexpr size_t SPLIT_TILES = 100, SPLIT_TILES_PARTIAL = 152;
+constexpr size_t SPLIT_TILES = 100, SPLIT_TILES_ONE_PER_SM = 152;
 bool split_path(const Lattice& L) {
   const bool partial = L.nx % TX || (L.ny_global > 0 ? L.ny_global : L.ny) % TY;
-  return L.precision == TFKT_FP64 || run_tiles(L) <= (partial ? SPLIT_TILES_PARTIAL : SPLIT_TILES);
+  return L.precision == TFKT_FP64 ||
+         run_tiles(L) <= (partial || L.precision == TFKT_FP16 ? SPLIT_TILES_ONE_PER_SM : SPLIT_TILES);
 }
 
 size_t store_size(const Lattice& L) {
