@@ -153,12 +153,12 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   const bool live = !RAGGED || (lx < box.w && ly < box.h);
   const int x = x0 + (RAGGED ? min(lx, box.w - 1) : lx), y = y0 + (RAGGED ? min(ly, box.h - 1) : ly);
   const size_t P = a.plane;
-  const real* __restrict__ Min = fa.Min;
+  const real* Min = fa.Min;
   real* __restrict__ Mout = fa.Mout;
   using SS = SolventT<S>;
-  const S* __restrict__ src = (const S*)a.src;
+  const S* src = (const S*)a.src;
   S* __restrict__ dst = (S*)a.dst;
-  const SS* __restrict__ ssrc = solvent_planes<S>(a.src, P, a.nq);
+  const SS* ssrc = solvent_planes<S>(a.src, P, a.nq);
   SS* __restrict__ sdst = solvent_planes<S>(a.dst, P, a.nq);
 
   // pull offsets within a plane (32-bit: a plane holds < 2^31 elements)

@@ -26,6 +26,9 @@ __device__ __forceinline__ void static_for(F&& f) {
 // arithmetic and table loads early, and reads or writes nothing of the state
 // before the kernels in front of it have completed. (Both are no-ops in a launch
 // without the attribute.)
+// Data that a predecessor may still be writing is not read through a __restrict__ pointer:
+// that promises that nobody writes it while the kernel runs, and the compiler may then load
+// it before the wait.
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 

@@ -259,7 +259,9 @@ __global__ void __launch_bounds__(NET_THREADS, 2) net_kernel(KernelArgs<float> a
   // 128-byte aligned view of the dynamic shared memory
   NetSmem& s = *reinterpret_cast<NetSmem*>(
       (unsigned char*)(((uintptr_t)net_smem + 127) & ~(uintptr_t)127));
-  // weights into the operand layout, the rest as FP32
+  // weights into the operand layout, the rest as FP32 (before the wait below: the kernel in
+  // front, prepare_kernel, lets this one start only when all before itself have completed,
+  // an optimiser step on the stream among them)
   for (int e = tid; e < NH * NET_K1; e += blockDim.x) {
     const int o = e / NET_K1, i = e % NET_K1;
     *reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(s.w1) + op_offset(o, i, NET_SBO1)) =
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(256) targets_kernel(KernelArgs<float> a, LpmAr
 // sub-step although most of them hit the cache (24 us at 1024 x 1024 nodes, now 18).
 template <bool FIRST>
 __global__ void __launch_bounds__(256) solvent_kernel(KernelArgs<float> a, LpmArgs l,
-                                                     const float* __restrict__ src,
+                                                     const float* src,
                                                      float* __restrict__ dst, float frac) {
   const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
   if (x >= a.nx || y >= a.ny) return;

@@ -215,10 +215,10 @@ __device__ __forceinline__ void train_store(const float (&c)[NN][4], int o0, int
 }
 
 // Loss and gradient partials of a block's tiles of TB samples; partial[b][NWEIGHTS].
-__global__ void __launch_bounds__(TT) loss_grad_kernel(const float* __restrict__ master,
-                                                       const __nv_bfloat16* __restrict__ wmat,
-                                                       const float* __restrict__ X,
-                                                       const float* __restrict__ T, int64_t n,
+__global__ void __launch_bounds__(TT) loss_grad_kernel(const float* master,
+                                                       const __nv_bfloat16* wmat,
+                                                       const float* X,
+                                                       const float* T, int64_t n,
                                                        float* __restrict__ partial,
                                                        double* __restrict__ lpart) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -365,10 +365,10 @@ __global__ void __launch_bounds__(TT) loss_grad_kernel(const float* __restrict__
 // of the blocks each, in a fixed order; loss = sum lpart / n by the last block. out:
 // the caller's copy of the gradient, or null.
 constexpr int RD_W = 32, RD_S = 8;   // weights and shares of a block
-__global__ void __launch_bounds__(RD_W * RD_S) reduce_kernel(const float* __restrict__ partial, int nblocks,
+__global__ void __launch_bounds__(RD_W * RD_S) reduce_kernel(const float* partial, int nblocks,
                                                              float* __restrict__ grad,
                                                              float* __restrict__ out,
-                                                             const double* __restrict__ lpart,
+                                                             const double* lpart,
                                                              double* __restrict__ loss, int64_t n) {
   __shared__ float part[RD_S][RD_W];
   __shared__ double lp[RD_S];
@@ -408,9 +408,9 @@ __global__ void __launch_bounds__(RD_W * RD_S) reduce_kernel(const float* __rest
 }
 
 // Adam on the master weights; c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t).
-__global__ void adam_kernel(float* __restrict__ master, __nv_bfloat16* __restrict__ wmat,
-                            float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ grad, float lr, float b1, float b2,
+__global__ void adam_kernel(float* master, __nv_bfloat16* __restrict__ wmat,
+                            float* m, float* v,
+                            const float* grad, float lr, float b1, float b2,
                             float eps, float c1, float c2) {
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
   let_successor_start();

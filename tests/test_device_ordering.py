@@ -3,6 +3,8 @@ else in the language keeps memory accesses on their side of an inline assembly s
 import pathlib
 import re
 
+import pytest
+
 CSRC = pathlib.Path(__file__).resolve().parents[1] / "paper_2201_10132_gb300" / "csrc"
 
 
@@ -37,3 +39,29 @@ def test_tensor_memory_load_and_its_wait_are_one_statement():
     loads = [a for a in (_balanced(text, m.end() - 1) for m in re.finditer(r"\basm volatile\(", text))
              if "tcgen05.ld." in a]
     assert loads and all("tcgen05.wait::ld" in a for a in loads)
+
+
+# Pointers that a kernel only writes may be __restrict__; one that it reads after a wait may not.
+WRITTEN_ONLY = {"Mout", "dst", "sdst", "partial", "lpart", "grad", "out", "loss", "wmat"}
+
+
+@pytest.mark.parametrize("name", sorted(f.name for f in CSRC.glob("*.cu")))
+def test_overlapped_kernels_read_nothing_through_restrict(name):
+    """A kernel that waits for its stream predecessor starts while that one still writes:
+    what it reads is not promised to be unwritten."""
+    text = _code(name)
+    found = 0
+    for m in re.finditer(r"\bvoid\s+(?:__launch_bounds__\s*\([^{;]*?\)\s*)?(\w+)\s*\(", text):
+        params = _balanced(text, m.end() - 1)
+        rest = text[m.end() - 1 + len(params):].lstrip()
+        if not rest.startswith("{"):
+            continue
+        body = _balanced(rest, 0, "{}")
+        if "wait_for_predecessor();" not in body:
+            continue
+        found += 1
+        for const, var in re.findall(r"(const\s+)?[\w:]+\s*\*\s*__restrict__\s+(\w+)", params + body):
+            assert not const, (m.group(1), var)
+            assert var in WRITTEN_ONLY, (m.group(1), var)
+    if name in ("tfkt_fused.cu", "tfkt_lpm.cu", "tfkt_mlp.cu", "tfkt_split.cu"):
+        assert found >= 2
