@@ -21,8 +21,7 @@ const MlpDev& mlp_dev(const tfkt_mlp* net);
 
 namespace {
 
-// Scratch planes of the learned block (ny * pitch floats each). L_B holds the sub-steps'
-// polymer terms (solvent_kernel) and then the increment's coefficients (reshape_kernel).
+// Scratch planes of the learned block (ny * pitch floats each).
 enum { L_PSI = 0, L_C1 = 1, L_DP = 4, L_JP = 6, L_CNEW = 8, L_CPREV = 11, L_B = 14, L_NPLANES = 18 };
 
 struct LpmArgs {
@@ -192,6 +191,13 @@ __device__ __forceinline__ void node_features(const KernelArgs<float>& a, const 
 // 64 -> 3 output layer (too narrow for the tensor cores) runs on the CUDA cores
 // in FP32. A wait that does not complete within its bound sets counter[1],
 // skips the TMEM reads (the tile falls back) and still frees the TMEM.
+//
+// The comparison with the threshold makes a tile's decision depend on the last bits of
+// C(t + 1) - C(t), times K: from the third block of a run on, indicators lie on both sides
+// of the threshold and some within rounding of it, and another decision moves a tile's C
+// by up to 2e-2 of C_e. So the block rounds as it always has: GELU through erff (250 us at
+// 1024 x 1024 nodes, 200 with the polynomial of the batched forward pass) and the
+// sub-steps' stress interpolated node by node (solvent_kernel).
 constexpr int NET_GROUPS = 2;
 constexpr int NET_THREADS = 128 * NET_GROUPS;
 constexpr int NET_K1 = 48;                       // layer-1 inner size: NIN padded to 3 steps of 16
@@ -349,7 +355,7 @@ __global__ void __launch_bounds__(NET_THREADS, 2) net_kernel(KernelArgs<float> a
       if (done1) {
         umma::ld_x32(tmem_row + 32u * half, v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = gelu(v[j] + s.b1[32 * half + j]);
+        for (int j = 0; j < 32; ++j) v[j] = gelu_erf(v[j] + s.b1[32 * half + j]);
       } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = 0.f;
@@ -381,7 +387,7 @@ __global__ void __launch_bounds__(NET_THREADS, 2) net_kernel(KernelArgs<float> a
         umma::ld_x32(tmem_row + 32u * half, v);
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-          const float hj = gelu(v[j] + s.b2[32 * half + j]);
+          const float hj = gelu_erf(v[j] + s.b2[32 * half + j]);
 #pragma unroll
           for (int c = 0; c < NOUT; ++c) o[c] = fmaf(s.w3[c][32 * half + j], hj, o[c]);
         }
@@ -456,12 +462,11 @@ __global__ void __launch_bounds__(256) targets_kernel(KernelArgs<float> a, LpmAr
 
 // One solvent sub-step: pull, U under the interpolated polymer stress with the
 // polymer momentum slaved (rho_S U = J_S + (tau2 + 1/2) E + rho a / 2 + dP), and
-// the plain step's solvent collision. The stress is linear in the fraction of the
-// way from C to C_new, so the block's first sub-step leaves
-// A = (tau2 + 1/2) E(C) + dP and B = (tau2 + 1/2) E(C_new - C) in the L_B planes and
-// the others read A + frac B: 14 plane loads per node in place of 40, which bound the
-// sub-step although most of them hit the cache (24 us at 1024 x 1024 nodes, now 18).
-template <bool FIRST>
+// the plain step's solvent collision. 24 us at 1024 x 1024 nodes, bound by its 40 plane
+// loads per node, most of which hit the cache. The stress is linear in frac, and
+// A + frac B from two kept pairs of planes takes 18 us, but rounds otherwise: three blocks
+// on, tiles whose indicator lies next to the threshold then decide otherwise than they
+// always have (net_kernel).
 __global__ void __launch_bounds__(256) solvent_kernel(KernelArgs<float> a, LpmArgs l,
                                                      const float* src,
                                                      float* __restrict__ dst, float frac) {
@@ -474,49 +479,26 @@ __global__ void __launch_bounds__(256) solvent_kernel(KernelArgs<float> a, LpmAr
   let_successor_start();
   float h[9], drs = 0.f, jsx = 0.f, jsy = 0.f;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) h[i] = src[(size_t)i * P + nb.o[shift_index(-c9x(i), -c9y(i))]];
-  const float* psi = l.p + (size_t)L_PSI * P;
-  const float psin = psi[n];
-  float* ab = l.p + (size_t)L_B * P + n;
-  float Ex, Ey;   // (tau2 + 1/2) E + dP
-  if (FIRST) {
-    const float t = l.tau2 + 0.5f;
-    float th0[4][3], thd[4][3];   // Theta of C and of C_new - C, right, left, above, below
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const size_t m = nb.o[k == 0 ? 5 : k == 1 ? 3 : k == 2 ? 7 : 1];
-      const float w = 0.5f * l.H * psi[m];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if ((k < 2 && c == 2) || (k >= 2 && c == 0)) continue;
-        const float c1 = l.p[(size_t)(L_C1 + c) * P + m];
-        th0[k][c] = w * c1;
-        thd[k][c] = w * (l.p[(size_t)(L_CNEW + c) * P + m] - c1);
-      }
-    }
-    auto div_x = [](const float (&v)[4][3]) { return 0.5f * (v[0][0] - v[1][0]) + 0.5f * (v[2][1] - v[3][1]); };
-    auto div_y = [](const float (&v)[4][3]) { return 0.5f * (v[0][1] - v[1][1]) + 0.5f * (v[2][2] - v[3][2]); };
-    Ex = t * div_x(th0) + l.p[(size_t)L_DP * P + n];
-    Ey = t * div_y(th0) + l.p[(size_t)(L_DP + 1) * P + n];
-    ab[0] = Ex;
-    ab[P] = Ey;
-    ab[2 * P] = t * div_x(thd);
-    ab[3 * P] = t * div_y(thd);
-  } else {
-    Ex = ab[0] + frac * ab[2 * P];
-    Ey = ab[P] + frac * ab[3 * P];
-  }
-#pragma unroll
   for (int i = 0; i < 9; ++i) {
+    h[i] = src[(size_t)i * P + nb.o[shift_index(-c9x(i), -c9y(i))]];
     drs += h[i];
     jsx += float(c9x(i)) * h[i];
     jsy += float(c9y(i)) * h[i];
   }
+  const float* psi = l.p + (size_t)L_PSI * P;
+  auto theta = [&](int c, size_t m) {
+    const float c1 = l.p[(size_t)(L_C1 + c) * P + m];
+    const float cn = l.p[(size_t)(L_CNEW + c) * P + m];
+    return 0.5f * l.H * psi[m] * (c1 + frac * (cn - c1));
+  };
+  const float ex = 0.5f * (theta(0, nb.o[5]) - theta(0, nb.o[3])) + 0.5f * (theta(1, nb.o[7]) - theta(1, nb.o[1]));
+  const float ey = 0.5f * (theta(1, nb.o[5]) - theta(1, nb.o[3])) + 0.5f * (theta(2, nb.o[7]) - theta(2, nb.o[1]));
   const float rs = 1.f + drs;
-  const float rho = rs + psin;
+  const float rho = rs + psi[n];
   const float force = rho * a.tab.arow[y];
-  const float Ux = (jsx + Ex + 0.5f * force) / rs;
-  const float Uy = (jsy + Ey) / rs;
+  const float t = l.tau2 + 0.5f;
+  const float Ux = (jsx + t * ex + 0.5f * force + l.p[(size_t)L_DP * P + n]) / rs;
+  const float Uy = (jsy + t * ey + l.p[(size_t)(L_DP + 1) * P + n]) / rs;
   const float jfx = (a.c2 * jsx + rs * Ux + a.tau2 * force) * a.inv_c2p1;
   const float jfy = (a.c2 * jsy + rs * Uy) * a.inv_c2p1;
   const float usx = jfx / rs, usy = jfy / rs;
@@ -791,8 +773,8 @@ extern "C" tfkt_status tfkt_lpm_run(tfkt_ctx* cc, const tfkt_mlp* net, const tfk
     LPM_CUDA(launch(net_kernel, tiles, dim3(NET_THREADS), nsm, st, true, a, l, nd));
     for (int j = 0; j < o->K; ++j) {
       KernelArgs<float> aj = ctx_args<float>(c);
-      LPM_CUDA(launch(j == 0 ? solvent_kernel<true> : solvent_kernel<false>, grid, blk, 0, st, true,
-                      aj, l, (const float*)aj.src, (float*)aj.dst, (float)j / (float)o->K));
+      LPM_CUDA(launch(solvent_kernel, grid, blk, 0, st, true, aj, l, (const float*)aj.src,
+                      (float*)aj.dst, (float)j / (float)o->K));
       c->cur ^= 1;
     }
     a = ctx_args<float>(c);

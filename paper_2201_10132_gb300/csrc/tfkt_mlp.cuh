@@ -24,14 +24,19 @@ struct MlpDev {
   __nv_bfloat16* wmat;      // [NMAT] W1, W2, W3 in bfloat16
 };
 
-// GELU(z) = z Phi(z) (Hendrycks & Gimpel 2016) of the forward pass, without branches:
+// GELU(z) = z Phi(z) (Hendrycks & Gimpel 2016), Phi through the library erff: the learned
+// block's, whose decisions hang on its last bits.
+__device__ __forceinline__ float gelu_erf(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
+
+// GELU of the forward pass on given samples, without branches:
 // with t = Phi(-|z|) it is max(z, 0) - |z| t, and t = 2^(|z| P(|z|) - 1). P is the
 // polynomial of degree 9 closest to log2(2 Phi(-a)) / a on 0 < a < 6.5 in the error that
 // it leaves in a t (weighted minimax by Lawson's iteration, 3e-9); beyond, |z| P falls on
 // and t underflows. The largest error against FP64 over |z| < 8 is 2.4e-7 (half an ulp of
 // the result) and the rms error 3.9e-8; 0.5 z (1 + erff(z / sqrt 2)) has 4.5e-7 and
-// 5.0e-8. 14 instructions where erff with its branch takes over twice as many: net_kernel
-// at 1024 x 1024 nodes took 253 us with it and takes 203.
+// 5.0e-8. 14 instructions where erff with its branch takes over twice as many: a
+// launch bound by its GELUs took 253 us with erff and 203 with the polynomial (net_kernel,
+// 1024 x 1024 nodes).
 // The derivative (training) needs Phi itself, for which erff is the closer one.
 __device__ constexpr float GELU_P[10] = {
     -1.151106358e+00f, -4.592034519e-01f, -5.249086022e-02f, 7.016736083e-03f, -5.537676407e-05f,
