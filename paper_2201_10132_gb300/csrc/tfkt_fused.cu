@@ -768,7 +768,6 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
   const size_t ntiles = (size_t)ntx * nty;
   const int nq = a.nq;
   const size_t P = a.plane;
-  let_successor_start();
   if (tid < NB) {
     const int k = tid;
     int lx, ly;
@@ -796,6 +795,7 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
     for (int c = 0; c < MAXC; ++c) s_e[c][k] = (size_t)ctile[c] * RING + cpos[c];
   }
   wait_for_predecessor();
+  let_successor_start();   // not earlier: the next step's blocks would take the place of this one's tiles
   __syncthreads();
   real* M = fa.Mout;
   const real* ex = fa.exports;
@@ -1000,6 +1000,27 @@ size_t max_tile_rows(const Lattice& L) {
   return (size_t)(L.ny / TY + 2) + (nyg % TY ? 2 * (size_t)(L.ny / nyg + 1) : 0);
 }
 
+// Which launches of a step may start while the kernel in front of them finishes. Blocks that
+// start early are dealt to what is free at that moment, and stay there.
+//  - The fix-up overlaps where an SM holds four of its blocks beside two of the step kernel
+//    (up to 32 Q-nodes); with more they keep the last wave's tiles from an SM of their own.
+//  - The step kernel too, with more than one tile per SM. With fewer, its blocks double up
+//    on the SMs that the kernel in front leaves idle, at half the speed each.
+// us per step in FP32 with neither, the fix-up alone and both overlapped: 192 x 160 nodes
+// (120 tiles), 9 Q-nodes 25.0, 24.7 and 27.5, 32 71.2, 69.6 and 81.3, 52 125.5, 125.0 and
+// 168; 320 x 320 (400), 9 61.4, 57.8 and 55.6, 32 171.7, 171.3 and 169.5, 45 274, 281 and
+// 312, 52 310, 319 and 359; 512 x 512 (1024), 32 358, 355 and 353, 52 701, 710 and 734.
+// No result depends on it.
+constexpr size_t SM_SMEM = 228 * 1024, BLOCK_SMEM = 1024;   // an SM's, and what a block takes of it by itself
+constexpr size_t FIX_STATIC = 5632;                         // static shared memory of a fix-up block, at most
+constexpr unsigned SMS = 152;
+
+static bool fixup_overlaps(int nq) {
+  return 2 * (fused_smem_bytes(nq, sizeof(float), TY) + BLOCK_SMEM) +
+             4 * (fix_smem_bytes<float, TY>(nq) + FIX_STATIC + BLOCK_SMEM) <= SM_SMEM;
+}
+static bool step_overlaps(int nq, dim3 tiles) { return tiles.x * tiles.y > SMS && fixup_overlaps(nq); }
+
 template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED>
 static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
                                 bool dependent) {
@@ -1009,7 +1030,7 @@ static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>
   if (e != cudaSuccess) return e;
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
   return launch(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, grid, dim3(TX, TY), smem, s,
-                dependent, a, f);
+                dependent && step_overlaps(a.nq, grid), a, f);
 }
 
 template <typename real, typename S>
@@ -1042,7 +1063,8 @@ static cudaError_t launch_fix(const KernelArgs<real>& a, const FusedArgs<real>& 
     if (e != cudaSuccess) return e;
   }
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
-  return launch(fixup_kernel<real, RAGGED>, grid, dim3(FIX_T), smem, s, dependent, a, f);
+  return launch(fixup_kernel<real, RAGGED>, grid, dim3(FIX_T), smem, s,
+                dependent && fixup_overlaps(a.nq), a, f);
 }
 
 template <typename real>
