@@ -1025,8 +1025,7 @@ template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED>
 static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
                                 bool dependent) {
   const size_t smem = fused_smem_bytes(a.nq, sizeof(real), TY);
-  cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
   return launch(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, grid, dim3(TX, TY), smem, s,
@@ -1057,11 +1056,8 @@ template <typename real, bool RAGGED>
 static cudaError_t launch_fix(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
                               bool dependent) {
   const size_t smem = fix_smem_bytes<real, TY>(a.nq);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fixup_kernel<real, RAGGED>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = allow_dynamic_smem(fixup_kernel<real, RAGGED>, smem);
+  if (e != cudaSuccess) return e;
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
   return launch(fixup_kernel<real, RAGGED>, grid, dim3(FIX_T), smem, s,
                 dependent && fixup_overlaps(a.nq), a, f);
@@ -1074,16 +1070,12 @@ cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cu
 }
 
 // Batches that launch each run's own single-run kernels (graph branches): the
-// attribute is set once here, so the launches below make no other API call.
+// limits are set once here, so the launches below make no other API call.
 cudaError_t prepare_single_fp32(int max_nq) {
-  const size_t smem = fused_smem_bytes(max_nq, sizeof(float), TY);
-  cudaError_t e = cudaFuncSetAttribute(step_fused_kernel<float, float, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const size_t fsmem = fix_smem_bytes<float, TY>(max_nq);
-  if (e == cudaSuccess && fsmem > 48 * 1024)
-    e = cudaFuncSetAttribute(fixup_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)fsmem);
-  return e;
+  cudaError_t e = allow_dynamic_smem(step_fused_kernel<float, float, false>,
+                                     fused_smem_bytes(max_nq, sizeof(float), TY));
+  if (e != cudaSuccess) return e;
+  return allow_dynamic_smem(fixup_kernel<float>, fix_smem_bytes<float, TY>(max_nq));
 }
 
 cudaError_t launch_single_fp32(const KernelArgs<float>& a, const FusedArgs<float>& f,
@@ -1099,9 +1091,8 @@ cudaError_t launch_single_fp32(const KernelArgs<float>& a, const FusedArgs<float
 
 template <int H>
 cudaError_t prepare_batch_h(int max_nq) {
-  const size_t smem = fused_smem_bytes(max_nq, sizeof(float), H);
-  return cudaFuncSetAttribute(step_fused_batch_kernel<float, float, H>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return allow_dynamic_smem(step_fused_batch_kernel<float, float, H>,
+                            fused_smem_bytes(max_nq, sizeof(float), H));
 }
 
 cudaError_t prepare_batch(int max_nq, int ty) {
@@ -1122,11 +1113,8 @@ cudaError_t launch_batch_step_h(const BatchRun<float>* runs, const int* tile_sta
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t fsmem = fix_smem_bytes<float, H>(max_nq);
-  if (fsmem > 48 * 1024) {
-    e = cudaFuncSetAttribute(fixup_batch_kernel<float, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)fsmem);
-    if (e != cudaSuccess) return e;
-  }
+  e = allow_dynamic_smem(fixup_batch_kernel<float, H>, fsmem);
+  if (e != cudaSuccess) return e;
   fixup_batch_kernel<float, H><<<total_tiles, FIX_T, fsmem, s>>>(runs, tile_start, nruns, parity);
   return cudaGetLastError();
 }

@@ -289,6 +289,21 @@ struct Ctx {
   int slab_ny = 0;        // owned rows (0: not a slab); the ghost rows are around them
 };
 
+// Lets a kernel take `bytes` of dynamic shared memory. The limit belongs to the kernel on its
+// device, not to the context or batch that asks: set to one caller's size it would fall
+// under another's, which has asked before and not launched yet, or launches from another
+// thread. So it goes to all that a block may have beside the kernel's static part, the
+// same for every caller.
+template <typename... Args>
+cudaError_t allow_dynamic_smem(void (*kernel)(Args...), size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;   // every block may have these
+  cudaFuncAttributes at;
+  cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              227 * 1024 - (int)at.sharedSizeBytes);
+}
+
 // Host helpers (tfkt_api.cu).
 tfkt_status fail(tfkt_status s, const std::string& msg);
 size_t align_up(size_t v, size_t a);

@@ -510,11 +510,8 @@ cudaError_t launch_velocity(const KernelArgs<real>& a, cudaStream_t s) {
 template <typename real>
 cudaError_t launch_fields(const KernelArgs<real>& a, uint32_t mask, double* out, cudaStream_t s) {
   const size_t smem = sizeof(real) == 4 ? FIELD_HEAD + (size_t)a.nq * sizeof(FieldRow) : 0;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fields_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = allow_dynamic_smem(fields_kernel<real>, smem);
+  if (e != cudaSuccess) return e;
   fields_kernel<real><<<node_grid(a.nx, a.ny), dim3(TX, TY), smem, s>>>(a, mask, out);
   return cudaGetLastError();
 }
