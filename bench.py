@@ -219,7 +219,7 @@ def run_reference(args, W):
 def precision_sweep(W, steps: int):
     """FP64 vs FP32 vs FP16 storage from the identical seeded state: per-field relative
     L2 / Linf errors against the FP64 run after `steps` steps, the growth rate of
-    sum U_y^2 (the instability indicator) over the run, and the fused-kernel time."""
+    sum U_y^2 (the instability indicator) over the run, and the time of a step's kernels."""
     import numpy as np
     import torch
     from paper_2201_10132_gb300 import tfkt
@@ -240,8 +240,7 @@ def precision_sweep(W, steps: int):
         s.close()
         del s, ws
         torch.cuda.empty_cache()
-        k = tfkt.KERNELS.index("fused")
-        r = {"fused_ms": kms[k] / max(n[k], 1), "ey2_rate": math.log(e1 / e0) / steps}
+        r = {"step_ms": float(kms.sum()) / steps, "ey2_rate": math.log(e1 / e0) / steps}
         if ref is None:
             ref = f
         else:
@@ -256,8 +255,19 @@ def precision_sweep(W, steps: int):
                 abs(out["fp64"]["ey2_rate"]), 1e-300)
         out[label] = r
     for label in ("fp32", "fp16"):
-        out[label]["speedup_vs_fp32"] = out["fp32"]["fused_ms"] / out[label]["fused_ms"]
+        out[label]["speedup_vs_fp32"] = out["fp32"]["step_ms"] / out[label]["step_ms"]
     return out
+
+
+def launch_models(path: str, nodes: int, pb: int, mb: int) -> dict:
+    """The kernel behind each counter of tfkt_step_profiled on a step path, and its
+    algorithmic bytes per launch: each population (pb bytes a node) read once and, by the
+    kernels that collide, written once; moment planes (mb bytes a node) read once by
+    those and written once by the kernels that produce them."""
+    moments, collide = ("moments_kernel", nodes * (pb + mb)), ("collide_kernel", nodes * (2 * pb + mb))
+    fused, fixup = ("fused_kernel", nodes * (2 * pb + 2 * mb)), ("fixup_kernel", None)
+    return {"moments": moments, "step": collide, "fused": fused if path == "fused" else collide,
+            "fixup": fixup if path == "fused" else moments}
 
 
 def capacity_run(steps: int, warmup: int):
@@ -439,7 +449,7 @@ def fp16_sub(W, steps: int, warmup: int, fp32_ms_per_step: float, fp32_fused_ms:
     stream = torch.cuda.Stream()
     s = tfkt.Solver(p, perturbation(W.nx, W.ny, W.seed, W.amp, W.u0), workspace=ws,
                     stream=stream.cuda_stream)
-    info = s.info
+    info, path = s.info, s.step_path()
     s.step(warmup)
     s.sync()
     kms = np.zeros(len(tfkt.KERNELS))
@@ -473,8 +483,9 @@ def fp16_sub(W, steps: int, warmup: int, fp32_ms_per_step: float, fp32_fused_ms:
             "ms_per_step": ms, "value": nodes / (ms / 1e3) / 1e9, "unit": "GLUPS",
             "fused_ms": fused_ms, "speedup_vs_fp32_step": fp32_ms_per_step / ms,
             "speedup_vs_fp32_fused": fp32_fused_ms / fused_ms,
-            "roofline": _hbm_roofline("fused", nodes * (2 * pb + 2 * nm * 4), fused_ms,
-                                      fused_traffic(nodes, "fp16"),
+            "roofline": _hbm_roofline("fused" if path == "fused" else "collide",
+                                      launch_models(path, nodes, pb, nm * 4)["fused"][1], fused_ms,
+                                      fused_traffic(nodes, "fp16") if path == "fused" else None,
                                       traffic_source="ncu capture of the 512^2 case, scaled by r-nodes"),
             "linf_vs_fp32_after_steps": err, "steps": steps,
             "gpu_launches": int(n.sum()), "clocks": clocks}
@@ -774,7 +785,7 @@ def main():
                                          W.u0)).pin_memory()
     stream = torch.cuda.Stream()
     solver = tfkt.Solver(p, pert.numpy(), workspace=ws, stream=stream.cuda_stream)
-    info = solver.info
+    info, path = solver.info, solver.step_path()
     solver.step(args.warmup)
     solver.sync()
 
@@ -827,16 +838,13 @@ def main():
         npl, nm = 9 + 25 * info["nq"], info["nq"] + 6
         # bytes of a node's populations: FP32, or FP32 solvent and FP16 polymer
         pb = npl * s if args.storage == "fp32" else 9 * 4 + 25 * info["nq"] * 2
-        # algorithmic bytes per launch: each population read once and written once;
-        # moment planes read once (and written once where the kernel produces them)
-        model = {"moments": nodes * (pb + nm * s), "step": nodes * (2 * pb + nm * s),
-                 "fused": nodes * (2 * pb + 2 * nm * s), "fixup": None}
+        model = launch_models(path, nodes, pb, nm * s)
         per = {}
         for k, name in enumerate(tfkt.KERNELS):
             if launches[k]:
                 ms_l = kms[k] / launches[k]
-                b = model[name]
-                per[name] = {"launches": int(launches[k]), "ms_per_launch": ms_l,
+                kernel, b = model[name]
+                per[name] = {"kernel": kernel, "launches": int(launches[k]), "ms_per_launch": ms_l,
                              "bytes_per_launch": b,
                              "achieved_gbs": None if b is None else b / (ms_l / 1e3) / 1e9}
         top = max(per, key=lambda k: per[k]["ms_per_launch"] * per[k]["launches"])
@@ -854,10 +862,10 @@ def main():
                        "l2": f"inputs larger than L2 (populations {nodes * pb / 1e9:.2f} GB "
                              "per buffer, L2 129 MB)",
                        "parallelism": f"{world} independent runs"},
-            "roofline": {"bound": "hbm", "kernel": top + "_kernel", "achieved": ach,
+            "roofline": {"bound": "hbm", "kernel": per[top]["kernel"], "achieved": ach,
                          "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak,
                          "peak_kind": peak_kind,
-                         "traffic": fused_traffic(nodes, args.storage) if top == "fused" else None,
+                         "traffic": fused_traffic(nodes, args.storage) if per[top]["kernel"] == "fused_kernel" else None,
                          "traffic_source": "ncu capture of the 512^2 case, scaled by r-nodes",
                          "bytes_per_launch": per[top]["bytes_per_launch"],
                          "step_model_gbs": nodes * (2 * pb + 2 * nm * s) / (ms / args.steps / 1e3) / 1e9,

@@ -115,17 +115,28 @@ typedef struct {
 
 typedef struct tfkt_ctx tfkt_ctx;
 
-/* Kernels timed by tfkt_step_profiled. */
+/* Launches timed by tfkt_step_profiled. Which kernels are behind them is what
+   tfkt_step_path says. */
 enum {
-  TFKT_K_MOMENTS = 0,  /* pull-read of all populations -> moment planes */
-  TFKT_K_STEP,         /* two-pass path (FP64 and up to 152 tiles where the grid is no multiple
-                          of the 32 x 8 tile, or too many Q-nodes for the fused kernel): pull,
-                          collide and write of all populations */
-  TFKT_K_FUSED,        /* fused path: pull, collide, write and next-step moments (the moments
-                          excepted in FP64 and on grids of up to 100 tiles) */
-  TFKT_K_FIXUP,        /* fused path: completion of the next step's moments (of the tiles'
-                          border nodes; in FP64 and on grids of up to 100 tiles of all nodes) */
+  TFKT_K_MOMENTS = 0,  /* TFKT_PATH_TWO_PASS: pull-read of all populations -> moment planes */
+  TFKT_K_STEP,         /* TFKT_PATH_TWO_PASS: pull, collide and write of all populations */
+  TFKT_K_FUSED,        /* first launch of the others: pull, collide and write of all
+                          populations, on TFKT_PATH_FUSED with the next step's moments */
+  TFKT_K_FIXUP,        /* second launch of the others: the next step's moments, on
+                          TFKT_PATH_FUSED those of the tiles' border nodes */
   TFKT_NKERNELS
+};
+
+/* The kernels that a step launches. The Q-split kernels (parallel over nodes and Q-nodes)
+   take FP64, and FP32 and FP16 storage up to a number of 32 x 8 tiles of the whole run's
+   grid: 100 in FP32 and 152 in FP16 storage on multiples of the tile, 152 on other grids;
+   and Q-disks that the fused kernel's shared memory does not hold. */
+enum {
+  TFKT_PATH_TWO_PASS = 0,  /* Q-split: the moments of the state, then its collision */
+  TFKT_PATH_SPLIT,         /* Q-split with double-buffered moments (tile multiples): the
+                              collision, then the moments of the state it wrote */
+  TFKT_PATH_FUSED          /* fused kernel on tiles (partial ones where the grid is no
+                              multiple) and its fix-up of the tiles' borders */
 };
 
 /* Macroscopic fields for tfkt_moments (bit i of the mask selects field i;
@@ -188,6 +199,10 @@ tfkt_status tfkt_step(tfkt_ctx* ctx, int64_t n);
    waiting in between; the host waits for the events once every 64 launches
    and at the end, so the call returns with the stream idle. */
 tfkt_status tfkt_step_profiled(tfkt_ctx* ctx, int64_t n, double* kernel_ms, int64_t* launches);
+
+/* *path: the TFKT_PATH_* of the context's next step (a step that follows a learned
+   block is fused on every context that runs one). Errors: TFKT_EINVAL for NULL. */
+tfkt_status tfkt_step_path(const tfkt_ctx* ctx, int32_t* path);
 
 /* Macroscopic fields of the current state (see TFKT_F_*: the moments of
    Sec. VI-A and VI-B, the mixture velocity of f of Sec. VI-C, the

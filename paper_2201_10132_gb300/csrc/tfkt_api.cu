@@ -459,9 +459,12 @@ tfkt_status ensure_moments(Ctx* c) {
   return TFKT_OK;
 }
 
-// Whether a step of a fused-path context takes the Q-split kernels. A pending
-// learned-block increment rides on the pull of the fused kernel only.
-inline bool step_split(const Ctx* c) { return c->split && !c->lpm_pending; }
+// The kernels of the next step. A pending learned-block increment rides on the pull of the
+// fused kernel only.
+inline int step_path(const Ctx* c) {
+  if (!c->fused) return TFKT_PATH_TWO_PASS;
+  return c->split && !c->lpm_pending ? TFKT_PATH_SPLIT : TFKT_PATH_FUSED;
+}
 
 // The fused kernel and its fix-up (FP64 contexts step with the Q-split kernels).
 template <typename real, typename S>
@@ -495,9 +498,10 @@ tfkt_status do_step(Ctx* c, int64_t n) {
       TFKT_CUDA(c, launch_moments<real, S>(a, c->stream, dep));
       c->m_valid = true;
     }
-    if (c->fused) {
+    const int path = step_path(c);
+    if (path != TFKT_PATH_TWO_PASS) {
       FusedArgs<real> f = make_fused<real>(c);
-      if (step_split(c)) {
+      if (path == TFKT_PATH_SPLIT) {
         TFKT_CUDA(c, launch_step<real, S>(a, c->stream, dep));
         TFKT_CUDA(c, launch_moments<real, S>(next_moments_args(a, f), c->stream, dep));
       } else {
@@ -569,9 +573,10 @@ tfkt_status do_step_profiled(Ctx* c, int64_t n, double* ms, int64_t* launches) {
       c->m_valid = true;
     }
     KernelArgs<real> a = make_args<real>(c);
-    if (c->fused) {
+    const int path = step_path(c);
+    if (path != TFKT_PATH_TWO_PASS) {
       FusedArgs<real> f = make_fused<real>(c);
-      const bool split = step_split(c);
+      const bool split = path == TFKT_PATH_SPLIT;
       if (c->lpm_pending) f.rshp = (const real*)c->lpm_rshp;
       tfkt_status s = timed(TFKT_K_FUSED, [&] {
         return split ? launch_step<real, S>(a, c->stream) : fused_kernel<real, S>(a, f, c->stream);
@@ -810,6 +815,12 @@ tfkt_status tfkt_step(tfkt_ctx* c, int64_t n) {
   if (s != TFKT_OK) return s;
   if (n < 0) return fail(TFKT_EINVAL, "n must be >= 0");
   return DISPATCH(c, do_step, c, n);
+}
+
+tfkt_status tfkt_step_path(const tfkt_ctx* c, int32_t* path) {
+  if (!c || !path) return fail(TFKT_EINVAL, "NULL argument");
+  *path = step_path(c);
+  return TFKT_OK;
 }
 
 tfkt_status tfkt_step_profiled(tfkt_ctx* c, int64_t n, double* kernel_ms, int64_t* launches) {

@@ -19,6 +19,7 @@ FP64, FP32, FP16 = 0, 1, 2
 FIELDS = ["rho_s", "psi_tot", "ux", "uy", "cxx", "cxy", "cyy", "thxx", "thxy", "thyy", "qrms",
           "vort"]
 KERNELS = ["moments", "step", "fused", "fixup"]
+STEP_PATHS = ["two_pass", "split", "fused"]
 DIAGS = ["mass_s", "mass_p", "px", "py", "ke", "enstrophy", "qrms_mean", "ey2", "umax",
          "qrms_max"]
 STATUS = {0: "TFKT_OK", 1: "TFKT_EINVAL", 2: "TFKT_ENOMEM", 3: "TFKT_ECUDA", 4: "TFKT_ENAN",
@@ -113,6 +114,7 @@ def lib() -> ctypes.CDLL:
                                   ctypes.POINTER(P)]
         L.tfkt_step.argtypes = [P, ctypes.c_int64]
         L.tfkt_step_profiled.argtypes = [P, ctypes.c_int64, D, ctypes.POINTER(ctypes.c_int64)]
+        L.tfkt_step_path.argtypes = [P, ctypes.POINTER(ctypes.c_int32)]
         L.tfkt_moments.argtypes = [P, ctypes.c_uint32, P, ctypes.c_size_t, ctypes.c_int]
         L.tfkt_psi.argtypes = [P, P, ctypes.c_size_t, ctypes.c_int]
         L.tfkt_moments_noalloc.argtypes = [ctypes.POINTER(_Params), P, ctypes.c_uint32, P,
@@ -175,7 +177,7 @@ def lib() -> ctypes.CDLL:
         L.tfkt_status_string.argtypes = [S]
         L.tfkt_status_string.restype = ctypes.c_char_p
         L.tfkt_last_error.restype = ctypes.c_char_p
-        for n in ("tfkt_required_bytes", "tfkt_create", "tfkt_step", "tfkt_step_profiled",
+        for n in ("tfkt_required_bytes", "tfkt_create", "tfkt_step", "tfkt_step_profiled", "tfkt_step_path",
                   "tfkt_moments", "tfkt_psi",
                   "tfkt_diagnostics", "tfkt_populations", "tfkt_get_info", "tfkt_lattice",
                   "tfkt_sync", "tfkt_destroy", "tfkt_save", "tfkt_load"):
@@ -274,6 +276,12 @@ class Solver:
         _check(lib().tfkt_step_profiled(self._h, int(n), _dptr(kernel_ms),
                                         launches.ctypes.data_as(ctypes.POINTER(ctypes.c_int64))),
                "tfkt_step_profiled")
+
+    def step_path(self) -> str:
+        """tfkt_step_path: the kernels of the next step, one of STEP_PATHS."""
+        p = ctypes.c_int32()
+        _check(lib().tfkt_step_path(self._h, ctypes.byref(p)), "tfkt_step_path")
+        return STEP_PATHS[p.value]
 
     def sync(self):
         _check(lib().tfkt_sync(self._h), "tfkt_sync")
