@@ -208,6 +208,8 @@ size_t layout(const Lattice& L, Workspace* w) {
   if (fused_path(L)) {
     w->off_M2 = o;
     o = align_up(o + (size_t)L.nm * L.plane * sz, A);
+  }
+  if (fused_path(L) && L.precision != TFKT_FP64) {   // what the fused kernel and its fix-up need
     w->off_exp = o;
     o = align_up(o + fused_export_capacity(L) * sz, A);
     w->off_ftab = o;
@@ -357,6 +359,7 @@ FusedArgs<real> make_fused(const Ctx* c) {
   FusedArgs<real> f{};
   f.Min = (const real*)(base + (c->mcur ? c->ws.off_M2 : c->ws.off_M));
   f.Mout = (real*)(base + (c->mcur ? c->ws.off_M : c->ws.off_M2));
+  if (sizeof(real) == 8) return f;   // FP64 steps with the Q-split kernels
   f.exports = (real*)(base + c->ws.off_exp);
   f.tgt = (const int*)(base + c->ws.off_ftab);
   f.dpsi = (const real*)(base + c->ws.off_ftab + align_up((size_t)L.nq * 9 * sizeof(int), 256));
@@ -370,8 +373,8 @@ FusedArgs<real> make_fused(const Ctx* c) {
   return f;
 }
 
-template <typename real>
 tfkt_status upload_fused_tables(Ctx* c, const HostTables& t) {
+  using real = float;
   std::vector<int> tgt;
   std::vector<double> dpsi;
   std::vector<long long> poff;
@@ -382,16 +385,14 @@ tfkt_status upload_fused_tables(Ctx* c, const HostTables& t) {
   if (c->ntrow)
     TFKT_CUDA(c, cudaMemcpy((void*)f.trow, trow.data(), trow.size() * sizeof(int2),
                             cudaMemcpyHostToDevice));
-  if constexpr (std::is_same<real, float>::value) {
-    const int cur = c->cur;
-    for (c->cur = 0; c->cur < 2; ++c->cur) {
-      const std::vector<char> img = fused_image(c->L, t, tgt, poff, (const char*)c->ws.base + c->ws.off_pop[c->cur],
-                                                store_size(c->L));
-      cudaError_t e = cudaMemcpy((void*)make_fused<real>(c).image, img.data(), img.size(), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) return cuda_fail(c, e, "table image");
-    }
-    c->cur = cur;
+  const int cur = c->cur;
+  for (c->cur = 0; c->cur < 2; ++c->cur) {
+    const std::vector<char> img = fused_image(c->L, t, tgt, poff, (const char*)c->ws.base + c->ws.off_pop[c->cur],
+                                              store_size(c->L));
+    cudaError_t e = cudaMemcpy((void*)make_fused<real>(c).image, img.data(), img.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_fail(c, e, "table image");
   }
+  c->cur = cur;
   std::vector<real> d(dpsi.begin(), dpsi.end());
   TFKT_CUDA(c, cudaMemcpy((void*)f.poff, poff.data(), poff.size() * sizeof(long long),
                           cudaMemcpyHostToDevice));
@@ -422,7 +423,8 @@ tfkt_status upload_tables(Ctx* c, const HostTables& t) {
   const std::vector<QRow<real>> rows = build_rows<real>(c->L, t);
   TFKT_CUDA(c, cudaMemcpy((void*)a.tab.row, rows.data(), rows.size() * sizeof(QRow<real>),
                           cudaMemcpyHostToDevice));
-  if (c->fused) return upload_fused_tables<real>(c, t);
+  if constexpr (std::is_same<real, float>::value)
+    if (c->fused) return upload_fused_tables(c, t);
   return TFKT_OK;
 }
 

@@ -56,7 +56,7 @@ tfkt_status check_runs(const tfkt_params* runs, int32_t n, std::vector<Lattice>&
     // Every run must take the single-run fused path (8-row tiles): its context
     // then holds the export ring, the second moment buffer and the fused tables
     // that the batch kernels use at any tile height.
-    if (!fused_supported(L[i].nx, L[i].ny, L[i].nq, 4, 8))
+    if (!fused_supported(L[i].nx, L[i].ny, L[i].nq, 8))
       return fail(TFKT_EINVAL, "batched runs need nx % 32 == 0 and ny % 8 == 0 (run " +
                                    std::to_string(i) + ")");
   }
@@ -169,7 +169,7 @@ std::vector<int> candidates(const std::vector<Lattice>& L) {
   std::vector<int> out;
   for (int ty : {4, 8, 16}) {
     bool ok = true;
-    for (const Lattice& l : L) ok = ok && fused_supported(l.nx, l.ny, l.nq, 4, ty);
+    for (const Lattice& l : L) ok = ok && fused_supported(l.nx, l.ny, l.nq, ty);
     if (ok) out.push_back(ty);
   }
   return out;

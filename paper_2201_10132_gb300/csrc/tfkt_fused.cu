@@ -924,17 +924,16 @@ __global__ void __launch_bounds__(FIX_T) fixup_batch_kernel(const BatchRun<real>
 }  // namespace
 
 template <int H>
-size_t smem_bytes_h(int nq, size_t real_bytes) {
+size_t smem_bytes_h(int nq) {
   size_t a, b, c, d, e, f;
-  return real_bytes == 8 ? smem_layout<double, H>(nq, &a, &b, &c, &d, &e, &f)
-                         : smem_layout<float, H>(nq, &a, &b, &c, &d, &e, &f);
+  return smem_layout<float, H>(nq, &a, &b, &c, &d, &e, &f);
 }
 
-size_t fused_smem_bytes(int nq, size_t real_bytes, int ty) {
+size_t fused_smem_bytes(int nq, int ty) {
   switch (ty) {
-    case 4: return smem_bytes_h<4>(nq, real_bytes);
-    case 8: return smem_bytes_h<8>(nq, real_bytes);
-    case 16: return smem_bytes_h<16>(nq, real_bytes);
+    case 4: return smem_bytes_h<4>(nq);
+    case 8: return smem_bytes_h<8>(nq);
+    case 16: return smem_bytes_h<16>(nq);
     default: return ~(size_t)0;
   }
 }
@@ -948,18 +947,18 @@ static size_t export_elems(size_t tiles, int nq, int ty) {
 size_t fused_export_capacity(const Lattice& L) {
   const size_t ntx = (L.nx + TX - 1) / TX;
   size_t m = 0;
-  if (L.precision == TFKT_FP64 || whole_tiles(L)) {
+  if (whole_tiles(L)) {
     for (int ty : {4, 8, 16})
       if (L.ny % ty == 0) m = std::max(m, export_elems(ntx * (L.ny / ty), L.nq, ty));
   }
-  if (L.precision != TFKT_FP64 && (!whole_tiles(L) || L.ny_global > 0))
+  if (!whole_tiles(L) || L.ny_global > 0)
     m = std::max(m, export_elems(ntx * max_tile_rows(L), L.nq, TY));
   return m;
 }
 
-bool fused_supported(int nx, int ny, int nq, size_t real_bytes, int ty) {
+bool fused_supported(int nx, int ny, int nq, int ty) {
   return nx % TX == 0 && ny % ty == 0 &&
-         fused_smem_bytes(nq, real_bytes, ty) <= 227 * 1024;
+         fused_smem_bytes(nq, ty) <= 227 * 1024;
 }
 
 // Tiles of the whole run that a context belongs to.
@@ -973,9 +972,15 @@ size_t run_tiles(const Lattice& L) {
 // step on 1000 x 750 nodes with 32 Q-nodes in FP32 (1026 in FP16 storage, 993 on 999 x 751
 // with the stress quasi-equilibrium), the Q-split kernels, which read the populations
 // twice, 1426 (1193, 1437); with 9 Q-nodes on 333 x 777 nodes 134 against 174.
+//
+// FP64 has no fused kernel. Whole tiles keep the second set of moment planes all the same
+// (2% of the workspace at 32 Q-nodes): a step then leaves the moments of its result, and
+// no read-out between steps reads the populations again. Disks of more than 58 Q-nodes, which
+// an FP64 tile never held, keep one set.
 bool fused_path(const Lattice& L) {
-  if (fused_smem_bytes(L.nq, L.precision == TFKT_FP64 ? 8 : 4) > 227 * 1024) return false;
-  return whole_tiles(L) || (L.precision != TFKT_FP64 && !split_path(L));
+  if (L.precision == TFKT_FP64) return whole_tiles(L) && L.nq <= 58;
+  if (fused_smem_bytes(L.nq) > 227 * 1024) return false;
+  return whole_tiles(L) || !split_path(L);
 }
 
 // First row and height of every tile row, or none where they are the whole tiles that
@@ -985,7 +990,7 @@ bool fused_path(const Lattice& L) {
 std::vector<int2> tile_rows(const Lattice& L) {
   const int nyg = L.ny_global > 0 ? L.ny_global : L.ny;
   std::vector<int2> rows;
-  if (L.precision == TFKT_FP64 || (whole_tiles(L) && nyg % TY == 0 && L.y_origin % TY == 0)) return rows;
+  if (whole_tiles(L) && nyg % TY == 0 && L.y_origin % TY == 0) return rows;
   for (int y = 0; y < L.ny; ++y) {
     const int yg = ((L.y_origin + y) % nyg + nyg) % nyg;
     if (y == 0 || yg % TY == 0) rows.push_back(make_int2(y, 0));
@@ -1016,7 +1021,7 @@ constexpr size_t FIX_STATIC = 5632;                         // static shared mem
 constexpr unsigned SMS = 152;
 
 static bool fixup_overlaps(int nq) {
-  return 2 * (fused_smem_bytes(nq, sizeof(float), TY) + BLOCK_SMEM) +
+  return 2 * (fused_smem_bytes(nq) + BLOCK_SMEM) +
              4 * (fix_smem_bytes<float, TY>(nq) + FIX_STATIC + BLOCK_SMEM) <= SM_SMEM;
 }
 static bool step_overlaps(int nq, dim3 tiles) { return tiles.x * tiles.y > SMS && fixup_overlaps(nq); }
@@ -1024,7 +1029,7 @@ static bool step_overlaps(int nq, dim3 tiles) { return tiles.x * tiles.y > SMS &
 template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED>
 static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
                                 bool dependent) {
-  const size_t smem = fused_smem_bytes(a.nq, sizeof(real), TY);
+  const size_t smem = fused_smem_bytes(a.nq);
   cudaError_t e = allow_dynamic_smem(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
@@ -1073,7 +1078,7 @@ cudaError_t launch_fixup(const KernelArgs<real>& a, const FusedArgs<real>& f, cu
 // limits are set once here, so the launches below make no other API call.
 cudaError_t prepare_single_fp32(int max_nq) {
   cudaError_t e = allow_dynamic_smem(step_fused_kernel<float, float, false>,
-                                     fused_smem_bytes(max_nq, sizeof(float), TY));
+                                     fused_smem_bytes(max_nq));
   if (e != cudaSuccess) return e;
   return allow_dynamic_smem(fixup_kernel<float>, fix_smem_bytes<float, TY>(max_nq));
 }
@@ -1081,7 +1086,7 @@ cudaError_t prepare_single_fp32(int max_nq) {
 cudaError_t launch_single_fp32(const KernelArgs<float>& a, const FusedArgs<float>& f,
                                cudaStream_t s) {
   const dim3 grid(a.nx / TX, a.ny / TY), block(TX, TY);
-  step_fused_kernel<float, float, false><<<grid, block, fused_smem_bytes(a.nq, sizeof(float), TY), s>>>(
+  step_fused_kernel<float, float, false><<<grid, block, fused_smem_bytes(a.nq), s>>>(
       a, f);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -1092,7 +1097,7 @@ cudaError_t launch_single_fp32(const KernelArgs<float>& a, const FusedArgs<float
 template <int H>
 cudaError_t prepare_batch_h(int max_nq) {
   return allow_dynamic_smem(step_fused_batch_kernel<float, float, H>,
-                            fused_smem_bytes(max_nq, sizeof(float), H));
+                            fused_smem_bytes(max_nq, H));
 }
 
 cudaError_t prepare_batch(int max_nq, int ty) {
@@ -1107,7 +1112,7 @@ cudaError_t prepare_batch(int max_nq, int ty) {
 template <int H>
 cudaError_t launch_batch_step_h(const BatchRun<float>* runs, const int* tile_start, int nruns,
                                 int total_tiles, int max_nq, int parity, cudaStream_t s) {
-  const size_t smem = fused_smem_bytes(max_nq, sizeof(float), H);
+  const size_t smem = fused_smem_bytes(max_nq, H);
   step_fused_batch_kernel<float, float, H><<<total_tiles, dim3(TX, H), smem, s>>>(
       runs, tile_start, nruns, parity);
   cudaError_t e = cudaGetLastError();

@@ -275,9 +275,9 @@ struct Ctx {
   bool poisoned = false;
   int64_t step = 0;
   int diag_blocks = 0;
-  bool fused = false;     // the fused path (double-buffered moment planes)
+  bool fused = false;     // double-buffered moment planes (fused_path)
   int ntrow = 0;          // tile rows of a fused-path context with partial tiles
-  bool split = false;     // a fused-path context that steps with the Q-split kernels
+  bool split = false;     // such a context that steps with the Q-split kernels
   int mcur = 0;           // moment buffer (0: off_M, 1: off_M2) of the current state
   double dvx = 0, dvy = 0;  // r-momentum of all pull shift differences (fused path)
   void* lpm = nullptr;    // scratch of the learned block (allocated on first use)
@@ -352,11 +352,11 @@ cudaError_t launch_diag(const KernelArgs<real>& a, double* partials, int nblocks
                         cudaStream_t s);
 
 // Fused single-pass step (tfkt_fused.cu).
-size_t fused_smem_bytes(int nq, size_t real_bytes, int ty = TY);
+size_t fused_smem_bytes(int nq, int ty = TY);   // (FP32 arithmetic)
 // ring-export elements of a context, enough for every tile height a batch may choose
 // (4, 8, 16)
 size_t fused_export_capacity(const Lattice& L);
-bool fused_supported(int nx, int ny, int nq, size_t real_bytes, int ty = TY);
+bool fused_supported(int nx, int ny, int nq, int ty = TY);
 size_t run_tiles(const Lattice& L);
 std::vector<int2> tile_rows(const Lattice& L);
 size_t max_tile_rows(const Lattice& L);
