@@ -229,8 +229,7 @@ struct tfkt_mlp {
   float* partial = nullptr;   // per-block gradient partials
   int partial_blocks = 0;     // blocks that it holds
   double* lpart = nullptr;    // per-block loss partials, then the loss
-  double* loss_host = nullptr;  // pinned: the last loss, from its second read on
-  bool loss_read = false;
+  double* loss_host = nullptr;  // pinned: the last loss (null: it stays behind lpart)
   int64_t t = 0;              // Adam steps taken
   cudaStream_t stream = nullptr;
 };
