@@ -91,8 +91,8 @@ typedef struct {
                             anti-diffusive in r, make the step unstable; keep the disk
                             well inside Q0. */
   int32_t qe_model;      /* tfkt_qe_model: which variables the collision holds
-                            quasi-conserved (Sec. V); both models run on
-                               every kernel path */
+                            quasi-conserved (Sec. V); both models run on every
+                            kernel path */
 } tfkt_params;
 
 /* Derived lattice parameters and layout of a context. */
@@ -388,9 +388,10 @@ tfkt_status tfkt_batch_destroy(tfkt_batch* b);
    the first slab). The ghost width is one row of the fused path's 32 x 8
    tiles, and a slab's tile rows are those of the single-domain run, so every
    owned node sums its arrivals in the same order. The owned rows are bit-
-   identical to the single-domain run: for any split in FP64, on runs of up to
-   100 tiles and on runs whose nx is no multiple of 32 or whose ny is none of 8,
-   and on the others with y0 and ny_local multiples of 8. The learned block does not run on a slab context (EINVAL). */
+   identical to the single-domain run: for any split where that run's path is not
+   TFKT_PATH_FUSED or its nx is no multiple of 32 or its ny none of 8, and on
+   the others with y0 and ny_local multiples of 8. The learned block does not
+   run on a slab context (EINVAL). */
 #define TFKT_SLAB_GHOST 8
 enum { TFKT_SLAB_LOW = 0, TFKT_SLAB_HIGH = 1 };
 

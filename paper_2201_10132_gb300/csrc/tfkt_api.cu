@@ -147,18 +147,23 @@ double polymer_scale(const Lattice& L) {
 // The Q-split kernels instead of the fused kernel: FP64 always (both are bound by
 // the FP64 pipe, of which the fused kernel needs about twice as much: 512 x 512 nodes, 32
 // Q-nodes, 4739 us per step against 3071), other precisions where the fused
-// kernel's tiles leave most SMs idle. That kernel takes the same time up to one
-// tile per SM, the Q-split kernels a time that grows with the nodes. FP32, us per
-// step, with 32 Q-nodes: 61.8 against 12.1 at 64 x 64 nodes (16 tiles), 64 against 35
-// at 128 x 128 (64), 71.5 against 60 at 160 x 160 (100), 77.5 against 90 at 192 x 192
-// (144); with 9 Q-nodes 25.4 against 13.8 at 128 x 128, 26.8 against 16.2 at 160 x 160,
-// 36 against 57 at 256 x 256. The line is drawn at 100 tiles. With partial tiles the
-// fused kernel takes about 90 us up to one tile per SM, whatever the tiles hold, and the
-// line is there: with 32, 52 and 9 Q-nodes 91, 182 and 30.7 against 71, 107 and 16.8 at
-// 161 x 161 nodes (126 tiles), 91, 178 and 31.0 against 84, 123 and 21.8 at 500 x 65
-// (144); 90, 187 and 31.5 against 108, 159 and 25.5 at 200 x 200 (175). So it is in FP16
-// storage: 86.6, 150 and 29.8 against 69.5, 105 and 23.2 at 192 x 192 (144). A slab steps as
-// its whole run does, so the whole run's size decides.
+// kernel's tiles leave most SMs idle. That kernel takes about the same time up to one
+// tile per SM, the Q-split kernels a time that grows with the nodes. The lines are those
+// of 32 Q-nodes. us per step, fused and Q-split, with 9, 32 and 52 Q-nodes:
+//   FP32, whole tiles    160 x 160 (100 tiles)  22.7 16.0    65.8  61.4    125  97
+//                        192 x 160 (120)        24.6 20.2    69.4  79.0    126 116
+//                        640 x 64  (160)        27.6 23.8    82.2 105.9    179 154
+//                        224 x 224 (196)        29.3 29.7    86.5 121.5    191 177
+//   FP32, partial tiles  161 x 161 (126)        26.3 16.7    74.5  70.8    133 107
+//                        500 x 65  (144)        26.8 21.7    76.2  83.1    134 122
+//                        200 x 200 (175)        30.3 25.2    89.6 107.6    188 158
+//   FP16, whole tiles    192 x 192 (144)        24.8 22.8    67.8  69.3    117 105
+//                        640 x 64  (160)        29.0 24.6    85.6  86.1    153 130
+//   FP16, partial tiles  200 x 193 (175)        35.4 23.3   106.8  74.3    179 110
+// (64 x 64 with 32 Q-nodes in FP32: 61.8 and 12.1). So with 9 and 52 Q-nodes the Q-split
+// kernels stay ahead up to about 190 tiles, and FP32 grids of 130 to 152 partial tiles
+// with 32 would take up to 9% less in the fused kernel: one line for all disks leaves
+// these. A slab steps as its whole run does, so the whole run's size decides.
 constexpr size_t SPLIT_TILES = 100, SPLIT_TILES_ONE_PER_SM = 152;
 bool split_path(const Lattice& L) {
   const bool partial = L.nx % TX || (L.ny_global > 0 ? L.ny_global : L.ny) % TY;
