@@ -160,10 +160,10 @@ double polymer_scale(const Lattice& L) {
 //   FP16, whole tiles    192 x 192 (144)        24.8 22.8    67.8  69.3    117 105
 //                        640 x 64  (160)        29.0 24.6    85.6  86.1    153 130
 //   FP16, partial tiles  200 x 193 (175)        35.4 23.3   106.8  74.3    179 110
-// (64 x 64 with 32 Q-nodes in FP32: 61.8 and 12.1). So with 9 and 52 Q-nodes the Q-split
-// kernels stay ahead up to about 190 tiles, and FP32 grids of 130 to 152 partial tiles
-// with 32 would take up to 9% less in the fused kernel: one line for all disks leaves
-// these. A slab steps as its whole run does, so the whole run's size decides.
+// (64 x 64 with 32 Q-nodes in FP32: 61.8 and 12.1). So with 9 and 52 Q-nodes, and in FP16
+// storage on partial tiles with 32, the Q-split kernels stay ahead up to about 190 tiles, and
+// FP32 grids of 130 to 152 partial tiles with 32 would take up to 9% less in the fused
+// kernel: one line for all disks leaves these. A slab steps as its whole run does, so the whole run's size decides.
 constexpr size_t SPLIT_TILES = 100, SPLIT_TILES_ONE_PER_SM = 152;
 bool split_path(const Lattice& L) {
   const bool partial = L.nx % TX || (L.ny_global > 0 ? L.ny_global : L.ny) % TY;

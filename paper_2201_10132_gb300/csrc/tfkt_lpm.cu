@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(256) targets_kernel(KernelArgs<float> a, LpmAr
 
 // One solvent sub-step: pull, U under the interpolated polymer stress with the
 // polymer momentum slaved (rho_S U = J_S + (tau2 + 1/2) E + rho a / 2 + dP), and
-// the plain step's solvent collision. 24 us at 1024 x 1024 nodes, bound by its 40 plane
+// the plain step's solvent collision. 24 to 26 us at 1024 x 1024 nodes, bound by its 40 plane
 // loads per node, most of which hit the cache. The stress is linear in frac, and
 // A + frac B from two kept pairs of planes takes 18 us, but rounds otherwise: three blocks
 // on, tiles whose indicator lies next to the threshold then decide otherwise than they
