@@ -18,6 +18,8 @@ thread_local std::string g_last_error;
 
 tfkt_status fail(tfkt_status s, const std::string& msg) {
   g_last_error = msg;
+  // reported once: left pending in the runtime, it would fail the next call's launch checks too
+  if (s == TFKT_ECUDA) cudaGetLastError();
   return s;
 }
 
