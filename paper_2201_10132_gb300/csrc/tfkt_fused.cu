@@ -750,22 +750,29 @@ constexpr int fix_nodes() { return 2 * TX + 2 * (H - 2); }
 template <typename real, int H>
 size_t fix_smem_bytes(int nq) { return (size_t)(nq + 1) * fix_nodes<H>() * sizeof(real); }
 
-template <typename real, int H, bool RAGGED = false>
-__device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const FusedArgs<real>& fa,
-                                           int tx, int ty, int ntx, int nty, real* s_d) {
+// Contributing neighbour tiles of a border node: 1 to 3, and up to 8 where a partial tile is
+// one node wide or high.
+template <int H, bool PARTIAL>
+struct FixNodes {
+  uint32_t n[fix_nodes<H>()];                    // node offset within a plane
+  uint32_t nc[fix_nodes<H>()];                   // contributing neighbour tiles
+  size_t e[PARTIAL ? 8 : 3][fix_nodes<H>()];     // their export positions (tile * RING + ring position)
+};
+
+// The fix-up of one tile; PARTIAL: the tile is `box`, else a whole one.
+template <typename real, int H, bool PARTIAL>
+__device__ __forceinline__ void fixup_tile(const KernelArgs<real>& a, const FusedArgs<real>& fa,
+                                           const TileBox& box, int tx, int ty, int ntx, int nty,
+                                           real* s_d, FixNodes<H, PARTIAL>& nodes) {
   constexpr int TY = H, RING = Geo<H>::RING;
   constexpr int MAXNB = fix_nodes<H>();
-  // contributing neighbour tiles of a node: 1 to 3, and up to 8 where a partial tile
-  // is one node wide or high
-  constexpr int MAXC = RAGGED ? 8 : 3;
-  __shared__ uint32_t s_n[MAXNB];     // node offset within a plane
-  __shared__ uint32_t s_nc[MAXNB];    // contributing neighbour tiles
-  __shared__ size_t s_e[MAXC][MAXNB]; // their export positions (tile * RING + ring position)
-  TileBox box{tx * TX, ty * TY, TX, TY};
-  if constexpr (RAGGED) box = tile_box(a.nx, fa.trow, tx, ty, ntx);
-  const int W = box.w, h = box.h;
+  constexpr int MAXC = PARTIAL ? 8 : 3;
+  auto& s_n = nodes.n;
+  auto& s_nc = nodes.nc;
+  auto& s_e = nodes.e;
+  const int W = PARTIAL ? box.w : TX, h = PARTIAL ? box.h : TY;
   const int top = h > 1 ? 2 * W : W;  // nodes of the first and the last row
-  const int NB = RAGGED ? top + (h > 2 ? (W > 1 ? 2 : 1) * (h - 2) : 0) : MAXNB;
+  const int NB = PARTIAL ? top + (h > 2 ? (W > 1 ? 2 : 1) * (h - 2) : 0) : MAXNB;
   const int tid = threadIdx.x;
   const size_t ntiles = (size_t)ntx * nty;
   const int nq = a.nq;
@@ -853,6 +860,25 @@ __device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const Fuse
     M[(size_t)(nq + M_THXX) * P + n] = a.hl2h * txx;
     M[(size_t)(nq + M_THXY) * P + n] = a.hl2h * txy;
     M[(size_t)(nq + M_THYY) * P + n] = a.hl2h * tyy;
+  }
+}
+
+// RAGGED: tiles may be partial. Most of such a grid's are whole and take the whole tiles' form,
+// whose node count is a constant and whose nodes have three contributions at most.
+template <typename real, int H, bool RAGGED = false>
+__device__ __forceinline__ void fixup_body(const KernelArgs<real>& a, const FusedArgs<real>& fa,
+                                           int tx, int ty, int ntx, int nty, real* s_d) {
+  if constexpr (RAGGED) {
+    __shared__ union {
+      FixNodes<H, false> whole;
+      FixNodes<H, true> partial;
+    } nodes;
+    const TileBox box = tile_box(a.nx, fa.trow, tx, ty, ntx);
+    if (box.w == TX && box.h == H) fixup_tile<real, H, false>(a, fa, box, tx, ty, ntx, nty, s_d, nodes.whole);
+    else fixup_tile<real, H, true>(a, fa, box, tx, ty, ntx, nty, s_d, nodes.partial);
+  } else {
+    __shared__ FixNodes<H, false> nodes;
+    fixup_tile<real, H, false>(a, fa, TileBox{tx * TX, ty * H, TX, H}, tx, ty, ntx, nty, s_d, nodes);
   }
 }
 
