@@ -136,8 +136,11 @@ __host__ __device__ constexpr int axis_vel(int g, int k) {
 // RAGGED: the tile may be partial (tile_box). Its idle threads repeat the loads of the
 // nearest node of the tile and write nothing, so their cells of the exchange buffer
 // stay zero like the halo, and the ring moves in to the tile's last column and row.
+// FEW: with fewer than four Q-nodes FP16 storage pulls the solvent early too (partial tiles,
+// one Q-node, 1999 x 1900 nodes: 446 us per step, with it 423; with 32 Q-nodes on 1000 x 750
+// it would take 1003 in place of 966).
 template <typename real, typename S, bool RESHAPE, int H, bool LEAN, bool STRESS = false,
-          bool RAGGED = false>
+          bool RAGGED = false, bool FEW = false>
 __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const FusedArgs<real>& fa,
                                            int btx, int bty, int ntx, int nty,
                                            unsigned char* smem_raw) {
@@ -179,7 +182,7 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   // and the stress collision spill with them)
   const real rho = a.rho0 + Min[(size_t)(nq + M_DRHO) * P + n];
   const real force = rho * a.tab.arow[y];
-  constexpr bool EARLY = std::is_same<S, real>::value && !STRESS;
+  constexpr bool EARLY = (std::is_same<S, real>::value || FEW) && !STRESS;
   real hs[9];
   auto pull_solvent = [&] {
     static_for<0, 9>([&](auto I) {
@@ -723,12 +726,13 @@ __device__ __forceinline__ void fused_body(const KernelArgs<real>& a, const Fuse
   }
 }
 
-template <typename real, typename S, bool RESHAPE, bool STRESS = false, bool RAGGED = false>
+template <typename real, typename S, bool RESHAPE, bool STRESS = false, bool RAGGED = false,
+          bool FEW = false>
 __global__ void __launch_bounds__(Geo<TY>::NT, 2)
 step_fused_kernel(KernelArgs<real> a, FusedArgs<real> fa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fused_body<real, S, RESHAPE, TY, false, STRESS, RAGGED>(a, fa, blockIdx.x, blockIdx.y, gridDim.x,
-                                                          gridDim.y, smem_raw);
+  fused_body<real, S, RESHAPE, TY, false, STRESS, RAGGED, FEW>(a, fa, blockIdx.x, blockIdx.y, gridDim.x,
+                                                               gridDim.y, smem_raw);
 }
 
 
@@ -1054,14 +1058,14 @@ static bool fixup_overlaps(int nq) {
 }
 static bool step_overlaps(int nq, dim3 tiles) { return tiles.x * tiles.y > SMS && fixup_overlaps(nq); }
 
-template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED>
+template <typename real, typename S, bool RESHAPE, bool STRESS, bool RAGGED, bool FEW = false>
 static cudaError_t launch_fused(const KernelArgs<real>& a, const FusedArgs<real>& f, cudaStream_t s,
                                 bool dependent) {
   const size_t smem = fused_smem_bytes(a.nq);
-  cudaError_t e = allow_dynamic_smem(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, smem);
+  cudaError_t e = allow_dynamic_smem(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED, FEW>, smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.nx + TX - 1) / TX, RAGGED ? f.ntrow : a.ny / TY);
-  return launch(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED>, grid, dim3(TX, TY), smem, s,
+  return launch(step_fused_kernel<real, S, RESHAPE, STRESS, RAGGED, FEW>, grid, dim3(TX, TY), smem, s,
                 dependent && step_overlaps(a.nq, grid), a, f);
 }
 
@@ -1078,6 +1082,8 @@ cudaError_t launch_step_fused(const KernelArgs<real>& a, const FusedArgs<real>& 
     }
   }
   const bool stress = a.qe == TFKT_QE_STRESS;
+  if constexpr (!std::is_same<S, real>::value)
+    if (f.ntrow && !stress && a.nq < 4) return launch_fused<real, S, false, false, true, true>(a, f, s, dependent);
   if (f.ntrow)
     return stress ? launch_fused<real, S, false, true, true>(a, f, s, dependent)
                   : launch_fused<real, S, false, false, true>(a, f, s, dependent);

@@ -1,4 +1,4 @@
-"""The fused kernel on whole tiles, which every large run takes: FP32 grids of more than 100
+"""The fused kernel, mostly on whole tiles, which every large run takes: FP32 grids of more than 100
 and FP16 grids of more than 152 tiles of 32 x 8. Parity with the oracle over the physical
 options, slabs, checkpoints, batches of single-run kernels and captured steps: the cases of
 the other files, whose grids are small enough for the Q-split kernels, above that line.
@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 from test_checkpoint import test_resume_is_bit_exact as _resume
-from test_gpu_paths import TOL, SCALE, test_steps_captured_in_a_graph as _captured
+from test_gpu_paths import TOL, SCALE, _check, test_steps_captured_in_a_graph as _captured
 from test_gpu_slabs import FIELDS, _params as _slab_params, _run_slabs, _single
 
 pytestmark = pytest.mark.gpu
@@ -65,6 +65,16 @@ def test_matches_oracle(T, oracle_mod, prec, shape, option):
     for k, t in SCALE.items():
         err = np.abs(g[k] - f[k]).max() / max(scale[t], 1e-300)
         assert err < TOL[prec], (k, err)
+
+
+@pytest.mark.parametrize("nx,ny", [(609, 57), (33, 617), (1, 1225)])
+@pytest.mark.parametrize("prec,beta", [("FP16", 0.2), ("FP16", 1.0), ("FP32", 1.0)])
+def test_partial_tiles_with_one_q_node(T, oracle_mod, nx, ny, prec, beta):
+    """The form of the kernel for a few Q-nodes in FP16 storage."""
+    p = T.Params(nx, ny, 1, 1.0, 5.0, 0.0 if beta == 1.0 else 0.5, beta, 0.05, 1, 0.0, 0.0, 1, getattr(T, prec))
+    with T.Solver(p) as s:
+        assert s.step_path() == "fused"
+    _check(T, oracle_mod, p, 3, prec)
 
 
 @pytest.mark.parametrize("nx,ny,parts,prec,stress", [
