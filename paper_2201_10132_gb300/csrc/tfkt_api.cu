@@ -315,6 +315,7 @@ KernelArgs<real> make_args(const Ctx* c, const HostTables* ht = nullptr) {
   a.ny = L.ny;
   a.nq = L.nq;
   a.mom_warps = moment_warps(L);
+  a.u_pass = velocity_pass(L);
   a.pitch = L.pitch;
   a.plane = L.plane;
   const double b = 1.0 / (2.0 * L.tau1 + 1.0);

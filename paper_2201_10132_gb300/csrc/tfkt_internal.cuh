@@ -177,6 +177,7 @@ struct KernelArgs {
   const double* perturb;         // [2][ny][nx] (init only)
   int nx, ny, nq;
   int mom_warps;                 // warps that share a node's moment sums (moment_warps)
+  bool u_pass;                   // the Q-split collision reads U from a pass of its own (velocity_pass)
   size_t pitch, plane;
   real tau2, c2, inv_c2p1;       // tau2, 2 tau2, 1 / (2 tau2 + 1)
   real om2b, tb, omb;            // 1 - 2 beta, 2 beta, 1 - beta
@@ -334,7 +335,8 @@ cudaError_t launch_moments(const KernelArgs<real>& a, cudaStream_t s, bool depen
 template <typename real, typename S>
 cudaError_t launch_step(const KernelArgs<real>& a, cudaStream_t s, bool dependent = false,
                         bool shared = false);
-int moment_warps(const Lattice& L);   // KernelArgs::mom_warps of a run
+int moment_warps(const Lattice& L);    // KernelArgs::mom_warps of a run
+bool velocity_pass(const Lattice& L);  // KernelArgs::u_pass of a run
 
 // Launchers (tfkt_kernels.cu). Each returns the launch status.
 template <typename real, typename S>

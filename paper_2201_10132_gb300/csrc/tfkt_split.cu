@@ -293,7 +293,8 @@ __global__ void __launch_bounds__(QN * MAXW, sizeof(real) == 8 ? 1 : 32 / MAXW) 
 }
 
 // ------------------------------------------------------------------ collide
-template <typename real, typename S, bool STRESS>
+// UPASS: U is read from its planes, which a velocity pass has written.
+template <typename real, typename S, bool STRESS, bool UPASS = false>
 __global__ void __launch_bounds__(QN * CW, 2) collide_kernel(KernelArgs<real> a) {
   __shared__ real su_[CW][2][5][QN];   // one part per group of 32 nodes
   auto& su = su_[threadIdx.z];
@@ -331,7 +332,13 @@ __global__ void __launch_bounds__(QN * CW, 2) collide_kernel(KernelArgs<real> a)
     const int x = k == 1 ? (nd.x == a.nx - 1 ? 0 : nd.x + 1) : (k == 2 ? (nd.x == 0 ? a.nx - 1 : nd.x - 1) : nd.x);
     const int y = k == 3 ? (nd.y == a.ny - 1 ? 0 : nd.y + 1) : (k == 4 ? (nd.y == 0 ? a.ny - 1 : nd.y - 1) : nd.y);
     real ux, uy;
-    velocity_at(a, a.M, x, y, ux, uy);
+    if constexpr (UPASS) {
+      const size_t m = (size_t)y * a.pitch + x;
+      ux = a.U[m];
+      uy = a.U[P + m];
+    } else {
+      velocity_at(a, a.M, x, y, ux, uy);
+    }
     su[0][k][lane] = ux;
     su[1][k][lane] = uy;
   }
@@ -617,6 +624,17 @@ int moment_warps(const Lattice& L) {
   return even_warps(L.nq + 1, most);
 }
 
+// A collision forms U at a node and its four neighbours for every group of Q-nodes. In FP64
+// that is a fifth of the operations of a run with one Q-node, the pipe's that bounds it, and
+// from a grid that fills the GPU on a pass that forms each U once pays for its launch: us per
+// step, 1024 x 1024 nodes, one Q-node 1194 without and 971 with it (stress model 1425 and
+// 1192), 256 x 256 (below the line) 90. The whole run decides, so that a
+// slab does as it does.
+bool velocity_pass(const Lattice& L) {
+  const size_t ny = L.ny_global > 0 ? L.ny_global : L.ny;
+  return L.precision == TFKT_FP64 && L.nq < 4 && (L.nx * ny + QN - 1) / QN >= MANY_GROUPS;
+}
+
 template <typename real, typename S>
 cudaError_t launch_moments(const KernelArgs<real>& a, cudaStream_t s, bool dependent) {
   auto go = [&](auto MW) {
@@ -658,6 +676,14 @@ cudaError_t launch_step(const KernelArgs<real>& a, cudaStream_t s, bool dependen
     }
   }
   const dim3 grid(nb, split), block(QN, w, g);
+  if constexpr (sizeof(real) == 8)
+    if (a.u_pass) {
+      const cudaError_t e = launch_velocity<real>(a, s);
+      if (e != cudaSuccess) return e;
+      if (a.qe == TFKT_QE_STRESS)
+        return launch(collide_kernel<real, S, true, true>, grid, block, 0, s, dependent, a);
+      return launch(collide_kernel<real, S, false, true>, grid, block, 0, s, dependent, a);
+    }
   if (a.qe == TFKT_QE_STRESS)
     return launch(collide_kernel<real, S, true>, grid, block, 0, s, dependent, a);
   return launch(collide_kernel<real, S, false>, grid, block, 0, s, dependent, a);
