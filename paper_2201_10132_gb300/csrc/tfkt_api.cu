@@ -207,6 +207,7 @@ size_t layout(const Lattice& L, Workspace* w) {
   const size_t tab = (5 * (size_t)L.nq + 25 * (size_t)L.nq + 2 * (size_t)L.ny) * sz +
                      25 * (size_t)L.nq * sizeof(int) +
                      (size_t)L.nq * (sz == 8 ? sizeof(QRow<double>) : sizeof(QRow<float>)) + 11 * A;
+  w->tab_bytes = tab;
   o = align_up(o + tab, A);
   w->off_part = o;
   o = align_up(o + (size_t)diag_blocks_for(L) * TFKT_NDIAG * sizeof(double), A);
@@ -220,8 +221,9 @@ size_t layout(const Lattice& L, Workspace* w) {
     w->off_exp = o;
     o = align_up(o + fused_export_capacity(L) * sz, A);
     w->off_ftab = o;
-    o = align_up(o + (size_t)L.nq * (9 * sizeof(int) + sz + 25 * sizeof(long long)) +
-                     max_tile_rows(L) * sizeof(int2) + 2 * fused_image_size(L.nq) + 5 * A, A);
+    w->ftab_bytes = (size_t)L.nq * (9 * sizeof(int) + sz + 25 * sizeof(long long)) +
+                    max_tile_rows(L) * sizeof(int2) + 2 * fused_image_size(L.nq) + 5 * A;
+    o = align_up(o + w->ftab_bytes, A);
   }
   return o;
 }
@@ -381,6 +383,25 @@ FusedArgs<real> make_fused(const Ctx* c) {
   return f;
 }
 
+// A context's tables go up in one copy per region, on its stream: a blocking copy from pageable
+// memory may return before the data has arrived, and a stream that does not wait for the
+// default stream (torch's are such) would then start without it. (One copy per table took
+// 5 us each, a third of the creation of a small context.)
+struct TableStage {
+  Ctx* c;
+  size_t off;              // of the region in the workspace
+  std::vector<char> host;
+  TableStage(Ctx* c_, size_t off_, size_t bytes) : c(c_), off(off_), host(bytes, 0) {}
+  template <typename T>
+  void put(const void* dptr, const std::vector<T>& v) {
+    if (!v.empty())
+      std::memcpy(host.data() + ((const char*)dptr - (const char*)c->ws.base - off), v.data(), v.size() * sizeof(T));
+  }
+  cudaError_t upload() {
+    return cudaMemcpyAsync((char*)c->ws.base + off, host.data(), host.size(), cudaMemcpyHostToDevice, c->stream);
+  }
+};
+
 tfkt_status upload_fused_tables(Ctx* c, const HostTables& t) {
   using real = float;
   std::vector<int> tgt;
@@ -389,48 +410,39 @@ tfkt_status upload_fused_tables(Ctx* c, const HostTables& t) {
   fused_tables(c->L, t, tgt, dpsi, c->dvx, c->dvy, poff);
   const std::vector<int2> trow = tile_rows(c->L);
   c->ntrow = (int)trow.size();
+  TableStage stage(c, c->ws.off_ftab, c->ws.ftab_bytes);
   FusedArgs<real> f = make_fused<real>(c);
-  if (c->ntrow)
-    TFKT_CUDA(c, cudaMemcpy((void*)f.trow, trow.data(), trow.size() * sizeof(int2),
-                            cudaMemcpyHostToDevice));
+  stage.put(f.trow, trow);
   const int cur = c->cur;
-  for (c->cur = 0; c->cur < 2; ++c->cur) {
-    const std::vector<char> img = fused_image(c->L, t, tgt, poff, (const char*)c->ws.base + c->ws.off_pop[c->cur],
-                                              store_size(c->L));
-    cudaError_t e = cudaMemcpy((void*)make_fused<real>(c).image, img.data(), img.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(c, e, "table image");
-  }
+  for (c->cur = 0; c->cur < 2; ++c->cur)
+    stage.put(make_fused<real>(c).image,
+              fused_image(c->L, t, tgt, poff, (const char*)c->ws.base + c->ws.off_pop[c->cur], store_size(c->L)));
   c->cur = cur;
-  std::vector<real> d(dpsi.begin(), dpsi.end());
-  TFKT_CUDA(c, cudaMemcpy((void*)f.poff, poff.data(), poff.size() * sizeof(long long),
-                          cudaMemcpyHostToDevice));
-  TFKT_CUDA(c, cudaMemcpy((void*)f.tgt, tgt.data(), tgt.size() * sizeof(int),
-                          cudaMemcpyHostToDevice));
-  TFKT_CUDA(c, cudaMemcpy((void*)f.dpsi, d.data(), d.size() * sizeof(real),
-                          cudaMemcpyHostToDevice));
+  stage.put(f.poff, poff);
+  stage.put(f.tgt, tgt);
+  stage.put(f.dpsi, std::vector<real>(dpsi.begin(), dpsi.end()));
+  TFKT_CUDA(c, stage.upload());
   return TFKT_OK;
 }
 
 template <typename real>
 tfkt_status upload_tables(Ctx* c, const HostTables& t) {
   KernelArgs<real> a = make_args<real>(c);
-  auto put = [&](const void* dptr, const std::vector<double>& v) -> cudaError_t {
-    std::vector<real> h(v.begin(), v.end());
-    return cudaMemcpy((void*)dptr, h.data(), h.size() * sizeof(real), cudaMemcpyHostToDevice);
+  TableStage stage(c, c->ws.off_tab, c->ws.tab_bytes);
+  auto put = [&](const void* dptr, const std::vector<double>& v) {
+    stage.put(dptr, std::vector<real>(v.begin(), v.end()));
   };
-  TFKT_CUDA(c, put(a.tab.qx, t.qx));
-  TFKT_CUDA(c, put(a.tab.qy, t.qy));
-  TFKT_CUDA(c, put(a.tab.fx, t.fx));
-  TFKT_CUDA(c, put(a.tab.fy, t.fy));
-  TFKT_CUDA(c, put(a.tab.psi0, t.psi0));
-  TFKT_CUDA(c, cudaMemcpy((void*)a.tab.pull, t.pull.data(), t.pull.size() * sizeof(int),
-                          cudaMemcpyHostToDevice));
-  TFKT_CUDA(c, put(a.tab.delta, t.delta));
-  TFKT_CUDA(c, put(a.tab.arow, t.arow));
-  TFKT_CUDA(c, put(a.tab.urow, t.urow));
-  const std::vector<QRow<real>> rows = build_rows<real>(c->L, t);
-  TFKT_CUDA(c, cudaMemcpy((void*)a.tab.row, rows.data(), rows.size() * sizeof(QRow<real>),
-                          cudaMemcpyHostToDevice));
+  put(a.tab.qx, t.qx);
+  put(a.tab.qy, t.qy);
+  put(a.tab.fx, t.fx);
+  put(a.tab.fy, t.fy);
+  put(a.tab.psi0, t.psi0);
+  stage.put(a.tab.pull, t.pull);
+  put(a.tab.delta, t.delta);
+  put(a.tab.arow, t.arow);
+  put(a.tab.urow, t.urow);
+  stage.put(a.tab.row, build_rows<real>(c->L, t));
+  TFKT_CUDA(c, stage.upload());
   if constexpr (std::is_same<real, float>::value)
     if (c->fused) return upload_fused_tables(c, t);
   return TFKT_OK;

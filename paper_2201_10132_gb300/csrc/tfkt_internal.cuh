@@ -265,6 +265,7 @@ struct Workspace {
   size_t off_pop[2] = {0, 0};
   size_t off_M = 0, off_U = 0, off_tab = 0, off_part = 0, off_diag = 0;
   size_t off_M2 = 0, off_exp = 0, off_ftab = 0;  // fused path: second M, ring exports, tables
+  size_t tab_bytes = 0, ftab_bytes = 0;          // of the tables' regions
 };
 
 struct Ctx {

@@ -65,3 +65,11 @@ def test_overlapped_kernels_read_nothing_through_restrict(name):
             assert var in WRITTEN_ONLY, (m.group(1), var)
     if name in ("tfkt_fused.cu", "tfkt_lpm.cu", "tfkt_mlp.cu", "tfkt_split.cu"):
         assert found >= 2
+
+
+@pytest.mark.parametrize("name", sorted(f.name for f in CSRC.glob("*.cu")))
+def test_copies_are_ordered_on_a_stream(name):
+    """A blocking cudaMemcpy or cudaMemset is ordered against the default stream only, and from
+    pageable memory it may return before the data has arrived: a kernel on a non-blocking
+    stream may then run without it."""
+    assert not re.findall(r"\bcuda(?:Memcpy|Memset|Memcpy2D)\s*\(", _code(name))
