@@ -162,6 +162,10 @@ constexpr uint32_t FIELDS_CONF = (1u << TFKT_F_CXX) | (1u << TFKT_F_CXY) | (1u <
                                  (1u << TFKT_F_QRMS);
 constexpr uint32_t FIELDS_STRESS = (1u << TFKT_F_THXX) | (1u << TFKT_F_THXY) | (1u << TFKT_F_THYY);
 
+// From this many Q-nodes on: with one the three floats' set-up and end cost more than they save
+// (C of 1024 x 1024 nodes, us: 206 with them, 170 in FP64; with 4 138 and 166).
+constexpr int EXACT_SUMS_NQ = 4;
+
 // A sum kept in three floats.
 struct ExactSum {
   float hi = 0, lo = 0, rest = 0;
@@ -259,10 +263,11 @@ __global__ void __launch_bounds__(256) fields_kernel(KernelArgs<real> a, uint32_
   const bool sums = mask & (FIELDS_PSUM | FIELDS_STRESS);
   const bool conf = mask & FIELDS_CONF, stress = mask & FIELDS_STRESS;
   const int nq = a.nq;
+  const bool exact = sums && !stress && nq >= EXACT_SUMS_NQ;
   double* s0 = reinterpret_cast<double*>(field_smem);
   FieldRow* row = reinterpret_cast<FieldRow*>(field_smem + FIELD_HEAD);
   if constexpr (std::is_same<real, float>::value)
-    if (sums && !stress) {
+    if (exact) {
       stage_field_rows(a, s0, row);
       __syncthreads();
     }
@@ -280,7 +285,7 @@ __global__ void __launch_bounds__(256) fields_kernel(KernelArgs<real> a, uint32_
   double s[7] = {};
   bool done = !sums;
   if constexpr (std::is_same<real, float>::value)
-    if (sums && !stress) {
+    if (exact) {
       ExactSum es[4];
       if (conf) exact_sums<true>(a, row, n, es);
       else exact_sums<false>(a, row, n, es);
