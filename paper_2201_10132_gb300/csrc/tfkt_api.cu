@@ -316,7 +316,7 @@ KernelArgs<real> make_args(const Ctx* c, const HostTables* ht = nullptr) {
   a.nx = L.nx;
   a.ny = L.ny;
   a.nq = L.nq;
-  a.mom_warps = moment_warps(L);
+  a.mom_warps = (int16_t)moment_warps(L);
   a.u_pass = velocity_pass(L);
   a.pitch = L.pitch;
   a.plane = L.plane;

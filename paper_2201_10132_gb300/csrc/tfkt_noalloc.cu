@@ -122,7 +122,7 @@ tfkt_status moments_noalloc(const tfkt_params& p, const Lattice& L, const void* 
   a.nx = L.nx;
   a.ny = L.ny;
   a.nq = L.nq;
-  a.mom_warps = moment_warps(L);
+  a.mom_warps = (int16_t)moment_warps(L);
   a.pitch = L.pitch;
   a.plane = L.plane;
   a.tau2 = (real)L.tau2;
