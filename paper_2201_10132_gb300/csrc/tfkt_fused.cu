@@ -15,8 +15,8 @@
 //
 // Grids that are no multiples of the tile end in partial tiles (template parameter
 // RAGGED; whole tiles keep their own instantiation). The partial tiles' idle threads
-// cost what their share of the tiles is: 1000 x 750 nodes in FP32 run at 4.95 TB/s of
-// population traffic, 1024 x 768 nodes, the same tiles filled, at 5.2.
+// cost what their share of the tiles is: 1000 x 750 nodes in FP32 run at 5.14 TB/s of
+// population traffic, 1024 x 768 nodes, the same tiles filled, at 5.17.
 //
 // M planes written for step n+1: interior nodes get final values (delta psi,
 // delta rho, J, delta Theta); border nodes get the tile's raw partial sums in
@@ -1000,10 +1000,10 @@ size_t run_tiles(const Lattice& L) {
 }
 
 // Grids of whole tiles, and in FP32 and FP16 storage any grid that does not take the
-// Q-split kernels: with partial tiles the fused kernel and its fix-up take 979 us per
-// step on 1000 x 750 nodes with 32 Q-nodes in FP32 (1026 in FP16 storage, 993 on 999 x 751
-// with the stress quasi-equilibrium), the Q-split kernels, which read the populations
-// twice, 1426 (1193, 1437); with 9 Q-nodes on 333 x 777 nodes 134 against 174.
+// Q-split kernels: with partial tiles the fused kernel and its fix-up take 944 us per
+// step on 1000 x 750 nodes with 32 Q-nodes in FP32 (966 in FP16 storage), the Q-split
+// kernels, which read the populations twice, 1430 (1205); with 9 Q-nodes 306 against 451, with
+// the stress quasi-equilibrium 314 against 450, with one 86 against 116.
 //
 // FP64 has no fused kernel. Whole tiles keep the second set of moment planes all the same
 // (2% of the workspace at 32 Q-nodes): a step then leaves the moments of its result, and
