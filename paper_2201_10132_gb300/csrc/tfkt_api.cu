@@ -385,13 +385,16 @@ FusedArgs<real> make_fused(const Ctx* c) {
 
 // A context's tables go up in one copy per region, on its stream: a blocking copy from pageable
 // memory may return before the data has arrived, and a stream that does not wait for the
-// default stream (torch's are such) would then start without it. (One copy per table took
-// 5 us each, a third of the creation of a small context.)
+// default stream (torch's are such) would then start without it. The host's side lives until
+// the stream has been waited for: where the GPU reads pageable memory itself, the copy
+// need not have read it when the call returns. (One copy per table took 5 us each, a third
+// of the creation of a small context.)
 struct TableStage {
   Ctx* c;
   size_t off;              // of the region in the workspace
-  std::vector<char> host;
-  TableStage(Ctx* c_, size_t off_, size_t bytes) : c(c_), off(off_), host(bytes, 0) {}
+  std::vector<char>& host;
+  TableStage(Ctx* c_, size_t off_, size_t bytes)
+      : c(c_), off(off_), host(c_->staged.emplace_back(bytes, (char)0)) {}
   template <typename T>
   void put(const void* dptr, const std::vector<T>& v) {
     if (!v.empty())
@@ -816,14 +819,18 @@ tfkt_status ctx_create(const Lattice& L, const double* perturb, void* dev_worksp
     c->ws.owned = true;
   }
   c->ws.bytes = need;
+  c->staged.reserve(2);   // (so that a stage stays where it is)
   HostTables t = build_tables(L);
   s = L.precision == TFKT_FP64 ? upload_tables<double>(c, t) : upload_tables<float>(c, t);
-  if (s == TFKT_OK) s = DISPATCH(c, init_state, c, perturb);
+  if (s == TFKT_OK) s = DISPATCH(c, init_state, c, perturb);   // (it waits for the stream)
   if (s != TFKT_OK) {
+    cudaStreamSynchronize(c->stream);
+    cudaGetLastError();
     if (c->ws.owned) cudaFree(c->ws.base);
     delete c;
     return s;
   }
+  std::vector<std::vector<char>>().swap(c->staged);
   *out = c;
   return TFKT_OK;
 }

@@ -273,6 +273,7 @@ struct Workspace {
 struct Ctx {
   Lattice L;
   Workspace ws;
+  std::vector<std::vector<char>> staged;   // tables on their way up; empty once created
   cudaStream_t stream = nullptr;
   int cur = 0;            // population buffer holding the state
   bool m_valid = false;   // M holds the moments of the current state
